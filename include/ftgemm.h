@@ -52,7 +52,8 @@ typedef struct ftgemm_ctx* ftgemm_handle_t;
 
 /* element type of A and B.  C is always fp32, accumulation is always fp32. */
 typedef enum {
-  FTGEMM_F32 = 0,  /* fp32 operands, CUDA-core (SIMT) kernels              */
+  FTGEMM_F32 = 0,  /* fp32 operands: CUDA-core (SIMT) kernels, or the tensor
+                      cores through exact bf16 planes (see ftgemm_gemm)     */
   FTGEMM_BF16 = 1, /* bf16 operands, tcgen05 tensor-core kernel            */
   FTGEMM_E4M3 = 2  /* fp8 E4M3 operands with per-tensor scales, tcgen05    */
 } ftgemm_dtype;
@@ -250,6 +251,17 @@ int ftgemm_quantize(ftgemm_handle_t handle, int64_t n, const float* x, void* y,
  * handle's events are cleared first, the stream is synchronised at the end
  * and the events of this call are returned.
  * Supported: F32 with OFF/THREAD/WARP/BLOCK; BF16 and E4M3 with OFF/TILE.
+ * F32 at OFF, WARP and BLOCK: larger products run on the tensor cores.  Each
+ * operand is split into three bf16 planes whose sum is the fp32 value exactly,
+ * six plane products make up the fp32 product (what is left out is below half
+ * an ulp of it), and chunks of 32 of K are added in fp32 with round-to-nearest:
+ * the error against 64 bits is about a fifth of the CUDA-core kernel's.  Units,
+ * tile grid, cadence, splits, thresholds and records are those of the schedule,
+ * whichever kernel runs; a fault is applied at the end of its verification
+ * period (the accumulation being additive, its k-step changes only rounding).
+ * Operands with a value the planes cannot hold (not finite, or a magnitude
+ * other than 0 outside 2^-100 .. 2^60) are found on the device and computed by
+ * the CUDA-core kernel in the same call.
  * Tensor-core path (BF16/E4M3): the MMA tile is 128 x 256; at level TILE
  * its last 3 (BF16) or 5 (E4M3) rows and its last 4 (BF16) or 8 (E4M3)
  * columns carry the checksums, so a CTA computes a 125 x 252 (BF16) or 123 x 248 (E4M3) tile

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "f32tc.cuh"
 #include "fp64.cuh"
 
 namespace ftg {
@@ -40,6 +41,12 @@ cudaError_t launch_encode_kmajor(const float*, long long, int, int, int, float*,
                                  float*, int*, cudaStream_t);
 cudaError_t launch_splitk_reduce(const float*, int, int, int, float, float, float*, long long,
                                  cudaStream_t);
+cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long lda, int M, int K, float* At,
+                                      long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
+                                      int* launches, cudaStream_t st);
+cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
+                               int* launches, cudaStream_t st);
+cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]);
 int tc_nb_parts(int dt, long long K);
 cudaError_t launch_tc_bind(TcProblem* probs, TcProbMaps* maps, const int* pos, const ftgemm_problem* in, int count,
@@ -373,6 +380,24 @@ static int make_map_sw128(CUtensorMap* m, const void* base, int elem, uint64_t i
   if (r != CUDA_SUCCESS)
     FAIL(FTGEMM_ERR_ALIGN, "cuTensorMapEncodeTiled (swizzled) failed (%d): dims {%llu,%llu} ld %llu box {%u,%u}",
          (int)r, (unsigned long long)inner, (unsigned long long)outer, (unsigned long long)ld, bi, bo);
+  return FTGEMM_OK;
+}
+
+// 2-D tensor map of operand planes seen as rows of 64 bf16 elements (128
+// bytes): box {64, rows}, no swizzle (the planes are stored swizzled).
+static int make_map_rows128(CUtensorMap* m, const uint16_t* base, uint64_t total_rows, uint32_t rows) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) FAIL(FTGEMM_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+  cuuint64_t dims[2] = {64, total_rows};
+  cuuint64_t strides[1] = {128};
+  cuuint32_t box[2] = {64, rows};
+  cuuint32_t es[2] = {1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)base, dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    FAIL(FTGEMM_ERR_CUDA, "cuTensorMapEncodeTiled (planes) failed (%d): %llu rows, box %u", (int)r,
+         (unsigned long long)total_rows, rows);
   return FTGEMM_OK;
 }
 
@@ -1370,6 +1395,124 @@ int ftgemm_gemm(ftgemm_handle_t h, int64_t m, int64_t n, int64_t k, double alpha
 
 }  // extern "C"
 
+// ---- fp32 on the tensor cores (f32tc.cuh) -----------------------------------
+
+struct F32TcPlan {
+  int nch;                  // 32-element chunks of K
+  int bn;                   // columns of a CTA pair's tile: 256 or 128
+  long long ldc_d, ldr_d;   // row strides of the checksum segments
+  int seg, segs_per_period, segs_per_split;
+  long long segs;           // over all splits
+};
+
+// Whether the tensor-core kernel takes this fp32 call, and its layout (pairs:
+// CTA pairs the device runs at once).
+//  - Levels OFF, WARP and BLOCK with units of 16 .. 128 rows and columns.
+//  - A verification period is whole 32-element chunks of K (or the whole
+//    split); splits start on such chunks.
+static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_schedule& s, int split,
+                       int ks_per_split, int cadence, int um, int un, int pairs, F32TcPlan* out) {
+  if (level != FTGEMM_FT_OFF && level != FTGEMM_FT_WARP && level != FTGEMM_FT_BLOCK) return false;
+  const bool abft = level != FTGEMM_FT_OFF;
+  const long long kps = (long long)ks_per_split * s.k_tb;
+  if (split > 1 && kps % F32TC_KC) return false;
+  long long period = kps;
+  if (abft) {
+    if (um < 16 || um > 128 || un < 16 || un > 128) return false;
+    if (cadence < ks_per_split) period = (long long)cadence * s.k_tb;
+    if (period < kps && period % F32TC_KC) return false;
+  }
+  // Where it is the faster one.  Its fixed part (operand planes, checksum
+  // segments, the stand-by of the CUDA-core kernel) is worth about 2e8 flop of
+  // CUDA-core work with checksums and 8e8 without, more when K is a few chunks;
+  // without checksums it also needs tiles to run side by side.  Measured, us per
+  // call, CUDA cores / tensor cores: BLOCK 384^3 48 / 58, 512^3 61 / 56, 1024^3
+  // 129 / 66, 2048x2048x64 44 / 47, 2048x2048x128 55 / 50, 256x256x8192 418 / 275;
+  // OFF 512^3 28 / 35, 768^3 44 / 40, 256x256x8192 147 / 192, 512x512x2048 83 / 67.
+  const double flop = 2.0 * M * N * K;
+  const long long tiles = (long long)split * ((M + 255) / 256) * ((N + 127) / 128);
+  if (abft ? flop < 2e8 || (K < 96 && flop < 4e9) : flop < 8e8 || tiles < 6 || (K < 192 && flop < 4e9)) return false;
+  F32TcPlan& t = *out;
+  t.nch = (K + F32TC_KC - 1) / F32TC_KC;
+  // rows of 128 bytes are addressed by 32-bit coordinates
+  if (((long long)std::max(M, N) + 127) / 128 * t.nch * 192 > INT32_MAX) return false;
+  t.bn = 128;
+  if (!abft || (um >= 64 && un >= 64)) {
+    // waves of CTA-pair tiles times the measured SM cycles (in tens) of a chunk
+    // of K: 256 x 256 tiles keep the tensor cores busier, 256 x 128 ones fill
+    // a small grid (BLOCK 1024^3: 83 us on the former, 66 on the latter)
+    auto waves = [&](int bn) {
+      return (int64_t)split * (((int64_t)M + 255) / 256) * (((int64_t)N + bn - 1) / bn) + pairs - 1;
+    };
+    t.bn = waves(256) / pairs * (abft ? 210 : 156) <= waves(128) / pairs * (abft ? 127 : 107) ? 256 : 128;
+  }
+  t.ldc_d = ((long long)N + 3) / 4 * 4;
+  t.ldr_d = ((long long)M + 3) / 4 * 4;
+  t.seg = (period >= kps || period % F32TC_SEG == 0) ? F32TC_SEG : (int)period;
+  const long long span = std::min<long long>(kps, K);
+  t.segs_per_split = (int)((span + t.seg - 1) / t.seg);
+  t.segs_per_period = period >= kps ? t.segs_per_split : (int)(period / t.seg);
+  t.segs = (long long)split * t.segs_per_split;
+  if (abft) {
+    const double nv = (M + um - 1) / um, nw = (N + un - 1) / un;
+    if (4.0 * t.segs * (nv * t.ldc_d + nw * t.ldr_d) > 2147483648.0) return false;  // checksum segments: 2 GiB
+  }
+  return true;
+}
+
+// The checksum segments and the product, timed as the call's main kernel.
+static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, double alpha, double beta, float* C,
+                     int64_t ldc, bool c16, ftgemm_ft_level level, const ftgemm_schedule& s, int split,
+                     int ks_per_split, int cadence, int ksteps, int tiles_n, int nf, float* Dc, float* Dr,
+                     float* partial, int* launches) {
+  const bool abft = level != FTGEMM_FT_OFF;
+  const int bn = t.bn;
+  F32TcMaps maps;
+  auto tile_rows = [&](int lines, int per) { return (uint64_t)((lines + per - 1) / per) * t.nch; };
+  int rc = make_map_rows128(&maps.A, e.Ap, tile_rows(e.M, 128) * 192, 192);
+  if (!rc) rc = make_map_rows128(&maps.B, e.Bp, tile_rows(e.N, 128) * 192, 96);
+  if (!rc && abft) rc = make_map_rows128(&maps.V, e.Vp, tile_rows(e.nv, 128) * 192, 192);
+  if (!rc && abft) rc = make_map_rows128(&maps.W, e.Wp, tile_rows(e.nw, 128) * 192, 192);
+  if (!rc && abft) rc = make_map_rows128(&maps.An, e.Ap, tile_rows(e.M, 128) * 192, 32);
+  if (rc) return rc;
+  if (!abft) maps.V = maps.W = maps.An = maps.A;
+  F32TcParams p;
+  memset(&p, 0, sizeof(p));
+  p.M = e.M; p.N = e.N; p.K = e.K;
+  p.tiles_m2 = (e.M + 2 * F32TC_BM - 1) / (2 * F32TC_BM);
+  p.tiles_n = (e.N + bn - 1) / bn;
+  p.group_m = std::min(p.tiles_m2, 8);
+  p.nsplit = split;
+  p.k_per_split = (int)std::min<long long>((long long)ks_per_split * s.k_tb, e.K);
+  p.seg = t.seg; p.segs_per_period = t.segs_per_period; p.segs_per_split = t.segs_per_split;
+  p.um = abft ? e.um : 128; p.un = abft ? e.un : 128;
+  p.nv = e.nv; p.nw = e.nw;
+  p.m_tb = s.m_tb; p.n_tb = s.n_tb; p.k_tb = s.k_tb;
+  p.tiles_n_sched = tiles_n; p.ks_per_split = ks_per_split; p.cadence = std::max(1, std::min(cadence, ks_per_split)); p.ksteps = ksteps;
+  p.nA = e.nA; p.nB = e.nB; p.sq16a = e.sq16a; p.sq16b = e.sq16b;
+  p.Dc = Dc; p.Dr = Dr; p.ldc_d = t.ldc_d; p.ldr_d = t.ldr_d;
+  p.lam_u = (float)(h->lambda * std::ldexp(1.0, -24));
+  p.mu_u = (float)(h->mu * std::ldexp(1.0, -24));
+  p.C = C; p.ldc = ldc; p.c_vec = (ldc % 4 == 0) && c16;
+  p.alpha = (float)alpha; p.beta = (float)beta;
+  p.partial = partial;
+  p.faults = nf > 0 ? h->d_faults : nullptr; p.nfaults = nf;
+  p.rep = h->rep; p.recs = h->recs;
+  p.bad = e.bad;
+  std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
+  if (h->timing) {
+    rc = take_events(h, &ev);
+    if (rc) return rc;
+    CK(cudaEventRecord(ev.first, h->stream));
+  }
+  CK(launch_f32tc(bn, abft, maps, p, h->num_sms > 0 ? h->num_sms : 148, launches, h->stream));
+  if (h->timing) {
+    CK(cudaEventRecord(ev.second, h->stream));
+    h->pending.push_back(ev);
+  }
+  return FTGEMM_OK;
+}
+
 // The SIMT path of ftgemm_gemm with an explicit schedule and level.
 // At_given (OFF only): A already k-major (K x M, row stride ldat, 16-byte
 // aligned rows); the transpose pass is skipped.
@@ -1419,7 +1562,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   const int NV = level == FTGEMM_FT_WARP ? s.m_tb / s.m_w : 1;
   const int NW = level == FTGEMM_FT_WARP ? s.n_tb / s.n_w : 1;
   const long long ldt = At_given ? ldat : (M + 3) / 4 * 4;  // A^T row stride (16-byte multiple)
-  const long long ldv = (K + 3) / 4 * 4;  // encoded-vector row stride
+  const long long ldv = ((long long)K + 7) / 8 * 8;  // encoded-vector row stride
   const bool b_ok = (ldb % 4 == 0) && al16(B);
   const long long ldbp = b_ok ? ldb : (N + 3) / 4 * 4;
   const int nvb = (M + m_u - 1) / m_u, nwb = (N + n_u - 1) / n_u;
@@ -1428,9 +1571,6 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   const size_t nV = need_vw ? (size_t)nvb * ldv : 0;
   const size_t nW = (need_vw && !detect) ? (size_t)nwb * ldv : 0;  // the detector keeps no B e
   const size_t nNa = abft ? (size_t)M : 0, nNb = abft ? (size_t)N : 0;
-  const size_t nScr = abft ? (size_t)std::max<long long>((long long)((K + 31) / 32) * M,
-                                                         kmajor_scratch_floats(K, N))
-                           : 0;
   const size_t nPart = split > 1 ? (size_t)split * M * N : 0;
   // learned threshold and residual sink (block level): block coherences
   const bool learned = level == FTGEMM_FT_BLOCK && h->mlp_on && !detect;
@@ -1439,30 +1579,83 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     FAIL(FTGEMM_ERR_ARG, "residual sink: %lld tiles, capacity %lld", (long long)tiles_m * tiles_n,
          (long long)h->sink_cap);
   const size_t nCo = (learned || sink) ? (size_t)(tiles_m + tiles_n) : 0;
-  const size_t oAt = 0, oBp = align64(oAt + nAt), oV = align64(oBp + nBp), oW = align64(oV + nV),
-               oNa = align64(oW + nW), oNb = align64(oNa + nNa), oScr = align64(oNb + nNb),
-               oPart = align64(oScr + nScr), oCo = align64(oPart + nPart), total = align64(oCo + nCo);
-  {
-    int rc = ensure_ws(h, total);
+  size_t o = 0;
+  auto take = [&](size_t floats) { const size_t at = o; o = align64(o + floats); return at; };
+  // the tensor-core kernel where it applies; its operand planes share their
+  // space with the operands of the CUDA-core kernel, which runs in its place
+  // when the planes cannot hold a value
+  F32TcPlan tc;
+  bool use_tc = !At_given && !detect && !learned && !sink &&
+                f32tc_plan(M, N, K, level, s, split, ks_per_split, cadence, m_u, n_u,
+                           (h->num_sms > 0 ? h->num_sms : 148) / 2, &tc);
+  size_t oAt, oBp, oV, oW, oNa, oNb, oPart, oScr = 0, oCo = 0, oTc[9] = {};
+  if (use_tc) {
+    auto planes = [&](int lines) { return (size_t)((lines + 127) / 128) * tc.nch * (3 * F32TC_APLANE / 2); };
+    oAt = take(std::max(planes(M), nAt));
+    oBp = take(std::max(planes(N), nBp));
+    oV = take(nV); oW = take(nW); oNa = take(nNa); oNb = take(nNb); oPart = take(nPart);
+    if (abft) {
+      oTc[0] = take(planes(nvb));
+      oTc[1] = take(planes(nwb));
+      oTc[2] = take((size_t)((K + 127) / 128) * M);
+      oTc[3] = take((size_t)((K + 127) / 128) * N);
+      oTc[4] = take((M + 15) / 16);
+      oTc[5] = take((N + 15) / 16);
+      oTc[6] = take((size_t)tc.segs * nvb * tc.ldc_d);
+      oTc[7] = take((size_t)tc.segs * nwb * tc.ldr_d);
+    }
+    oTc[8] = take(1);
+    if (ensure_ws(h, o) != FTGEMM_OK) {  // no room for the planes
+      cudaGetLastError();
+      use_tc = false;
+    }
+  }
+  if (!use_tc) {
+    const size_t nScr = abft ? (size_t)std::max<long long>((long long)((K + 31) / 32) * M,
+                                                           kmajor_scratch_floats(K, N))
+                             : 0;
+    o = 0;
+    oAt = take(nAt); oBp = take(nBp); oV = take(nV); oW = take(nW); oNa = take(nNa); oNb = take(nNb);
+    oScr = take(nScr); oPart = take(nPart); oCo = take(nCo);
+    int rc = ensure_ws(h, o);
     if (rc) return rc;
   }
   float* ws = h->ws;
   int launches = 0;
-  // A^T, with the A side of the encoding (block sums, row norms) in the same pass
   const float* At = At_given ? At_given : ws + oAt;
-  if (!At_given)
-    CK(launch_transpose_encode(Af, lda, M, K, ws + oAt, ldt, m_u, need_vw ? ws + oV : nullptr, ldv,
-                               abft ? ws + oNa : nullptr, ws + oScr, &launches, h->stream));
-  const float* Bk = Bf;
-  if (!b_ok) {
-    CK(launch_copy_pad(Bf, ldb, K, N, ws + oBp, ldbp, h->stream));
-    ++launches;
-    Bk = ws + oBp;
-  }
-  if (abft) {
-    CK(launch_encode_kmajor(Bk, ldbp, K, N, (need_vw && !detect) ? n_u : 2,
-                            (need_vw && !detect) ? ws + oW : nullptr, ldv, ws + oNb, ws + oScr, &launches,
-                            h->stream));
+  const float* Bk = b_ok ? Bf : ws + oBp;
+  if (use_tc) {
+    F32TcPrep e;
+    memset(&e, 0, sizeof(e));
+    e.M = M; e.N = N; e.K = K;
+    e.um = abft ? m_u : 0; e.un = abft ? n_u : 0; e.nv = nvb; e.nw = nwb;
+    e.Ap = (uint16_t*)(ws + oAt);
+    e.Bp = (uint16_t*)(ws + oBp);
+    e.V = ws + oV; e.W = ws + oW; e.ldv = ldv;
+    e.Vp = (uint16_t*)(ws + oTc[0]); e.Wp = (uint16_t*)(ws + oTc[1]);
+    e.pa = ws + oTc[2]; e.pb = ws + oTc[3];
+    e.nA = ws + oNa; e.nB = ws + oNb; e.sq16a = ws + oTc[4]; e.sq16b = ws + oTc[5];
+    e.bad = (int*)(ws + oTc[8]);
+    CK(launch_f32tc_split(Af, lda, Bf, ldb, e, &launches, h->stream));
+    int rc = f32tc_run(h, tc, e, alpha, beta, C, ldc, al16(C), level, s, split, ks_per_split, cadence, ksteps, tiles_n,
+                       nf, ws + oTc[6], ws + oTc[7], split > 1 ? ws + oPart : nullptr, &launches);
+    if (rc) return rc;
+    CK(launch_kmajor_operands_if(e.bad, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
+                                 &launches, h->stream));
+  } else {
+    // A^T, with the A side of the encoding (block sums, row norms) in the same pass
+    if (!At_given)
+      CK(launch_transpose_encode(Af, lda, M, K, ws + oAt, ldt, m_u, need_vw ? ws + oV : nullptr, ldv,
+                                 abft ? ws + oNa : nullptr, ws + oScr, &launches, h->stream));
+    if (!b_ok) {
+      CK(launch_copy_pad(Bf, ldb, K, N, ws + oBp, ldbp, h->stream));
+      ++launches;
+    }
+    if (abft) {
+      CK(launch_encode_kmajor(Bk, ldbp, K, N, (need_vw && !detect) ? n_u : 2,
+                              (need_vw && !detect) ? ws + oW : nullptr, ldv, ws + oNb, ws + oScr, &launches,
+                              h->stream));
+    }
   }
   if (learned || sink) {
     CK(launch_block_coherence(ws + oV, ws + oW, ldv, K, ws + oNa, ws + oNb, M, N, m_u, n_u, ws + oCo,
@@ -1508,8 +1701,10 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   p.coB = (learned || sink) ? ws + oCo + tiles_m : nullptr;
   p.sink_lam = sink ? h->sink_lam : nullptr;
   p.sink_x = sink ? h->sink_x : nullptr;
+  p.only_if = use_tc ? (const int*)(ws + oTc[8]) : nullptr;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-  if (h->timing) {
+  const bool timed = h->timing && !use_tc;  // the tensor-core kernels were timed themselves
+  if (timed) {
     int rc = take_events(h, &ev);
     if (rc) return rc;
     CK(cudaEventRecord(ev.first, h->stream));
@@ -1517,7 +1712,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   if (detect) CK(simt_launch_wide32_detect(maps, p, split, h->stream));
   else CK(cfg->launch((int)level, maps, p, split, h->stream));
   ++launches;
-  if (h->timing) {
+  if (timed) {
     CK(cudaEventRecord(ev.second, h->stream));
     h->pending.push_back(ev);
   }

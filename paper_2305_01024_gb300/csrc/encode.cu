@@ -44,7 +44,9 @@ __global__ void transpose_kernel(const float* __restrict__ A, long long lda, int
 __global__ void __launch_bounds__(256) transpose_encode_kernel(const float* __restrict__ A, long long lda, int M,
                                                                int K, float* __restrict__ At, long long ldt,
                                                                int m_u, float* __restrict__ V, long long ldv,
-                                                               float* __restrict__ part) {
+                                                               float* __restrict__ part,
+                                                               const int* __restrict__ gate) {
+  if (gate && !*gate) return;  // only run if *gate is set
   __shared__ float tile[128][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * 32, m0 = blockIdx.y * 128;
@@ -107,7 +109,8 @@ __global__ void __launch_bounds__(256) transpose_encode_kernel(const float* __re
 }
 
 __global__ void copy_pad_kernel(const float* __restrict__ X, long long ldx, int R, int Cn,
-                                float* __restrict__ Y, long long ldy) {
+                                float* __restrict__ Y, long long ldy, const int* __restrict__ gate) {
+  if (gate && !*gate) return;  // only run if *gate is set
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)R * Cn) return;
   const int r = (int)(idx / Cn), c = (int)(idx % Cn);
@@ -319,7 +322,8 @@ cudaError_t launch_transpose_encode(const float* A, long long lda, int M, int K,
                                     cudaStream_t st) {
   if (V && (m_u < 2 || m_u > 128 || (m_u & (m_u - 1)))) return cudaErrorInvalidValue;
   dim3 g((K + 31) / 32, (M + 127) / 128);
-  transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, V ? m_u : 0, V, ldv, nrm ? scratch : nullptr);
+  transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, V ? m_u : 0, V, ldv, nrm ? scratch : nullptr,
+                                          nullptr);
   ++*launches;
   if (nrm) {
     colnorm_finish_kernel<<<(M + 31) / 32, 256, 0, st>>>(scratch, (K + 31) / 32, M, nrm);
@@ -331,7 +335,23 @@ cudaError_t launch_transpose_encode(const float* A, long long lda, int M, int K,
 cudaError_t launch_copy_pad(const float* X, long long ldx, int R, int Cn, float* Y, long long ldy,
                             cudaStream_t st) {
   const long long total = (long long)R * Cn;
-  copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(X, ldx, R, Cn, Y, ldy);
+  copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(X, ldx, R, Cn, Y, ldy, nullptr);
+  return cudaGetLastError();
+}
+
+// The operand layout of the CUDA-core kernel, produced only if *gate is set
+// when the kernels run: A^T, and (Bp not null) B with padded rows.
+cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long lda, int M, int K, float* At,
+                                      long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
+                                      int* launches, cudaStream_t st) {
+  dim3 g((K + 31) / 32, (M + 127) / 128);
+  transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, 0, nullptr, 0, nullptr, gate);
+  ++*launches;
+  if (Bp) {
+    const long long total = (long long)K * N;
+    copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, ldb, K, N, Bp, ldbp, gate);
+    ++*launches;
+  }
   return cudaGetLastError();
 }
 

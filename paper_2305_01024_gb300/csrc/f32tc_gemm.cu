@@ -1,0 +1,775 @@
+// f32tc_gemm.cu -- fp32 GEMM with online block- and warp-level ABFT on the
+// tensor cores (f32tc.cuh gives the arithmetic: three exact bf16 planes per
+// operand, six bf16 MMAs per product, fp32 accumulation in registers).
+//
+// A 2-CTA cluster computes a 256 x BN tile of C with cta_group::2 MMAs, each
+// CTA its own 128 rows, as the bf16 kernel does (tc_gemm.cu).  Warp 0 issues
+// TMA loads (the three planes of an operand tile in one 3-D box), warp 1 of
+// the even CTA the MMAs: per 32-element chunk of K the six plane products,
+// smallest first, into one of the tensor-memory accumulators.  Eight epilogue
+// warps read each finished chunk and add it to the accumulators they hold in
+// registers (thread = 4 rows x BN / 8 columns), while the MMAs of the next chunks
+// run.  At the end of a verification period they inject the scheduled faults
+// (Section 5.3), form the unit's row and column sums, compare them with the
+// checksums and locate and correct (Section 4.2.1), exactly as the CUDA-core
+// kernel does on its fragments (simt_ftgemm.cuh).
+//
+// The checksums (Eq. 4) come from the same kernel (SUMS = true) run first on
+// the encoded operands: (e^T A) B and A (B e), one result per segment of at
+// most 256 of K, all segments in parallel; the main kernel adds a period's
+// segments to the running checksums when it verifies the period.  They cost
+// the units' share of a tile (1/128 of the product each for 128 x 128 units)
+// instead of an extra operand row in every MMA, so the verification unit
+// stays the schedule's own tile.
+#include <climits>
+#include <cstddef>
+
+#include "f32tc.cuh"
+#include "ptx.cuh"
+
+namespace ftg {
+
+// BN = 256: the large-problem tile, units of 64 rows and columns or more.
+// BN = 128: finer waves for small problems, units from 16.  The issuing
+// thread needs 64 cycles or more per MMA, which is what a 256 x 128 one runs
+// for, and some 300 between chunks; a 256 x 256 one runs 128 and its queue
+// covers the gap (8192^3 without checksums: 1080 cycles a chunk of 256 x 128,
+// 1560 of 256 x 256, against 768 and 1536 of MMA time; 4.4 and 3.5 ms).
+// What bounds it at BN = 256: the tensor cores without checksums (16384^3
+// 29.4-30.6 ms, 290 TFLOP/s = 1740 of bf16 MMAs, the power cap); with block
+// checksums the verification, which stops the MMAs once both accumulators are
+// full (34-36 ms; the CUDA-core kernel 133.8).
+template <int BN>
+struct F32TcCfg {
+  static constexpr int BM = F32TC_BM, KC = F32TC_KC;
+  static constexpr int A_BYTES = 3 * BM * KC * 2;        // three planes, 64-byte rows
+  static constexpr int B_BYTES = 3 * (BN / 2) * KC * 2;  // this CTA's half of the columns
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = 4;
+  static constexpr int NBUF = 512 / BN;                  // tensor-memory accumulators
+  // warps: TMA, MMA, two idle (register hand-over works on groups of four),
+  // then the epilogue's, EW / 4 per tensor-memory lane quarter
+  static constexpr int EW0 = 4, EW = BN == 256 ? 16 : 8, EPI_T = 32 * EW, THREADS = 32 * (EW0 + EW);
+  static constexpr int CPT = BN / (EW / 4);              // columns per epilogue warp
+  static constexpr int GC = BN == 256 ? 64 : 16;         // columns per row partial: the smallest unit
+  static constexpr int GR = BN == 256 ? 32 : 16;         // rows per column partial
+  static constexpr int MAXE = 128 * (BN / GC) + BN * (128 / GC);  // checksum entries with the smallest units
+  static constexpr int MAXU = 128 / GC * (BN / GC);      // units per CTA tile
+  static constexpr int MN_BOX = 64 * KC * 2;             // one plane's 64-column box
+  // registers: 64 accumulators a thread and the rest of the epilogue need
+  // more than an even split over 640 threads; the TMA / MMA group gives up
+  // part of its share
+  static constexpr bool SPLIT_REGS = BN == 256;
+  static constexpr int REGS = 96, REGS_LOW = 64, REGS_EPI = 104;
+  static_assert(4 * REGS_LOW + EW * REGS_EPI <= (4 + EW) * REGS, "register hand-over");
+};
+
+template <int BN>
+struct F32TcTail {
+  using Cfg = F32TcCfg<BN>;
+  // verification: partial sums, and (while a flagged period is confirmed)
+  // the fp64 sums and flags of its entries
+  alignas(16) float colpart[128 / Cfg::GR][BN];  // column sums of GR rows
+  float rowpart[BN / Cfg::GC][128];     // row sums of GC columns
+  double sum64[Cfg::MAXE];
+  uint8_t eflag[Cfg::MAXE];
+  float c[Cfg::MAXE];                   // running checksums: rows per column unit, then columns per row unit
+  float d[Cfg::MAXE];                   // the coming period's checksum segments, copied ahead
+  float tn[Cfg::MAXE];                  // norm term of each entry's threshold
+  float sFA[128 / Cfg::GC], sFB[BN / Cfg::GC];
+  uint64_t full[Cfg::STAGES], empty[Cfg::STAGES], acc_full[Cfg::NBUF], acc_empty[Cfg::NBUF];
+  unsigned long long bestr[Cfg::MAXU], bestc[Cfg::MAXU];
+  double fix_delta[Cfg::MAXU];
+  int nr[Cfg::MAXU], nc[Cfg::MAXU], fix_row[Cfg::MAXU], fix_col[Cfg::MAXU];
+  uint32_t tmem_base;
+  int abort;
+};
+
+template <int BN>
+constexpr size_t f32tc_smem() {
+  static_assert(offsetof(F32TcTail<BN>, colpart) % 16 == 0 && offsetof(F32TcTail<BN>, sum64) % 8 == 0, "vector access");
+  static_assert(1024 + F32TcCfg<BN>::STAGES * F32TcCfg<BN>::STAGE_BYTES + sizeof(F32TcTail<BN>) <= 227 * 1024,
+                "shared memory of one CTA");
+  return 1024 + (size_t)F32TcCfg<BN>::STAGES * F32TcCfg<BN>::STAGE_BYTES + sizeof(F32TcTail<BN>);
+}
+
+// Shared-memory descriptors: K-major tile of 64-byte rows, 64-byte swizzle
+// (8-row groups 512 bytes apart); MN-major tile of 128-byte swizzled boxes of
+// 64 columns x KC k-rows (8-row groups along K 1024 bytes apart, the next 64
+// columns `group` bytes further).
+__device__ __forceinline__ uint64_t desc_k_sw64(const void* p) {
+  return (uint64_t)((smem_u32(p) & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 |
+         (uint64_t)1 << 46 | (uint64_t)4 << 61;
+}
+__device__ __forceinline__ uint64_t desc_mn_sw128(const void* p, uint32_t group) {
+  return (uint64_t)((smem_u32(p) & 0x3FFFFu) >> 4) | (uint64_t)((group >> 4) & 0x3FFF) << 16 |
+         (uint64_t)(1024 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)2 << 61;
+}
+
+// 16 tensor-memory lanes x 32 columns in the 16x256b shape: registers 4j ..
+// 4j + 3 hold (row t/4, columns 8j + 2(t%4), + 1) and (row t/4 + 8, the same
+// columns) of lane t.
+__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+        "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Half of a reduce-scatter step: the N values of v, each summed with the
+// partner's over lane bit `o`, the lanes with the bit set keeping the upper
+// N / 2 of them (in v[0 .. N/2)).
+template <int N>
+__device__ __forceinline__ void fold(float* v, int lane, int o) {
+  const bool up = lane & o;
+#pragma unroll
+  for (int e = 0; e < N / 2; ++e) {
+    const float lo = v[e], hi = v[N / 2 + e];
+    v[e] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+  }
+}
+
+// (d0, d1) += (a0, a1), packed
+__device__ __forceinline__ void acc2(float& d0, float& d1, float a0, float a1) {
+  asm("{\n.reg .b64 ra, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rd, {%0, %1};\n add.rn.f32x2 rd, rd, ra;\n"
+      " mov.b64 {%0, %1}, rd;\n}"
+      : "+f"(d0), "+f"(d1)
+      : "f"(a0), "f"(a1));
+}
+
+// One unit of work of a CTA pair.  MAIN: a tile of C over one split of K.
+// SUMS: a tile of a checksum product over one segment of K.
+struct F32TcItem {
+  int type;            // SUMS: 0 (e^T A) B, 1 (B e)^T A^T
+  int row0, col0;      // of the pair's tile
+  int z, seg;          // split (MAIN), segment (SUMS)
+  int k0, klen;
+};
+
+template <int BN, bool SUMS>
+__device__ __forceinline__ int f32tc_items(const F32TcParams& p) {
+  if constexpr (!SUMS) return p.nsplit * p.tiles_m2 * p.tiles_n;
+  const int n0 = (p.nv + 255) / 256 * ((p.N + BN - 1) / BN), n1 = (p.nw + 255) / 256 * ((p.M + BN - 1) / BN);
+  return p.nsplit * p.segs_per_split * (n0 + n1);
+}
+
+template <int BN, bool SUMS>
+__device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
+  F32TcItem t;
+  if constexpr (!SUMS) {
+    const int tiles = p.tiles_m2 * p.tiles_n;
+    t.z = id / tiles;
+    id -= t.z * tiles;
+    const int per_group = p.group_m * p.tiles_n, first = id / per_group * p.group_m;
+    const int gsize = min(p.tiles_m2 - first, p.group_m), in = id % per_group;
+    t.type = 0;
+    t.seg = 0;
+    t.row0 = (first + in % gsize) * 256;
+    t.col0 = in / gsize * BN;
+    t.k0 = t.z * p.k_per_split;
+    t.klen = min(p.k_per_split, p.K - t.k0);
+  } else {
+    const int c0 = (p.N + BN - 1) / BN, c1 = (p.M + BN - 1) / BN;
+    const int n0 = (p.nv + 255) / 256 * c0, n1 = (p.nw + 255) / 256 * c1;
+    t.seg = id / (n0 + n1);
+    int j = id - t.seg * (n0 + n1);
+    t.type = j >= n0;
+    if (t.type) j -= n0;
+    const int cols = t.type ? c1 : c0;
+    t.row0 = j / cols * 256;
+    t.col0 = j % cols * BN;
+    t.z = t.seg / p.segs_per_split;
+    const int s0 = (t.seg - t.z * p.segs_per_split) * p.seg;  // inside the split
+    t.k0 = t.z * p.k_per_split + s0;
+    t.klen = min(p.seg, min(p.k_per_split - s0, p.K - t.k0));
+    if (t.klen < 0) t.klen = 0;
+  }
+  return t;
+}
+
+template <int BN, bool ABFT, bool SUMS>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREADS, 1)
+    f32tc_kernel(const __grid_constant__ F32TcMaps maps, const __grid_constant__ F32TcParams p) {
+  using Cfg = F32TcCfg<BN>;
+  constexpr int S = Cfg::STAGES, NBUF = Cfg::NBUF, CPT = Cfg::CPT, KC = Cfg::KC, EPI_T = Cfg::EPI_T;
+  if (*p.bad) return;  // an operand outside the split's range: the CUDA-core kernel runs instead
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* base = smem_raw + (-smem_u32(smem_raw) & 1023u);  // (shared address space kept)
+  F32TcTail<BN>& T = *reinterpret_cast<F32TcTail<BN>*>(base + S * Cfg::STAGE_BYTES);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_ctarank();
+  const bool leader = rank == 0;
+  const int worker = blockIdx.x >> 1, workers = gridDim.x >> 1;
+  const int items = f32tc_items<BN, SUMS>(p), nch = (p.K + KC - 1) / KC;
+  auto sA = [&](int s) { return base + s * Cfg::STAGE_BYTES; };
+  auto sB = [&](int s) { return base + s * Cfg::STAGE_BYTES + Cfg::A_BYTES; };
+
+  if (tid == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&T.full[s], 1);
+      mbar_init(&T.empty[s], 1);
+    }
+    for (int a = 0; a < NBUF; ++a) {
+      mbar_init(&T.acc_full[a], 1);
+      mbar_init(&T.acc_empty[a], 2 * Cfg::EW);  // one arrival per epilogue warp of both CTAs
+    }
+    T.abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(&T.tmem_base, 512);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // the leader's barriers are initialised before the other CTA signals them
+  tc_fence_after();
+  const uint32_t tmem = T.tmem_base;
+
+  if (warp < Cfg::EW0) {
+    if constexpr (Cfg::SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Cfg::REGS_LOW));
+  if (warp == 0 && lane == 0) {
+    // ---- TMA producer: this CTA's 128 rows and its half of the columns ----
+    uint32_t it = 0;
+    bool dead = false;
+    for (int id = worker; id < items && !dead; id += workers) {
+      const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
+      const CUtensorMap* mA = !SUMS ? &maps.A : (x.type ? &maps.W : &maps.V);
+      const bool kmajor_b = SUMS && x.type;
+      const int row = x.row0 + rank * 128, col = x.col0 + rank * (BN / 2);
+      for (int k = 0; k < x.klen; k += KC, ++it) {
+        const int s = it % S;
+        if (it >= S && !mbar_wait(&T.empty[s], ((it / S) & 1u) ^ 1u)) {
+          dead = true;
+          break;
+        }
+        const uint32_t cbar = mapa_rank(&T.full[s], 0);
+        if (leader) mbar_arrive_expect_tx(&T.full[s], 2 * Cfg::STAGE_BYTES);
+        const int chunk = (x.k0 + k) / KC;
+        tma_load_2d_pair(sA(s), mA, cbar, 0, (row / 128 * nch + chunk) * 192);
+        if (kmajor_b) {
+          // rows col .. col + BN/2 - 1 of A, plane by plane in 64-row pieces
+#pragma unroll
+          for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+            for (int g = 0; g < BN / 128; ++g)
+              tma_load_2d_pair(sB(s) + (pl * (BN / 128) + g) * 4096, &maps.An, cbar, 0,
+                               ((col + 64 * g) / 128 * nch + chunk) * 192 + pl * 64 + (col + 64 * g) % 128 / 2);
+        } else {
+#pragma unroll
+          for (int g = 0; g < BN / 128; ++g)
+            tma_load_2d_pair(sB(s) + g * 3 * Cfg::MN_BOX, &maps.B, cbar, 0, ((col / 64 + g) * nch + chunk) * 96);
+        }
+      }
+    }
+    if (dead) atomicExch(&T.abort, 1);
+    // let the last loads land before the CTAs may exit (bounded)
+    if (leader)
+      for (uint32_t q = it > (uint32_t)S ? it - S : 0; q < it; ++q) mbar_wait(&T.full[q % S], (q / S) & 1u);
+  } else if (warp == 1 && lane == 0 && leader) {
+    // ---- MMA issuer: per chunk the six plane products, smallest first ----
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((256u >> 4) << 24);
+    uint32_t it = 0;
+    bool dead = false;
+    for (int id = worker; id < items && !dead; id += workers) {
+      const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
+      const bool kmajor_b = SUMS && x.type;
+      const uint32_t id_t = kmajor_b ? idesc : idesc | (1u << 16);  // B MN-major
+      for (int k = 0; k < x.klen; k += KC, ++it) {
+        const int s = it % S, ab = it % NBUF;
+        if ((it >= (uint32_t)NBUF && !mbar_wait(&T.acc_empty[ab], ((it / NBUF) & 1u) ^ 1u)) ||
+            !mbar_wait(&T.full[s], (it / S) & 1u)) {
+          dead = true;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(ab * BN);
+        const uint64_t da = desc_k_sw64(sA(s));
+        // planes of the operands, smallest product first; 16 elements of K at a time
+        auto products = [&](uint64_t db, uint32_t pb, uint32_t kb, int nk16) {
+          constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+          for (int q = 0; q < 6; ++q)
+#pragma unroll
+            for (int kk = 0; kk < KC / 16; ++kk)
+              if (kk < nk16)
+                tc_mma_f16_pair(d, da + (uint64_t)(PA[q] * (128 * KC * 2 >> 4) + kk * 2),
+                                db + (uint64_t)(PB[q] * pb + kk * kb), id_t, (q | kk) != 0);
+        };
+        constexpr uint32_t PB_MN = Cfg::MN_BOX >> 4, PB_K = (BN / 2) * KC * 2 >> 4;
+        if (!kmajor_b) {
+          const uint64_t db = desc_mn_sw128(sB(s), 3 * Cfg::MN_BOX);
+          if (x.klen - k > KC / 2) products(db, PB_MN, 16 * 128 >> 4, KC / 16);
+          else products(db, PB_MN, 16 * 128 >> 4, 1);
+        } else {
+          const uint64_t db = desc_k_sw64(sB(s));
+          if (x.klen - k > KC / 2) products(db, PB_K, 2, KC / 16);
+          else products(db, PB_K, 2, 1);
+        }
+        tc_commit_pair(&T.empty[s], (uint16_t)3);
+        tc_commit_pair(&T.acc_full[ab], (uint16_t)3);
+      }
+    }
+    if (dead) atomicExch(&T.abort, 1);
+    // let the last MMAs finish before tensor memory may be released (bounded)
+    if (it > 0) mbar_wait(&T.acc_full[(it - 1) % NBUF], ((it - 1) / NBUF) & 1u);
+    }
+  } else {
+    if constexpr (Cfg::SPLIT_REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Cfg::REGS_EPI));
+    // ---- epilogue: accumulate, verify, store -------------------------------
+    // Thread layout of the accumulators (the 16x256b tensor-memory shape): rows
+    // rbase + 8 i, columns cbase + 8 j + b.  Column sums then need 3 shuffle
+    // levels instead of the 5 of one row per lane, and C is written straight
+    // from registers in whole 32-byte sectors.
+    constexpr int NJ = CPT / 8;
+    const int lq = warp & 3, eh = (warp - Cfg::EW0) >> 2, q = (warp - Cfg::EW0) * 32 + lane;
+    const int rbase = lq * 32 + (lane >> 2), cbase = eh * CPT + 2 * (lane & 3);
+    uint32_t it = 0;
+    bool dead = false;
+    float acc[4][NJ][2];
+    // Hand a chunk's accumulator back to the MMA thread (in the leader CTA).
+    // Relaxed: the reads completed (wait::ld) and no store precedes, so the
+    // arrival has nothing to publish.  With release at cluster scope, an
+    // arrival cost each warp some 1700 cycles a chunk, twice the chunk's MMAs
+    // of 256 x 128 (8192^3 without checksums: 7.0 ms against 4.9).
+    auto acc_release = [&](int ab) {
+      asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa_rank(&T.acc_empty[ab], 0))
+                   : "memory");
+    };
+    // the tile's rows < rows and columns < cols from the registers to memory
+    auto store = [&](float* out, long long ld, int rows, int cols, float alpha, float beta, bool vec) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int tr = rbase + 8 * i;
+        if (tr >= rows) continue;
+        float* line = out + (long long)tr * ld + cbase;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const int tc = cbase + 8 * j;
+          float2 o = make_float2(alpha * acc[i][j][0], alpha * acc[i][j][1]);
+          if (vec && tc + 1 < cols) {
+            if (beta != 0.f) {
+              const float2 ci = *reinterpret_cast<const float2*>(line + 8 * j);
+              o = make_float2(fmaf(beta, ci.x, o.x), fmaf(beta, ci.y, o.y));
+            }
+            *reinterpret_cast<float2*>(line + 8 * j) = o;
+          } else {
+            if (tc < cols) line[8 * j] = beta != 0.f ? fmaf(beta, line[8 * j], o.x) : o.x;
+            if (tc + 1 < cols) line[8 * j + 1] = beta != 0.f ? fmaf(beta, line[8 * j + 1], o.y) : o.y;
+          }
+        }
+      }
+    };
+
+    for (int id = worker; id < items; id += workers) {
+      const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
+      const int row0 = x.row0 + rank * 128, col0 = x.col0;
+      // schedule k-steps of this split, and its verification periods
+      const int ks0 = x.z * p.ks_per_split, ks1 = min(ks0 + p.ks_per_split, p.ksteps);
+      const int um_sh = 31 - __clz(p.um), un_sh = 31 - __clz(p.un);
+      const int nRow = ABFT ? 128 * (BN >> un_sh) : 0, nE = ABFT ? nRow + BN * (128 >> um_sh) : 0;
+      int period = 0, next_ks = INT_MAX;  // next_ks: k-step that ends the current period
+      bool has_fault = false;
+      if constexpr (!SUMS) {
+        next_ks = min(ks0 + (ABFT ? p.cadence : p.ks_per_split), ks1) - 1;
+        if (p.nfaults > 0) {
+          // any scheduled fault in the schedule tiles this CTA tile covers?
+          const int tm0 = row0 / p.m_tb, tn0 = col0 / p.n_tb;
+          const int ntr = row0 < p.M ? (min(row0 + 128, p.M) - 1) / p.m_tb - tm0 + 1 : 0;
+          const int ntc = (min(col0 + BN, p.N) - 1) / p.n_tb - tn0 + 1;
+          bool mine = false;
+          for (int t = lane; t < ntr * ntc; t += 32) {
+            const int tile = (tm0 + t / ntc) * p.tiles_n_sched + tn0 + t % ntc;
+            const int f = first_fault(p.faults, p.nfaults, tile);
+            mine |= f < p.nfaults && p.faults[f].tile == tile;
+          }
+          has_fault = __any_sync(0xffffffffu, mine);
+        }
+      }
+      // the checksum segment g of the current period at entry e: its address
+      // (null outside the matrix) for g = 0 and the distance to the next
+      auto seg_of = [&](int e, long long* stride) -> const float* {
+        const int s0 = x.z * p.segs_per_split + period * p.segs_per_period;
+        if (e < nRow) {
+          const int J = (col0 >> un_sh) + (e >> 7), gr = row0 + (e & 127);
+          *stride = (long long)p.nw * p.ldr_d;
+          return J < p.nw && gr < p.M ? p.Dr + ((long long)s0 * p.nw + J) * p.ldr_d + gr : nullptr;
+        }
+        const int I = (row0 >> um_sh) + (e - nRow) / BN, gc = col0 + (e - nRow) % BN;
+        *stride = (long long)p.nv * p.ldc_d;
+        return I < p.nv && gc < p.N ? p.Dc + ((long long)s0 * p.nv + I) * p.ldc_d + gc : nullptr;
+      };
+      // start copying the first segment of the current period for this
+      // thread's entries; it lands while the period's MMAs run
+      auto fetch_segments = [&]() {
+        for (int e = q; e < nE; e += EPI_T) {
+          long long stride;
+          const float* src = seg_of(e, &stride);
+          if (src)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(&T.d[e])), "l"(src) : "memory");
+          else
+            T.d[e] = 0.f;
+        }
+      };
+      if constexpr (ABFT) {
+        // Frobenius norms of the units' rows and columns
+        auto fro = [](const float* sq16, int first, int per, int count) {
+          float s = 0.f;
+          for (int g = 0; g < per && first + g < count; ++g) s += sq16[first + g];
+          return sqrtf(s);
+        };
+        if (q < 128 >> um_sh) T.sFA[q] = fro(p.sq16a, row0 / 16 + q * (p.um / 16), p.um / 16, (p.M + 15) / 16);
+        if (q < BN >> un_sh) T.sFB[q] = fro(p.sq16b, col0 / 16 + q * (p.un / 16), p.un / 16, (p.N + 15) / 16);
+        bar_red_or(1, EPI_T, 0);
+        for (int e = q; e < nE; e += EPI_T) {
+          T.c[e] = 0.f;
+          // lambda * u times the norms, rounded as ft_tau does
+          const int gr = row0 + (e & 127), gc = col0 + (e - nRow) % BN;
+          T.tn[e] = e < nRow ? __fmul_rn(__fmul_rn(p.lam_u, gr < p.M ? p.nA[gr] : 0.f), T.sFB[e >> 7])
+                             : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), gc < p.N ? p.nB[gc] : 0.f);
+        }
+        fetch_segments();
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) acc[i][j][0] = acc[i][j][1] = 0.f;
+
+      for (int k = 0; k < x.klen; k += KC, ++it) {
+        const int ab = it % NBUF;
+        const bool ok = !dead && mbar_wait(&T.acc_full[ab], (it / NBUF) & 1u);
+        if (!ok && !dead) {
+          dead = true;
+          atomicExch(&T.abort, 1);
+        }
+        tc_fence_after();
+        __syncwarp();
+        if (ok) {
+          const uint32_t tl = tmem + (uint32_t)(ab * BN + eh * CPT) + ((uint32_t)(lq * 32) << 16);
+          // 32 columns of 16 rows are added while the next load is in flight
+          constexpr int NL = CPT / 16;
+          float v[2][16];
+          auto load = [&](int l) { tmem_ld_16x256b_x4(tl + l / 2 * 32 + ((uint32_t)(l % 2 * 16) << 16), v[l & 1]); };
+          load(0);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            tmem_wait_ld();
+            if (l + 1 < NL) load(l + 1);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float(&lo)[2] = acc[2 * (l & 1)][4 * (l >> 1) + j];
+              float(&hi)[2] = acc[2 * (l & 1) + 1][4 * (l >> 1) + j];
+              acc2(lo[0], lo[1], v[l & 1][4 * j], v[l & 1][4 * j + 1]);
+              acc2(hi[0], hi[1], v[l & 1][4 * j + 2], v[l & 1][4 * j + 3]);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) acc_release(ab);
+
+        if constexpr (!SUMS) {
+          // the last schedule k-step complete after this chunk
+          const int done = k + KC >= x.klen ? ks1 - 1 : ks0 + (k + KC) / p.k_tb - 1;
+          if (done < next_ks) continue;
+          const int ks = next_ks, ks_first = ks0 + period * (ABFT ? p.cadence : p.ks_per_split);
+          // ----- faults scheduled in this period (Section 5.3): additive
+          // offsets on the accumulators or the running checksums -----
+          if (has_fault) {
+            const int tm0 = row0 / p.m_tb, tn0 = col0 / p.n_tb;
+            const int tm1 = (min(row0 + 128, p.M) - 1) / p.m_tb, tn1 = (min(col0 + BN, p.N) - 1) / p.n_tb;
+            for (int tm = tm0; tm <= tm1; ++tm)
+              for (int tn = tn0; tn <= tn1; ++tn) {
+                const int tile = tm * p.tiles_n_sched + tn;
+                for (int f = first_fault(p.faults, p.nfaults, tile); f < p.nfaults && p.faults[f].tile == tile; ++f) {
+                  const Fault F = p.faults[f];
+                  if (F.kstep < ks_first || F.kstep > ks) continue;
+                  const int fr = tm * p.m_tb + F.row - row0, fc = tn * p.n_tb + F.col - col0;
+                  if (F.target == T_ACC) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                      for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                        for (int b = 0; b < 2; ++b)
+                          if (rbase + 8 * i == fr && cbase + 8 * j + b == fc) acc[i][j][b] += F.delta;
+                  } else if constexpr (ABFT) {
+                    const int e = F.target == T_ROWSUM ? fc / p.un * 128 + fr : nRow + fr / p.um * BN + fc;
+                    if (e % EPI_T == q) T.c[e] += F.delta;  // the thread that keeps the entry
+                  }
+                }
+              }
+          }
+          if constexpr (ABFT) {
+            // ----- verification: partial sums of GC columns of each row and
+            // of GR rows of each column -----
+            constexpr int GC = Cfg::GC, GR = Cfg::GR;
+            // this thread's running checksums through the period
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            const int segs = min(p.segs_per_period, p.segs_per_split - period * p.segs_per_period);
+            for (int e = q; e < nE; e += EPI_T) {
+              float c = T.c[e] + T.d[e];
+              if (segs > 1) {  // periods longer than a segment
+                long long stride;
+                const float* src = seg_of(e, &stride);
+                for (int g = 1; src && g < segs; ++g) c += __ldg(src + g * stride);
+              }
+              T.c[e] = c;
+            }
+            {
+              // rows: this thread's columns of each group, then its quad's
+              constexpr int NG = CPT / GC, JG = GC / 8;
+              float t[NG * 4];
+#pragma unroll
+              for (int g = 0; g < NG; ++g)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  float s[JG][2];
+#pragma unroll
+                  for (int j = 0; j < JG; ++j) {
+                    s[j][0] = acc[i][g * JG + j][0];
+                    s[j][1] = acc[i][g * JG + j][1];
+                  }
+#pragma unroll
+                  for (int st = JG / 2; st > 0; st >>= 1)
+#pragma unroll
+                    for (int j = 0; j < st; ++j) acc2(s[j][0], s[j][1], s[j + st][0], s[j + st][1]);
+                  t[g * 4 + i] = s[0][0] + s[0][1];
+                }
+              fold<NG * 4>(t, lane, 2);
+              fold<NG * 2>(t, lane, 1);
+              const int v0 = (lane & 2 ? NG * 2 : 0) + (lane & 1 ? NG : 0);
+#pragma unroll
+              for (int e = 0; e < NG; ++e) T.rowpart[eh * NG + (v0 + e) / 4][rbase + 8 * ((v0 + e) % 4)] = t[e];
+            }
+            {
+              // columns: this thread's rows of each group, then 8 lanes'
+              constexpr int NG = 32 / GR, IG = 4 / NG, NV = NG * NJ * 2;
+              static_assert(NV >= 16, "three folds leave pairs");
+              float t[NV];
+#pragma unroll
+              for (int g = 0; g < NG; ++g)
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                  float(&d)[2] = *reinterpret_cast<float(*)[2]>(&t[(g * NJ + j) * 2]);
+                  d[0] = acc[g * IG][j][0];
+                  d[1] = acc[g * IG][j][1];
+#pragma unroll
+                  for (int i = 1; i < IG; ++i) acc2(d[0], d[1], acc[g * IG + i][j][0], acc[g * IG + i][j][1]);
+                }
+              fold<NV>(t, lane, 16);
+              fold<NV / 2>(t, lane, 8);
+              fold<NV / 4>(t, lane, 4);
+              const int v0 = (lane & 16 ? NV / 2 : 0) + (lane & 8 ? NV / 4 : 0) + (lane & 4 ? NV / 8 : 0);
+#pragma unroll
+              for (int e = 0; e < NV / 8; e += 2) {
+                const int g = (v0 + e) / (NJ * 2), j = (v0 + e) % (NJ * 2) / 2;
+                *reinterpret_cast<float2*>(&T.colpart[lq * NG + g][cbase + 8 * j]) = make_float2(t[e], t[e + 1]);
+              }
+            }
+            bar_red_or(1, EPI_T, 0);
+            // growth term of the threshold after k elements of K in this split
+            const float grow = __fmul_rn(p.mu_u, sqrtf((float)(min((ks + 1) * p.k_tb, p.K) - ks0 * p.k_tb)));
+            // threshold of entry e with checksum c
+            auto tau_of = [&](int e, float c) { return __fmaf_rn(grow, fabsf(c), T.tn[e]); };
+            unsigned flags = 0u;
+            const int row_per = p.un / GC, col_per = p.um / GR;
+#pragma unroll 1
+            for (int i = 0; i < Cfg::MAXE / EPI_T; ++i) {
+              const int e = q + i * EPI_T;
+              if (e >= nE) break;
+              const float c = T.c[e];
+              const bool is_row = e < nRow;
+              const int sh = is_row ? 7 : BN == 256 ? 8 : 7;  // entries of a line of partial sums
+              const int per = is_row ? row_per : col_per, at = is_row ? e : e - nRow;
+              const float* src = (is_row ? &T.rowpart[0][0] : &T.colpart[0][0]) + ((at >> sh) * per << sh) + (at & ((1 << sh) - 1));
+              float s = 0.f;
+#pragma unroll
+              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g)
+                if (g < per) s += src[g << sh];
+              if (ok && fabsf(s - c) > kScreen * tau_of(e, c)) flags |= 1u << i;
+            }
+            if (bar_red_or(1, EPI_T, flags != 0u)) {
+              // ----- fp64 confirmation of the screened entries -----
+              const int units_n = BN / p.un, units = units_n * (128 / p.um);
+              int i = 0;
+              for (int e = q; e < nE; e += EPI_T, ++i) {
+                T.eflag[e] = (flags >> i) & 1u;
+                T.sum64[e] = 0.0;
+              }
+              if (q < units) {
+                T.nr[q] = 0; T.nc[q] = 0; T.bestr[q] = 0ull; T.bestc[q] = 0ull; T.fix_row[q] = -1;
+              }
+              bar_red_or(1, EPI_T, 0);
+#pragma unroll
+              for (int i2 = 0; i2 < 4; ++i2) {
+                const int r = rbase + 8 * i2;
+#pragma unroll
+                for (int g = 0; g < CPT / GC; ++g) {
+                  const int e = ((eh * CPT + GC * g) >> un_sh) * 128 + r;
+                  if (T.eflag[e]) {
+                    double s = 0.0;
+#pragma unroll
+                    for (int j = 0; j < GC / 8; ++j) s += (double)acc[i2][g * (GC / 8) + j][0] + (double)acc[i2][g * (GC / 8) + j][1];
+                    atomicAdd(&T.sum64[e], s);
+                  }
+                }
+#pragma unroll
+                for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                  for (int b = 0; b < 2; ++b) {
+                    const int e = nRow + (r >> um_sh) * BN + cbase + 8 * j + b;
+                    if (T.eflag[e]) atomicAdd(&T.sum64[e], (double)acc[i2][j][b]);
+                  }
+              }
+              bar_red_or(1, EPI_T, 0);
+              i = 0;
+              for (int e = q; e < nE; e += EPI_T, ++i) {
+                if (!((flags >> i) & 1u)) continue;
+                const float c = T.c[e], tau = tau_of(e, c);
+                const double d = T.sum64[e] - (double)c;
+                if (!(fabs(d) > (double)tau)) continue;
+                const float sc = flag_score((float)d, tau);
+                if (e < nRow) {
+                  const int u = (e & 127) / p.um * units_n + (e >> 7);
+                  atomicAdd(&T.nr[u], 1);
+                  atomicMax(&T.bestr[u], flag_key(sc, e & 127));
+                } else {
+                  const int col = (e - nRow) % BN, u = (e - nRow) / BN * units_n + col / p.un;
+                  atomicAdd(&T.nc[u], 1);
+                  atomicMax(&T.bestc[u], flag_key(sc, col));
+                }
+              }
+              bar_red_or(1, EPI_T, 0);
+              if (q < units && (T.nr[q] | T.nc[q])) {
+                const int nr = T.nr[q], nc = T.nc[q];
+                const int ir = nr ? key_index(T.bestr[q]) : -1, jc = nc ? key_index(T.bestc[q]) : -1;
+                const int er = nr ? q % units_n * 128 + ir : 0, ec = nc ? nRow + q / units_n * BN + jc : 0;
+                const double dR = nr ? T.sum64[er] - (double)T.c[er] : 0.0, dC = nc ? T.sum64[ec] - (double)T.c[ec] : 0.0;
+                const float tR = nr ? tau_of(er, T.c[er]) : 0.f, tC = nc ? tau_of(ec, T.c[ec]) : 0.f;
+                ftgemm_fault_record rec;
+                rec.tile_m = (row0 + q / units_n * p.um) / p.m_tb;
+                rec.tile_n = (col0 + q % units_n * p.un) / p.n_tb;
+                rec.kstep = ks;
+                rec.problem = 0; rec.reserved = 0;
+                rec.row = nr ? row0 + ir : -1;
+                rec.col = nc ? col0 + jc : -1;
+                rec.residual_r = dR; rec.residual_c = dC; rec.tau = (double)tR + (double)tC;
+                rec.delta = 0.0;
+                if (nr == 1 && nc == 1) {
+                  if (fabs(dR - dC) <= (double)tR + (double)tC) {
+                    rec.kind = K_CORRECTED; rec.delta = dR;
+                    T.fix_row[q] = ir; T.fix_col[q] = jc; T.fix_delta[q] = dR;
+                  } else {
+                    rec.kind = K_UNCORRECTABLE;
+                  }
+                } else if (nr == 1 && nc == 0) {
+                  rec.kind = K_CHECKSUM; rec.delta = -dR; T.c[er] = (float)T.sum64[er];
+                } else if (nr == 0 && nc == 1) {
+                  rec.kind = K_CHECKSUM; rec.delta = -dC; T.c[ec] = (float)T.sum64[ec];
+                } else {
+                  rec.kind = K_UNCORRECTABLE;
+                }
+                report_event(p.rep, p.recs, rec);
+              }
+              bar_red_or(1, EPI_T, 0);
+              // ----- correct the located elements (Section 4.2.1) -----
+#pragma unroll
+              for (int i2 = 0; i2 < 4; ++i2)
+#pragma unroll
+                for (int g = 0; g < CPT / GC; ++g) {
+                  const int r = rbase + 8 * i2, u = (r >> um_sh) * units_n + ((eh * CPT + GC * g) >> un_sh);
+                  if (T.fix_row[u] == r) {
+#pragma unroll
+                    for (int j = g * (GC / 8); j < (g + 1) * (GC / 8); ++j)
+#pragma unroll
+                      for (int b = 0; b < 2; ++b)
+                        if (T.fix_col[u] == cbase + 8 * j + b) acc[i2][j][b] = (float)((double)acc[i2][j][b] - T.fix_delta[u]);
+                  }
+                }
+              bar_red_or(1, EPI_T, 0);  // the shared arrays are reused
+            }
+          }
+          ++period;
+          next_ks = min(next_ks + (ABFT ? p.cadence : p.ks_per_split), ks1 - 1);
+          if constexpr (ABFT) {
+            if (k + KC < x.klen) fetch_segments();
+          }
+        }
+      }
+      if (dead) continue;
+      if constexpr (SUMS) {
+        const int nu = x.type ? p.nw : p.nv;
+        const long long ld = x.type ? p.ldr_d : p.ldc_d;
+        float* out = (x.type ? p.Dr : p.Dc) + ((long long)x.seg * nu + row0) * ld + col0;
+        store(out, ld, nu - row0, (x.type ? p.M : p.N) - col0, 1.f, 0.f, true);
+      } else if (p.partial) {
+        store(p.partial + ((long long)x.z * p.M + row0) * p.N + col0, p.N, p.M - row0, p.N - col0, 1.f, 0.f,
+              (p.N & 1) == 0);
+      } else {
+        store(p.C + (long long)row0 * p.ldc + col0, p.ldc, p.M - row0, p.N - col0, p.alpha, p.beta, p.c_vec);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && T.abort) atomicAdd(&p.rep->timeouts, 1);
+  cluster_sync();  // both CTAs are done with each other's barriers and tensor memory
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, 512);
+  }
+}
+
+template <int BN, bool ABFT, bool SUMS>
+static cudaError_t f32tc_launch(const F32TcMaps& maps, const F32TcParams& p, int items, int sms, cudaStream_t st) {
+  constexpr size_t smem = f32tc_smem<BN>();
+  cudaError_t e = cudaFuncSetAttribute(f32tc_kernel<BN, ABFT, SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  if constexpr (F32TcCfg<BN>::SPLIT_REGS) {
+    // the hand-over draws on what the launch allocates
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, f32tc_kernel<BN, ABFT, SUMS>);
+    if (e != cudaSuccess) return e;
+    if (fa.numRegs != F32TcCfg<BN>::REGS) return cudaErrorInvalidConfiguration;
+  }
+  const int workers = items < sms / 2 ? items : sms / 2;
+  f32tc_kernel<BN, ABFT, SUMS><<<2 * workers, F32TcCfg<BN>::THREADS, smem, st>>>(maps, p);
+  return cudaGetLastError();
+}
+
+// The checksum segments (ABFT only), then the product.  bn: columns per tile.
+template <int BN>
+static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st) {
+  if (abft) {
+    // the tile's shared arrays hold units of GC rows and columns or more
+    if (p.um < F32TcCfg<BN>::GC || p.un < F32TcCfg<BN>::GC || p.um > 128 || p.un > 128) return cudaErrorInvalidValue;
+    const long long n0 = (long long)((p.nv + 255) / 256) * ((p.N + BN - 1) / BN);
+    const long long n1 = (long long)((p.nw + 255) / 256) * ((p.M + BN - 1) / BN);
+    const long long items = (n0 + n1) * p.nsplit * p.segs_per_split;
+    if (items > INT_MAX) return cudaErrorInvalidValue;
+    cudaError_t e = f32tc_launch<BN, false, true>(maps, p, (int)items, sms, st);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+  }
+  const long long items = (long long)p.nsplit * p.tiles_m2 * p.tiles_n;
+  if (items > INT_MAX) return cudaErrorInvalidValue;
+  ++*launches;
+  return abft ? f32tc_launch<BN, true, false>(maps, p, (int)items, sms, st)
+              : f32tc_launch<BN, false, false>(maps, p, (int)items, sms, st);
+}
+
+cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches,
+                         cudaStream_t st) {
+  return bn == 256 ? f32tc_run_bn<256>(abft, maps, p, sms, launches, st)
+                   : f32tc_run_bn<128>(abft, maps, p, sms, launches, st);
+}
+
+}  // namespace ftg

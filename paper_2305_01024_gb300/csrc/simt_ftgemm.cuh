@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(T::NTHR, T::MINB)
   using L = SimtLayout<T, LEVEL>;
   using Aux = SimtAux<T, LEVEL>;
   constexpr int NV = L::NV, NW = L::NW;
+  if (p.only_if && !*p.only_if) return;
 
   extern __shared__ unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
