@@ -46,6 +46,7 @@ cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long
                                       int* launches, cudaStream_t st);
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
                                int* launches, cudaStream_t st);
+bool f32tc_scan_units(int um, int un);
 cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]);
 int tc_nb_parts(int dt, long long K);
@@ -1403,6 +1404,8 @@ struct F32TcPlan {
   long long ldc_d, ldr_d;   // row strides of the checksum segments
   int seg, segs_per_period, segs_per_split;
   long long segs;           // over all splits
+  bool by_segments;         // few tiles, long K: the product by segments, then a scan
+  long long ldp;            // row stride of the product's segments
 };
 
 // Whether the tensor-core kernel takes this fp32 call, and its layout (pairs:
@@ -1425,13 +1428,12 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
   // Where it is the faster one.  Its fixed part (operand planes, checksum
   // segments, the stand-by of the CUDA-core kernel) is worth about 2e8 flop of
   // CUDA-core work with checksums and 8e8 without, more when K is a few chunks;
-  // without checksums it also needs tiles to run side by side.  Measured, us per
+  // without checksums it also needs tiles or segments to run side by side.  Measured, us per
   // call, CUDA cores / tensor cores: BLOCK 384^3 48 / 58, 512^3 61 / 56, 1024^3
   // 129 / 66, 2048x2048x64 44 / 47, 2048x2048x128 55 / 50, 256x256x8192 418 / 275;
   // OFF 512^3 28 / 35, 768^3 44 / 40, 256x256x8192 147 / 192, 512x512x2048 83 / 67.
   const double flop = 2.0 * M * N * K;
-  const long long tiles = (long long)split * ((M + 255) / 256) * ((N + 127) / 128);
-  if (abft ? flop < 2e8 || (K < 96 && flop < 4e9) : flop < 8e8 || tiles < 6 || (K < 192 && flop < 4e9)) return false;
+  if (abft ? flop < 2e8 || (K < 96 && flop < 4e9) : flop < 8e8 || (K < 192 && flop < 4e9)) return false;
   F32TcPlan& t = *out;
   t.nch = (K + F32TC_KC - 1) / F32TC_KC;
   // rows of 128 bytes are addressed by 32-bit coordinates
@@ -1453,6 +1455,41 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
   t.segs_per_split = (int)((span + t.seg - 1) / t.seg);
   t.segs_per_period = period >= kps ? t.segs_per_split : (int)(period / t.seg);
   t.segs = (long long)split * t.segs_per_split;
+  t.by_segments = false;
+  t.ldp = ((long long)N + 3) / 4 * 4;
+  if (split == 1 && (!abft || f32tc_scan_units(um, un))) {
+    // Few tiles and a long K leave most CTA pairs idle in a pass over K; the
+    // segments of K run side by side and a scan adds them up.  Both routes in
+    // tens of SM cycles: a chunk 107 (127 with verification), the scan 135 a
+    // segment with verification, 300 for its launch, and 21 KB of segments
+    // written and read.  Measured, us per call, one pass / by segments: BLOCK
+    // 256x256x65536 1890 / 383, 512x512x8192 (32 x 32 units) 190 / 126, but
+    // 777x1531x2049 114 / 125, 2543x700x3717 189 / 197; OFF 640x640x4096 98 / 53.
+    const long long m2 = ((long long)M + 255) / 256, n1 = ((long long)N + 127) / 128, tiles = m2 * n1;
+    long long sums = 0;
+    int seg = t.seg, segs = t.segs_per_split;
+    if (abft) {
+      sums = ((M + um - 1) / um + 255) / 256 * n1 + ((N + un - 1) / un + 255) / 256 * (((long long)M + 127) / 128);
+    } else {
+      // no periods: as many segments as fill the device once, of 256 of K or more
+      segs = (int)std::min<long long>((K + 255) / 256, std::max<long long>(1, pairs / tiles));
+      seg = ((K + segs - 1) / segs + F32TC_KC - 1) / F32TC_KC * F32TC_KC;
+      segs = (K + seg - 1) / seg;
+    }
+    auto waves = [&](long long items) { return (items + pairs - 1) / pairs; };
+    const long long per = seg / F32TC_KC;
+    const long long direct = waves(tiles) * t.nch * (abft ? 127 : 107) + waves(sums * segs) * per * 107;
+    const long long scan = waves((tiles + sums) * segs) * per * 107 + (abft ? 135 : 0) * segs + 300 +
+                           8LL * segs * M * N / 21000;
+    if (segs > 1 && 4.0 * segs * M * t.ldp <= 536870912.0 && scan * 20 < direct * 19) {
+      t.by_segments = true;
+      t.bn = 128;
+      t.seg = seg;
+      t.segs = t.segs_per_split = segs;
+      if (!abft) t.segs_per_period = segs;
+    }
+  }
+  if (!abft && !t.by_segments && (long long)split * ((M + 255) / 256) * ((N + 127) / 128) < 6) return false;
   if (abft) {
     const double nv = (M + um - 1) / um, nw = (N + un - 1) / un;
     if (4.0 * t.segs * (nv * t.ldc_d + nw * t.ldr_d) > 2147483648.0) return false;  // checksum segments: 2 GiB
@@ -1464,7 +1501,7 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
 static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, double alpha, double beta, float* C,
                      int64_t ldc, bool c16, ftgemm_ft_level level, const ftgemm_schedule& s, int split,
                      int ks_per_split, int cadence, int ksteps, int tiles_n, int nf, float* Dc, float* Dr,
-                     float* partial, int* launches) {
+                     float* P, float* partial, int* launches) {
   const bool abft = level != FTGEMM_FT_OFF;
   const int bn = t.bn;
   F32TcMaps maps;
@@ -1490,7 +1527,8 @@ static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, doub
   p.m_tb = s.m_tb; p.n_tb = s.n_tb; p.k_tb = s.k_tb;
   p.tiles_n_sched = tiles_n; p.ks_per_split = ks_per_split; p.cadence = std::max(1, std::min(cadence, ks_per_split)); p.ksteps = ksteps;
   p.nA = e.nA; p.nB = e.nB; p.sq16a = e.sq16a; p.sq16b = e.sq16b;
-  p.Dc = Dc; p.Dr = Dr; p.ldc_d = t.ldc_d; p.ldr_d = t.ldr_d;
+  p.Dc = abft ? Dc : nullptr; p.Dr = abft ? Dr : nullptr; p.P = t.by_segments ? P : nullptr; p.ldp = t.ldp;
+  p.ldc_d = t.ldc_d; p.ldr_d = t.ldr_d;
   p.lam_u = (float)(h->lambda * std::ldexp(1.0, -24));
   p.mu_u = (float)(h->mu * std::ldexp(1.0, -24));
   p.C = C; p.ldc = ldc; p.c_vec = (ldc % 4 == 0) && c16;
@@ -1588,7 +1626,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   bool use_tc = !At_given && !detect && !learned && !sink &&
                 f32tc_plan(M, N, K, level, s, split, ks_per_split, cadence, m_u, n_u,
                            (h->num_sms > 0 ? h->num_sms : 148) / 2, &tc);
-  size_t oAt, oBp, oV, oW, oNa, oNb, oPart, oScr = 0, oCo = 0, oTc[9] = {};
+  size_t oAt, oBp, oV, oW, oNa, oNb, oPart, oScr = 0, oCo = 0, oTc[10] = {};
   if (use_tc) {
     auto planes = [&](int lines) { return (size_t)((lines + 127) / 128) * tc.nch * (3 * F32TC_APLANE / 2); };
     oAt = take(std::max(planes(M), nAt));
@@ -1605,6 +1643,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
       oTc[7] = take((size_t)tc.segs * nwb * tc.ldr_d);
     }
     oTc[8] = take(1);
+    if (tc.by_segments) oTc[9] = take((size_t)tc.segs * M * tc.ldp);
     if (ensure_ws(h, o) != FTGEMM_OK) {  // no room for the planes
       cudaGetLastError();
       use_tc = false;
@@ -1638,7 +1677,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     e.bad = (int*)(ws + oTc[8]);
     CK(launch_f32tc_split(Af, lda, Bf, ldb, e, &launches, h->stream));
     int rc = f32tc_run(h, tc, e, alpha, beta, C, ldc, al16(C), level, s, split, ks_per_split, cadence, ksteps, tiles_n,
-                       nf, ws + oTc[6], ws + oTc[7], split > 1 ? ws + oPart : nullptr, &launches);
+                       nf, ws + oTc[6], ws + oTc[7], ws + oTc[9], split > 1 ? ws + oPart : nullptr, &launches);
     if (rc) return rc;
     CK(launch_kmajor_operands_if(e.bad, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
                                  &launches, h->stream));

@@ -50,6 +50,9 @@ struct F32TcParams {
   const float* sq16a; const float* sq16b;  // sums of squares of every 16 rows of A / columns of B
   float* Dc; float* Dr;        // checksum segments: [seg][nv][ldc_d] and [seg][nw][ldr_d]
   long long ldc_d, ldr_d;
+  // the product itself by segments, [seg][M][ldp] (f32tc_scan.cu adds them
+  // up; one split), or null: one pass over K per tile
+  float* P; long long ldp;
   float lam_u, mu_u;
   float* C; long long ldc; int c_vec;
   float alpha, beta;

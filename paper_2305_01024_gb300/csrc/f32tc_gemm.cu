@@ -29,6 +29,8 @@
 
 namespace ftg {
 
+cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cudaStream_t st);
+
 // BN = 256: the large-problem tile, units of 64 rows and columns or more.
 // BN = 128: finer waves for small problems, units from 16.  The issuing
 // thread needs 64 cycles or more per MMA, which is what a 256 x 128 one runs
@@ -146,17 +148,32 @@ __device__ __forceinline__ void acc2(float& d0, float& d1, float a0, float a1) {
 // One unit of work of a CTA pair.  MAIN: a tile of C over one split of K.
 // SUMS: a tile of a checksum product over one segment of K.
 struct F32TcItem {
-  int type;            // SUMS: 0 (e^T A) B, 1 (B e)^T A^T
+  int type;            // SUMS: 0 (e^T A) B, 1 (B e)^T A^T, 2 A B
   int row0, col0;      // of the pair's tile
   int z, seg;          // split (MAIN), segment (SUMS)
   int k0, klen;
 };
 
+// Tiles of one segment by type.
+struct F32TcSums {
+  int cols[3], n[3];
+};
+template <int BN>
+__host__ __device__ __forceinline__ F32TcSums f32tc_sums(const F32TcParams& p) {
+  F32TcSums t;
+  t.cols[0] = t.cols[2] = (p.N + BN - 1) / BN;
+  t.cols[1] = (p.M + BN - 1) / BN;
+  t.n[0] = p.Dc ? (p.nv + 255) / 256 * t.cols[0] : 0;
+  t.n[1] = p.Dc ? (p.nw + 255) / 256 * t.cols[1] : 0;
+  t.n[2] = p.P ? p.tiles_m2 * t.cols[2] : 0;
+  return t;
+}
+
 template <int BN, bool SUMS>
 __device__ __forceinline__ int f32tc_items(const F32TcParams& p) {
   if constexpr (!SUMS) return p.nsplit * p.tiles_m2 * p.tiles_n;
-  const int n0 = (p.nv + 255) / 256 * ((p.N + BN - 1) / BN), n1 = (p.nw + 255) / 256 * ((p.M + BN - 1) / BN);
-  return p.nsplit * p.segs_per_split * (n0 + n1);
+  const F32TcSums t = f32tc_sums<BN>(p);
+  return p.nsplit * p.segs_per_split * (t.n[0] + t.n[1] + t.n[2]);
 }
 
 template <int BN, bool SUMS>
@@ -175,13 +192,14 @@ __device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
     t.k0 = t.z * p.k_per_split;
     t.klen = min(p.k_per_split, p.K - t.k0);
   } else {
-    const int c0 = (p.N + BN - 1) / BN, c1 = (p.M + BN - 1) / BN;
-    const int n0 = (p.nv + 255) / 256 * c0, n1 = (p.nw + 255) / 256 * c1;
-    t.seg = id / (n0 + n1);
-    int j = id - t.seg * (n0 + n1);
-    t.type = j >= n0;
-    if (t.type) j -= n0;
-    const int cols = t.type ? c1 : c0;
+    const F32TcSums u = f32tc_sums<BN>(p);
+    const int per = u.n[0] + u.n[1] + u.n[2];
+    t.seg = id / per;
+    int j = id - t.seg * per;
+    t.type = j < u.n[0] ? 0 : j < u.n[0] + u.n[1] ? 1 : 2;
+    if (t.type > 0) j -= u.n[0];
+    if (t.type > 1) j -= u.n[1];
+    const int cols = t.type == 1 ? u.cols[1] : u.cols[0];
     t.row0 = j / cols * 256;
     t.col0 = j % cols * BN;
     t.z = t.seg / p.segs_per_split;
@@ -240,8 +258,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     bool dead = false;
     for (int id = worker; id < items && !dead; id += workers) {
       const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
-      const CUtensorMap* mA = !SUMS ? &maps.A : (x.type ? &maps.W : &maps.V);
-      const bool kmajor_b = SUMS && x.type;
+      const CUtensorMap* mA = !SUMS || x.type == 2 ? &maps.A : (x.type ? &maps.W : &maps.V);
+      const bool kmajor_b = SUMS && x.type == 1;
       const int row = x.row0 + rank * 128, col = x.col0 + rank * (BN / 2);
       for (int k = 0; k < x.klen; k += KC, ++it) {
         const int s = it % S;
@@ -279,7 +297,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     bool dead = false;
     for (int id = worker; id < items && !dead; id += workers) {
       const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
-      const bool kmajor_b = SUMS && x.type;
+      const bool kmajor_b = SUMS && x.type == 1;
       const uint32_t id_t = kmajor_b ? idesc : idesc | (1u << 16);  // B MN-major
       for (int k = 0; k < x.klen; k += KC, ++it) {
         const int s = it % S, ab = it % NBUF;
@@ -705,10 +723,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       }
       if (dead) continue;
       if constexpr (SUMS) {
-        const int nu = x.type ? p.nw : p.nv;
-        const long long ld = x.type ? p.ldr_d : p.ldc_d;
-        float* out = (x.type ? p.Dr : p.Dc) + ((long long)x.seg * nu + row0) * ld + col0;
-        store(out, ld, nu - row0, (x.type ? p.M : p.N) - col0, 1.f, 0.f, true);
+        const int lines = x.type == 2 ? p.M : x.type ? p.nw : p.nv;
+        const long long ld = x.type == 2 ? p.ldp : x.type ? p.ldr_d : p.ldc_d;
+        float* out = (x.type == 2 ? p.P : x.type ? p.Dr : p.Dc) + ((long long)x.seg * lines + row0) * ld + col0;
+        store(out, ld, lines - row0, (x.type == 1 ? p.M : p.N) - col0, 1.f, 0.f, true);
       } else if (p.partial) {
         store(p.partial + ((long long)x.z * p.M + row0) * p.N + col0, p.N, p.M - row0, p.N - col0, 1.f, 0.f,
               (p.N & 1) == 0);
@@ -745,20 +763,21 @@ static cudaError_t f32tc_launch(const F32TcMaps& maps, const F32TcParams& p, int
   return cudaGetLastError();
 }
 
-// The checksum segments (ABFT only), then the product.  bn: columns per tile.
+// The segments (checksums; the product too if it goes by segments), then the
+// product in one pass or its scan.  bn: columns per tile.
 template <int BN>
 static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st) {
-  if (abft) {
-    // the tile's shared arrays hold units of GC rows and columns or more
-    if (p.um < F32TcCfg<BN>::GC || p.un < F32TcCfg<BN>::GC || p.um > 128 || p.un > 128) return cudaErrorInvalidValue;
-    const long long n0 = (long long)((p.nv + 255) / 256) * ((p.N + BN - 1) / BN);
-    const long long n1 = (long long)((p.nw + 255) / 256) * ((p.M + BN - 1) / BN);
-    const long long items = (n0 + n1) * p.nsplit * p.segs_per_split;
+  // the tile's shared arrays hold units of GC rows and columns or more
+  if (abft && (p.um < F32TcCfg<BN>::GC || p.un < F32TcCfg<BN>::GC || p.um > 128 || p.un > 128)) return cudaErrorInvalidValue;
+  if (abft || p.P) {
+    const F32TcSums t = f32tc_sums<BN>(p);
+    const long long items = ((long long)t.n[0] + t.n[1] + t.n[2]) * p.nsplit * p.segs_per_split;
     if (items > INT_MAX) return cudaErrorInvalidValue;
     cudaError_t e = f32tc_launch<BN, false, true>(maps, p, (int)items, sms, st);
     if (e != cudaSuccess) return e;
     ++*launches;
   }
+  if (p.P) return launch_f32tc_scan(abft, p, launches, st);
   const long long items = (long long)p.nsplit * p.tiles_m2 * p.tiles_n;
   if (items > INT_MAX) return cudaErrorInvalidValue;
   ++*launches;

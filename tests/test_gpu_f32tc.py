@@ -119,6 +119,32 @@ def test_splits_and_periods_bit_exact(ft, orc, K, split, period):
     assert rep.corrected == 3
 
 
+@pytest.mark.parametrize("shape", [(200, 130, 5000), (256, 256, 4099), (47, 300, 8192)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("name,level", [("wide32", "block"), ("wide", "warp"), ("large", "block"), ("tall", "block"),
+                                        ("tall", "warp"), ("medium", "block"), ("medium", "warp"), ("small", "block"),
+                                        ("wide", "off")])
+def test_long_k_by_segments_bit_exact(ft, orc, shape, name, level):
+    """Few tiles and a long K: the product by segments of K, then a scan that
+    verifies period by period."""
+    M, N, K = shape
+    s, lv, seed = _sched(name), LEVELS[level], 7600 + M
+    A, B, Cin = synth.integers((M, K), seed), synth.integers((K, N), seed + 1), synth.integers((M, N), seed + 2)
+    tm, tn, ks = -(-M // s["m_tb"]), -(-N // s["n_tb"]), -(-K // s["k_tb"])
+    faults = [(0, 0, 3, 5, 7, 512.0), (0, tn // 2, ks // 2, 2, 1, -256.0), (0, 0, ks // 3, 1, 2, 128.0, 1),
+              (tm // 2, 0, ks - 1, 3, 4, 64.0, 2), (0, 0, ks // 2, 0, 0, 32.0), (0, 0, ks // 2, 9, 9, 64.0)]
+    if level == "off":
+        C, rep = _run(ft, A, B, Cin, -2.0, 3.0, lv, s, None)
+        assert np.array_equal(C, -2 * (A.astype(np.int64) @ B.astype(np.int64)) + 3 * Cin.astype(np.int64))
+        return
+    C, rep = _run(ft, A, B, Cin, -2.0, 3.0, lv, s, faults)
+    res = _oracle(orc, A, B, Cin, -2.0, 3.0, lv, s, faults)
+    assert np.array_equal(C, res.C)
+    assert [_key(r) for r in rep.records] == [_key(r) for r in res.records]
+    for g, o in zip(rep.records, res.records):
+        assert (g["delta"], g["residual_r"], g["residual_c"]) == (o.delta, o.residual_r, o.residual_c)
+    assert rep.corrected >= 1 and rep.checksum_only >= 1
+
+
 def test_two_faults_in_a_unit_stay_uncorrectable(ft, orc):
     M, N, K = 400, 700, 800
     s = _sched("wide")
