@@ -214,12 +214,33 @@ def make_inject(faults):
 class Handle:
     """Owns an ftgemm handle bound to a device and a stream."""
 
+    def _report(self, capacity):
+        """A Report over `capacity` record slots.  The slots (64 bytes each,
+        262 KB at the default capacity) are kept for the next call; a call
+        made meanwhile by another thread gets slots of its own."""
+        try:
+            recs = self._slots.pop()
+        except IndexError:
+            recs = None
+        if recs is None or len(recs) != capacity:
+            recs = (FaultRecord * capacity)()
+        return Report(capacity=capacity, records=recs), recs
+
+    def _taken(self, rep, recs, records=_records):
+        """The PyReport of a filled Report; its slots go back."""
+        out = PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only, rep.n_records,
+                       bool(rep.overflow), records(rep, len(recs)))
+        if not self._slots:
+            self._slots.append(recs)
+        return out
+
     def __init__(self, device: int = 0, stream=None):
         import torch
         self.device = device
         with torch.cuda.device(device):
             s = _stream_ptr(stream)
         self._h = C.c_void_p()
+        self._slots = []
         _check(lib().ftgemm_create(C.byref(self._h), device, s))
 
     def close(self):
@@ -284,8 +305,7 @@ class Handle:
         spec = make_inject(inject) if inject else None
         rep, recs = None, None
         if report:
-            recs = (FaultRecord * capacity)()
-            rep = Report(capacity=capacity, records=recs)
+            rep, recs = self._report(capacity)
         st = lib().ftgemm_gemm(self._h, M, N, K, float(alpha), _ptr(A), A.stride(0), _ptr(B),
                                B.stride(0), float(beta), _ptr(C_out), C_out.stride(0), dtype,
                                level, C.byref(spec) if spec else None,
@@ -293,15 +313,12 @@ class Handle:
         _check(st)
         if not report:
             return None
-        return PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only,
-                        rep.n_records, bool(rep.overflow), _records(rep, capacity))
+        return self._taken(rep, recs)
 
     def report_fetch(self, capacity: int = 4096) -> PyReport:
-        recs = (FaultRecord * capacity)()
-        rep = Report(capacity=capacity, records=recs)
+        rep, recs = self._report(capacity)
         _check(lib().ftgemm_report_fetch(self._h, C.byref(rep)))
-        return PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only,
-                        rep.n_records, bool(rep.overflow), _records(rep, capacity))
+        return self._taken(rep, recs)
 
     def autotune(self, A, B, C_out, level=FT_BLOCK, reps: int = 3):
         """Time the candidate F32 schedules on these operands (C_out is
@@ -329,15 +346,13 @@ class Handle:
         arr = (C.POINTER(InjectSpec) * max_runs)(*[C.pointer(sp) if sp else C.POINTER(InjectSpec)()
                                                    for sp in specs[:max_runs]])
         runs = C.c_int32(0)
-        recs = (FaultRecord * capacity)()
-        rep = Report(capacity=capacity, records=recs)
+        rep, recs = self._report(capacity)
         st = lib().ftgemm_gemm_offline(self._h, M, N, K, float(alpha), _ptr(A), A.stride(0), _ptr(B),
                                        B.stride(0), float(beta), _ptr(C_out), C_out.stride(0), arr, max_runs,
                                        C.byref(runs), C.byref(rep))
         if st not in (OK, ERR_UNRECOVERED):
             _check(st)
-        return st, runs.value, PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only,
-                                        rep.n_records, bool(rep.overflow), _records(rep, capacity))
+        return st, runs.value, self._taken(rep, recs)
 
     def dgemm(self, A, B, C_out, alpha=1.0, beta=0.0, level=FT_BLOCK, cadence: int = 16, inject=None,
               report=True, capacity: int = 4096):
@@ -352,15 +367,13 @@ class Handle:
         spec = make_inject(inject) if inject else None
         rep, recs = None, None
         if report:
-            recs = (FaultRecord * capacity)()
-            rep = Report(capacity=capacity, records=recs)
+            rep, recs = self._report(capacity)
         _check(lib().ftgemm_dgemm(self._h, M, N, K, float(alpha), _ptr(A), A.stride(0), _ptr(B), B.stride(0),
                                   float(beta), _ptr(C_out), C_out.stride(0), level, int(cadence),
                                   C.byref(spec) if spec else None, C.byref(rep) if rep else None))
         if not report:
             return None
-        return PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only,
-                        rep.n_records, bool(rep.overflow), _records(rep, capacity))
+        return self._taken(rep, recs)
 
     def zgemm(self, A, B, C_out, alpha=1.0, beta=0.0, level=FT_BLOCK, cadence: int = 16, inject=None,
               report=True, capacity: int = 4096):
@@ -377,21 +390,21 @@ class Handle:
         be = (C.c_double * 2)(complex(beta).real, complex(beta).imag)
         rep, recs, im = None, None, None
         if report:
-            recs = (FaultRecord * capacity)()
-            rep = Report(capacity=capacity, records=recs)
+            rep, recs = self._report(capacity)
             im = (C.c_double * (3 * capacity))()
         _check(lib().ftgemm_zgemm(self._h, M, N, K, al, _ptr(A), A.stride(0), _ptr(B), B.stride(0), be,
                                   _ptr(C_out), C_out.stride(0), level, int(cadence),
                                   C.byref(spec) if spec else None, C.byref(rep) if rep else None, im))
         if not report:
             return None
-        rl = _records(rep, capacity)
-        for q, r in enumerate(rl):
-            r["delta"] = complex(r["delta"], im[3 * q])
-            r["residual_r"] = complex(r["residual_r"], im[3 * q + 1])
-            r["residual_c"] = complex(r["residual_c"], im[3 * q + 2])
-        return PyReport(rep.detected, rep.corrected, rep.uncorrectable, rep.checksum_only,
-                        rep.n_records, bool(rep.overflow), rl)
+        def complex_records(r, cap):
+            rl = _records(r, cap)
+            for q, d in enumerate(rl):
+                d["delta"] = complex(d["delta"], im[3 * q])
+                d["residual_r"] = complex(d["residual_r"], im[3 * q + 1])
+                d["residual_c"] = complex(d["residual_c"], im[3 * q + 2])
+            return rl
+        return self._taken(rep, recs, complex_records)
 
     def set_residual_sink(self, lam_needed=None, features=None):
         """Route every later TILE-level tensor-core call's and BLOCK-level

@@ -59,6 +59,7 @@ cudaError_t launch_tc_gemm(int dt, bool abft, bool pair, const TcBatch& b, const
 cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, unsigned int* amax_bits, float* scale,
                             int* launches, cudaStream_t st);
 cudaError_t launch_fault_bits(const Fault* f, int n, uint32_t* bits, size_t words, cudaStream_t st);
+cudaError_t launch_report_collect(DevReport* rep, const ftgemm_fault_record* recs, HostReport* out, cudaStream_t st);
 cudaError_t launch_wait_selftest(DevReport* rep, long long limit_cycles, cudaStream_t st);
 cudaError_t launch_nonfused_inject(const Fault* f, int nf, int ks_lo, int ks_hi, int tiles_n, float* acc,
                                    long long ldacc, float* Cc, long long ldcc, float* CrT, long long ldcr,
@@ -132,6 +133,9 @@ struct ftgemm_ctx {
   DevReport* rep = nullptr;
   ftgemm_fault_record* recs = nullptr;
   int rep_cap = 1 << 16;
+  HostReport* h_rep = nullptr;  // page-locked: where a fetch reads the report
+  bool rep_clean = true;        // nothing that may report was enqueued since the counters were last zero
+  bool rep_replayed = false;    // a captured call reports here whenever its graph is replayed: never clean
   // fault table
   Fault* d_faults = nullptr;
   Fault* h_faults = nullptr;  // pinned staging
@@ -427,9 +431,19 @@ static int drain_events(ftgemm_ctx* h) {
   return FTGEMM_OK;
 }
 
+// Zero the report before a call that returns it.
 static int clear_report(ftgemm_ctx* h) {
-  CK(cudaMemsetAsync(h->rep, 0, offsetof(DevReport, capacity), h->stream));
-  CK(cudaMemsetAsync(&h->rep->timeouts, 0, 2 * sizeof(int), h->stream));  // timeouts, bind_errors
+  if (!h->rep_clean || h->rep_replayed) CK(cudaMemsetAsync(h->rep, 0, offsetof(DevReport, capacity), h->stream));
+  h->rep_clean = false;  // the call's own kernels follow
+  return FTGEMM_OK;
+}
+
+// A call whose events stay in the report until it is fetched.
+static int keep_report(ftgemm_ctx* h) {
+  h->rep_clean = false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(h->stream, &cs));
+  if (cs != cudaStreamCaptureStatusNone) h->rep_replayed = true;
   return FTGEMM_OK;
 }
 extern "C" int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out);
@@ -578,8 +592,8 @@ static int tc_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alpha,
     if (rc) return rc;
   }
   tc_layout(P, dt, abft, h->ws);
-  if (report) {
-    int rc = clear_report(h);
+  {
+    int rc = report ? clear_report(h) : keep_report(h);
     if (rc) return rc;
   }
   int total[P_KINDS];
@@ -976,6 +990,7 @@ int ftgemm_grouped_gemm_dev(ftgemm_handle_t h, ftgemm_group_t g, int32_t count, 
   if (h->sink_lam && g->abft && g->total_tiles > h->sink_cap)
     FAIL(FTGEMM_ERR_ARG, "residual sink holds %lld tiles, the group has %d", (long long)h->sink_cap, g->total_tiles);
   CK(cudaSetDevice(h->device));
+  h->rep_clean = false;
   CK(launch_tc_bind(g->d_probs, g->d_maps, g->d_pos, problems, g->count, g->dt, h->rep, h->stream));
   h->launches += 1;
   return group_enqueue(h, g);
@@ -1014,6 +1029,8 @@ static int group_enqueue(ftgemm_ctx* h, ftgemm_group* g) {
   const int grid = g->pair ? 2 * g->ncta : g->ncta;  // the schedule was built for this many workers
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(h->stream, &cs));
+  h->rep_clean = false;  // its events stay in the report until it is fetched
+  if (cs != cudaStreamCaptureStatusNone) h->rep_replayed = true;
   const bool timed = h->timing && cs == cudaStreamCaptureStatusNone;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
   if (timed) {
@@ -1103,6 +1120,7 @@ int ftgemm_create(ftgemm_handle_t* handle, int device, void* cuda_stream) {
   cudaError_t e = cudaMalloc(&h->rep, sizeof(DevReport));
   if (e == cudaSuccess) e = cudaMalloc(&h->recs, sizeof(ftgemm_fault_record) * h->rep_cap);
   if (e == cudaSuccess) e = cudaMemcpy(h->rep, &r, sizeof(r), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaHostAlloc(&h->h_rep, sizeof(HostReport), cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->faults_free, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     ftgemm_destroy(h);  // releases whatever was allocated
@@ -1120,6 +1138,7 @@ int ftgemm_destroy(ftgemm_handle_t h) {
   if (h->rep) cudaFree(h->rep);
   if (h->recs) cudaFree(h->recs);
   if (h->zimag) cudaFree(h->zimag);
+  if (h->h_rep) cudaFreeHost(h->h_rep);
   if (h->d_faults) cudaFree(h->d_faults);
   if (h->h_faults) cudaFreeHost(h->h_faults);
   if (h->faults_free) cudaEventDestroy(h->faults_free);
@@ -1312,15 +1331,18 @@ int ftgemm_quantize(ftgemm_handle_t h, int64_t n, const float* x, void* y, ftgem
 int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out) {
   if (!h || !out) FAIL(FTGEMM_ERR_ARG, "ftgemm_report_fetch: NULL argument");
   CK(cudaSetDevice(h->device));
-  DevReport r;
-  CK(cudaMemcpyAsync(&r, h->rep, sizeof(r), cudaMemcpyDeviceToHost, h->stream));
+  CK(launch_report_collect(h->rep, h->recs, h->h_rep, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  h->rep_clean = true;
+  const DevReport r = h->h_rep->r;
   int n = std::min(r.n_records, h->rep_cap);
   std::vector<ftgemm_fault_record> v(n);
-  if (n > 0) {
+  if (n > HostReport::kRecords) {
     CK(cudaMemcpyAsync(v.data(), h->recs, sizeof(ftgemm_fault_record) * n, cudaMemcpyDeviceToHost,
                        h->stream));
     CK(cudaStreamSynchronize(h->stream));
+  } else if (n > 0) {
+    memcpy(v.data(), h->h_rep->recs, sizeof(ftgemm_fault_record) * n);
   }
   std::sort(v.begin(), v.end(), [](const ftgemm_fault_record& a, const ftgemm_fault_record& b) {
     if (a.problem != b.problem) return a.problem < b.problem;
@@ -1340,8 +1362,6 @@ int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out) {
   const int w = std::min(cap, n);
   if (w > 0 && out->records) memcpy(out->records, v.data(), sizeof(ftgemm_fault_record) * w);
   out->overflow = (r.n_records > cap || r.n_records > h->rep_cap) ? 1 : 0;
-  int rc = clear_report(h);
-  if (rc) return rc;
   if (r.timeouts > 0) FAIL(FTGEMM_ERR_TIMEOUT, "%d bounded device waits gave up", r.timeouts);
   if (r.bind_errors > 0)
     FAIL(FTGEMM_ERR_ARG, "%d device-array entries broke a rebinding rule; their problems were skipped",
@@ -1586,8 +1606,8 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     if (rc) return rc;
   }
 
-  if (report) {
-    int rc = clear_report(h);
+  {
+    int rc = report ? clear_report(h) : keep_report(h);
     if (rc) return rc;
   }
 
@@ -2028,8 +2048,8 @@ int ftgemm_gemm_nonfused(ftgemm_handle_t h, int64_t m, int64_t n, int64_t k, dou
     int rc = upload_faults(h, inject, unit, M, N, ksteps, tiles_m, tiles_n, FTGEMM_FT_BLOCK, &nf);
     if (rc) return rc;
   }
-  if (report) {
-    int rc = clear_report(h);
+  {
+    int rc = report ? clear_report(h) : keep_report(h);
     if (rc) return rc;
   }
   // workspace (its own buffer: the GEMM calls below use the handle's)
@@ -2185,8 +2205,8 @@ static int f64_gemm(ftgemm_ctx* h, bool cplx, int64_t m, int64_t n, int64_t k, c
     int rc = upload_faults(h, inject, unit, M, N, ksteps, tiles_m, tiles_n, level, &nf, cplx);
     if (rc) return rc;
   }
-  if (report) {
-    int rc = clear_report(h);
+  {
+    int rc = report ? clear_report(h) : keep_report(h);
     if (rc) return rc;
   }
   if (cplx && !h->zimag) CK(cudaMalloc(&h->zimag, sizeof(double) * 3 * (size_t)h->rep_cap));

@@ -26,12 +26,19 @@ struct Fault {
 struct DevReport {
   unsigned long long detected, corrected, uncorrectable, checksum_only;
   int n_records;
-  int capacity;
   int timeouts;     // bounded device waits that gave up
   int bind_errors;  // device-array entries that broke a rebinding rule (problem skipped)
+  int capacity;     // last: a clear covers what stands before it
 };
 
 static_assert(sizeof(ftgemm_fault_record) == 64, "record layout");
+
+// Page-locked host copy of a report: the header and its first records.
+struct HostReport {
+  static constexpr int kRecords = 64;
+  DevReport r;
+  alignas(16) ftgemm_fault_record recs[kRecords];
+};
 
 __device__ __forceinline__ void report_event(DevReport* rep, ftgemm_fault_record* recs,
                                              const ftgemm_fault_record& r) {
