@@ -59,7 +59,8 @@ cudaError_t launch_tc_gemm(int dt, bool abft, bool pair, const TcBatch& b, const
 cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, unsigned int* amax_bits, float* scale,
                             int* launches, cudaStream_t st);
 cudaError_t launch_fault_bits(const Fault* f, int n, uint32_t* bits, size_t words, cudaStream_t st);
-cudaError_t launch_report_collect(DevReport* rep, const ftgemm_fault_record* recs, HostReport* out, cudaStream_t st);
+cudaError_t launch_report_collect(DevReport* rep, const ftgemm_fault_record* recs, const int* flag, HostReport* out,
+                                  cudaStream_t st);
 cudaError_t launch_wait_selftest(DevReport* rep, long long limit_cycles, cudaStream_t st);
 cudaError_t launch_nonfused_inject(const Fault* f, int nf, int ks_lo, int ks_hi, int tiles_n, float* acc,
                                    long long ldacc, float* Cc, long long ldcc, float* CrT, long long ldcr,
@@ -447,6 +448,7 @@ static int keep_report(ftgemm_ctx* h) {
   return FTGEMM_OK;
 }
 extern "C" int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out);
+static int fetch_report(ftgemm_ctx* h, ftgemm_report* out, const int* flag, int* flag_out);
 
 // ---- tensor-core path: problem layout shared by ftgemm_gemm and groups ----
 
@@ -1330,10 +1332,19 @@ int ftgemm_quantize(ftgemm_handle_t h, int64_t n, const float* x, void* y, ftgem
 
 int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out) {
   if (!h || !out) FAIL(FTGEMM_ERR_ARG, "ftgemm_report_fetch: NULL argument");
+  return fetch_report(h, out, nullptr, nullptr);
+}
+
+}  // extern "C"
+
+// The events since the last clear, sorted, and (flag not null) a device flag
+// as it stands now; synchronises the stream.
+static int fetch_report(ftgemm_ctx* h, ftgemm_report* out, const int* flag, int* flag_out) {
   CK(cudaSetDevice(h->device));
-  CK(launch_report_collect(h->rep, h->recs, h->h_rep, h->stream));
+  CK(launch_report_collect(h->rep, h->recs, flag, h->h_rep, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   h->rep_clean = true;
+  if (flag_out) *flag_out = h->h_rep->flag;
   const DevReport r = h->h_rep->r;
   int n = std::min(r.n_records, h->rep_cap);
   std::vector<ftgemm_fault_record> v(n);
@@ -1368,6 +1379,8 @@ int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out) {
          r.bind_errors);
   return FTGEMM_OK;
 }
+
+extern "C" {
 
 int ftgemm_encode(ftgemm_handle_t h, int64_t m, int64_t n, int64_t k, const float* A, int64_t lda,
                   const float* B, int64_t ldb, int32_t m_u, int32_t n_u, float* V, float* W,
@@ -1681,6 +1694,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   }
   float* ws = h->ws;
   int launches = 0;
+  const int* gate = nullptr;  // the CUDA-core kernel runs only if this flag is set on the device
   const float* At = At_given ? At_given : ws + oAt;
   const float* Bk = b_ok ? Bf : ws + oBp;
   if (use_tc) {
@@ -1699,7 +1713,19 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     int rc = f32tc_run(h, tc, e, alpha, beta, C, ldc, al16(C), level, s, split, ks_per_split, cadence, ksteps, tiles_n,
                        nf, ws + oTc[6], ws + oTc[7], ws + oTc[9], split > 1 ? ws + oPart : nullptr, &launches);
     if (rc) return rc;
-    CK(launch_kmajor_operands_if(e.bad, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
+    gate = e.bad;
+    if (report && split == 1) {
+      // the report's wait tells whether the planes held every value; with a
+      // split the reduction is already behind it, so the gate decides there
+      int bad = 0;
+      h->launches += launches;
+      launches = 0;
+      rc = fetch_report(h, report, e.bad, &bad);
+      if (rc || !bad) return rc;
+      gate = nullptr;
+      h->rep_clean = false;
+    }
+    CK(launch_kmajor_operands_if(gate, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
                                  &launches, h->stream));
   } else {
     // A^T, with the A side of the encoding (block sums, row norms) in the same pass
@@ -1760,9 +1786,9 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   p.coB = (learned || sink) ? ws + oCo + tiles_m : nullptr;
   p.sink_lam = sink ? h->sink_lam : nullptr;
   p.sink_x = sink ? h->sink_x : nullptr;
-  p.only_if = use_tc ? (const int*)(ws + oTc[8]) : nullptr;
+  p.only_if = gate;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-  const bool timed = h->timing && !use_tc;  // the tensor-core kernels were timed themselves
+  const bool timed = h->timing && !gate;  // (the tensor-core kernels were timed themselves)
   if (timed) {
     int rc = take_events(h, &ev);
     if (rc) return rc;

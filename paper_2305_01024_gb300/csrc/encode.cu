@@ -340,7 +340,7 @@ cudaError_t launch_copy_pad(const float* X, long long ldx, int R, int Cn, float*
 }
 
 // The operand layout of the CUDA-core kernel, produced only if *gate is set
-// when the kernels run: A^T, and (Bp not null) B with padded rows.
+// when the kernels run (null: always): A^T, and (Bp not null) B with padded rows.
 cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long lda, int M, int K, float* At,
                                       long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
                                       int* launches, cudaStream_t st) {

@@ -37,6 +37,7 @@ static_assert(sizeof(ftgemm_fault_record) == 64, "record layout");
 struct HostReport {
   static constexpr int kRecords = 64;
   DevReport r;
+  int flag;  // a device flag read in the same go
   alignas(16) ftgemm_fault_record recs[kRecords];
 };
 
