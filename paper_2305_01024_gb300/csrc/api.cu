@@ -49,10 +49,11 @@ cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, lo
 bool f32tc_scan_units(int um, int un);
 cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]);
-int tc_nb_parts(int dt, long long K);
+int tc_nb_parts(int dt, long long K, int sub);
+int tc_enc_sub(int dt, long long K, long long tiles_n);
 cudaError_t launch_tc_bind(TcProblem* probs, TcProbMaps* maps, const int* pos, const ftgemm_problem* in, int count,
                            int dt, DevReport* rep, cudaStream_t st);
-cudaError_t launch_tc_prep(int dt, bool abft, const TcBatch& b, const int total[P_KINDS],
+cudaError_t launch_tc_prep(int dt, bool abft, bool sink, const TcBatch& b, const int total[P_KINDS],
                            const int* const* bmap, int* launches, cudaStream_t st);
 cudaError_t launch_tc_gemm(int dt, bool abft, bool pair, const TcBatch& b, const TcMapsBatch& mb, const TcRun& run, int grid,
                            cudaStream_t st);
@@ -480,6 +481,7 @@ static void tc_set_problem(TcProblem& P, int dt, bool abft, int M, int N, int K,
   P.nkb = (K + kblk - 1) / kblk;
   P.A = A; P.lda = lda; P.B = B; P.ldb = ldb;
   P.ldk = (K + 127) / 128 * 128;  // elements; a 16-byte multiple for both types
+  P.enc_sub = tc_enc_sub(dt, K, P.tiles_n);
   P.b_mn = tc_b_in_place(dt, abft, B, ldb);
   P.C = C; P.ldc = ldc;
   P.c_vec = (ldc % 4 == 0) && (((uintptr_t)C & 15) == 0);
@@ -500,20 +502,21 @@ static size_t tc_layout(TcProblem& P, int dt, bool abft, float* ws) {
     o = align64(o + floats);
     return ws ? ws + at : nullptr;
   };
-  P.Bt = P.b_mn ? nullptr : take(fl(eb * (size_t)P.N * P.ldk));
+  if (tc_packed_b(dt, abft)) P.Bt = take(fl(eb * tn * P.nkb * (TC_PACK_ROWS * 64)));
+  else P.Bt = P.b_mn ? nullptr : take(fl(eb * (size_t)P.N * P.ldk));
   if (abft) {
     P.Vf = take(tm * P.ldk);
     P.Wf = take(tn * P.ldk);
     P.Vt = take(fl(eb * tm * ns * P.ldk));
-    P.Wt = take(fl(eb * tn * ns * P.ldk));
-    P.vscale = take(tm * ns);
-    P.wscale = take(tn * ns);
-    P.s0v = take(tm);
-    P.s0w = take(tn);
+    if (dt == 1) {
+      P.Wt = take(fl(eb * tn * ns * P.ldk));
+      P.vscale = take(tm * ns);
+      P.wscale = take(tn * ns);
+    }
     P.nA = take(P.M);
     P.nB = take(P.N);
     P.nA_part = take((size_t)((K + 255) / 256) * P.M);
-    P.nB_part = take((size_t)tc_nb_parts(dt, K) * P.N);
+    P.nB_part = take((size_t)tc_nb_parts(dt, K, P.enc_sub) * P.N);
     P.froA = take(tm);
     P.froB = take(tn);
     P.coA = take(tm);
@@ -531,7 +534,10 @@ static int tc_make_maps(TcProbMaps& mp, const TcProblem& P, int dt, bool abft, b
   memset(&mp, 0, sizeof(mp));
   int rc = make_map_sw128(&mp.A, P.A, elem, P.K, P.M, P.lda, BK, am);
   if (!rc) {
-    if (P.b_mn) {
+    if (tc_packed_b(dt, abft)) {  // the tile's block of a k-block, or a CTA's half of it
+      rc = make_map_rows128(&mp.B, (const uint16_t*)P.Bt, (uint64_t)P.tiles_n * P.nkb * TC_PACK_ROWS,
+                            pair ? TC_PACK_ROWS / 2 : TC_PACK_ROWS);
+    } else if (P.b_mn) {
       rc = make_map_sw128(&mp.B, P.B, elem, P.N, P.K, P.ldb, 64, BK);  // 64-column boxes
     } else if (pair) {  // the two halves of a pair's 256-column MMA tile
       rc = make_map_sw128(&mp.B, P.Bt, elem, P.K, P.N, P.ldk, BK, 128);
@@ -540,11 +546,12 @@ static int tc_make_maps(TcProbMaps& mp, const TcProblem& P, int dt, bool abft, b
       rc = make_map_sw128(&mp.B, P.Bt, elem, P.K, P.N, P.ldk, BK, bn);
     }
   }
-  if (!rc && abft) rc = make_map_sw128(&mp.W, P.Wt, elem, P.K, (uint64_t)P.tiles_n * ns, P.ldk, BK, ns);
+  if (!rc && abft && dt == 1) rc = make_map_sw128(&mp.W, P.Wt, elem, P.K, (uint64_t)P.tiles_n * ns, P.ldk, BK, ns);
   if (!rc && abft) rc = make_map_sw128(&mp.V, P.Vt, elem, P.K, (uint64_t)P.tiles_m * ns, P.ldk, BK, ns);
   if (rc) return rc;
-  if (!abft) { mp.W = mp.A; mp.V = mp.A; }
-  if (!pair || P.b_mn) mp.B1 = mp.B;  // not used
+  if (!abft) mp.V = mp.A;
+  if (!abft || dt == 0) mp.W = mp.A;                                    // not used
+  if (!pair || P.b_mn || tc_packed_b(dt, abft)) mp.B1 = mp.B;           // not used
   return FTGEMM_OK;
 }
 
@@ -601,7 +608,7 @@ static int tc_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alpha,
   int total[P_KINDS];
   tc_prep_blocks(P, dt, total);
   int launches = 0;
-  CK(launch_tc_prep(dt, abft, b, total, nullptr, &launches, h->stream));
+  CK(launch_tc_prep(dt, abft, h->sink_lam != nullptr, b, total, nullptr, &launches, h->stream));
   TcMapsBatch mb;
   memset(&mb, 0, sizeof(mb));
   {
@@ -775,11 +782,15 @@ int ftgemm_group_create(ftgemm_handle_t h, int32_t count, const ftgemm_problem* 
   long long tiles = 0, blocks[P_KINDS] = {};
   size_t ws_floats = 0;
   std::vector<size_t> ws_at(count);
+  long long b_blocks = 0;  // of the B pass over the whole group, 4 k-blocks each
+  for (int i = 0; i < count; ++i)
+    b_blocks += ((pr[i].k + (dt == 0 ? 255 : 511)) / (dt == 0 ? 256 : 512)) * ((pr[i].n + tc_dn(dt, abft) - 1) / tc_dn(dt, abft));
   for (int q = 0; q < count; ++q) {
     const ftgemm_problem& u = pr[order[q]];
     TcProblem& P = g->probs[q];
     tc_set_problem(P, dt, abft, (int)u.m, (int)u.n, (int)u.k, u.A, u.lda, u.B, u.ldb, u.C, u.ldc, u.alpha, u.beta,
                    dt == 1 ? u.scale_a * u.scale_b : 1.f, lam_u, h->mu);
+    P.enc_sub = b_blocks >= 304 ? 4 : 1;
     P.id = order[q];
     P.mlp = h->mlp_on ? h->mlp_theta : nullptr;
     P.mlp_scale = h->mlp_scale;
@@ -1022,7 +1033,7 @@ static int group_enqueue(ftgemm_ctx* h, ftgemm_group* g) {
   b.nprob = g->count;
   b.total_tiles = g->total_tiles;
   int launches = 0;
-  CK(launch_tc_prep(g->dt, g->abft, b, g->total, g->bmap, &launches, h->stream));
+  CK(launch_tc_prep(g->dt, g->abft, h->sink_lam != nullptr, b, g->total, g->bmap, &launches, h->stream));
   TcMapsBatch mb;
   memset(&mb, 0, sizeof(mb));
   mb.table = g->d_maps;

@@ -149,7 +149,7 @@ constexpr int TC_GROUP_M = 16;  // tile rows per raster group
 
 // Batched encode launches of the tensor-core path; a problem's first block
 // in launch `kind` is TcProblem::blk_start[kind].
-enum TcPrepKind { P_ENC_A = 0, P_ENC_B, P_FIN, P_SCALE, P_PIECES, P_KINDS };
+enum TcPrepKind { P_ENC_A = 0, P_ENC_B, P_FIN, P_PIECES, P_KINDS };
 
 // One GEMM of the tensor-core path: operands, encode buffers, epilogue.
 // A table of these drives the encode launches and the persistent GEMM; a
@@ -160,14 +160,15 @@ struct TcProblem {
   int blk_start[P_KINDS];
   const void* A; long long lda;   // M x K, operand type, K contiguous
   const void* B; long long ldb;   // K x N, operand type, N contiguous
-  void* Bt; long long ldk;        // B^T (N x ldk); ldk also the row stride of Vt / Wt
+  void* Bt; long long ldk;        // B^T (N x ldk); ldk also the row stride of Vt / Wt.  bf16 with
+                                  // checksums: B packed by tiles instead (tc_packed_b)
+  int enc_sub;                    // k-blocks per block of the B pass
   int b_mn;                       // checksums off, bf16, B 16-byte aligned: the MMA reads B
                                   // in place as an MN-major operand (no B^T, no encode pass)
   float* Vf; float* Wf;           // fp32 e^T A [tiles_m][ldk], B e [tiles_n][ldk] (first K used)
   void* Vt; void* Wt;             // tails [tiles * TC_TAIL][ldk], operand type: a tile's last
                                   // data rows of A (of B^T), then its pieces
   float* vscale; float* wscale;   // [tiles * TC_TAIL] multiplier of piece p at p
-  float* s0v; float* s0w;         // [tiles] fp8 piece base scales
   float* nA; float* nB;           // [M] row 2-norms of A, [N] column 2-norms of B
   float* nA_part; float* nB_part; // squared-norm partials per k-chunk: [ceil(K/256)][M], [ceil(K/kc)][N]
   float* froA; float* froB;       // [tiles_m], [tiles_n] Frobenius norms of the blocks
@@ -183,6 +184,13 @@ struct TcProblem {
   int off;                        // 1: skipped (its last device-array rebinding broke a rule):
                                   // nothing of it is read or written
 };
+
+// With checksums a bf16 B is packed by tiles: [tiles_n][k-blocks][4 column
+// groups][64 k-rows][64 columns], the tile's data columns, then the pieces of
+// B e, then a zero column, every block the 128-byte swizzled image (the 16-byte
+// units of k-row k permuted by k % 8) of an MN-major operand.
+__host__ __device__ constexpr bool tc_packed_b(int dt, bool abft) { return dt == 0 && abft; }
+constexpr int TC_PACK_ROWS = 256;  // rows of 128 bytes per (tile, k-block)
 
 // Without checksums a bf16 B is read in place by the MMA (MN-major) when
 // TMA can address it: 256-column tiles keep its boxes on 128-byte lines.
@@ -268,6 +276,23 @@ __device__ __forceinline__ int tc_find_block(const TcBatch& b, int kind, int blk
     if (b.table[mid].blk_start[kind] <= blk) lo = mid; else hi = mid - 1;
   }
   return lo;
+}
+
+// Launch with programmatic stream serialisation: the kernel may be scheduled
+// while its predecessor drains, and waits for it itself (pdl_wait).
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, P(a)...);
 }
 
 }  // namespace ftg

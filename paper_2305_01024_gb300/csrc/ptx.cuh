@@ -94,6 +94,12 @@ __device__ __forceinline__ void tensormap_release() {
   asm volatile("fence.proxy.tensormap::generic.release.gpu;" ::: "memory");
 }
 
+// Programmatic dependent launch: wait until the grids this one depends on have
+// completed and their writes are visible (returns at once without such a
+// launch); let the grids that depend on this one be scheduled.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Barrier `id` over `n` threads that also ORs a predicate across them: every
 // participating thread gets the same result.
 __device__ __forceinline__ int bar_red_or(int id, int n, int pred) {

@@ -35,13 +35,14 @@
 // store -- so the epilogue of one tile overlaps the main loop of the next.
 // k-block = one 128-byte swizzle row (64 bf16 or 128 fp8 elements).
 //
-// B operand.  Without checksums, for bf16 with a 16-byte aligned B, the MMA
+// B operand.  bf16 with checksums: the encode pass packs B by tiles, the data
+// columns of a tile and its pieces of B e side by side, as the MN-major
+// swizzled image the MMA reads, so a stage's B is one contiguous load and no
+// tail box.  Without checksums, for bf16 with a 16-byte aligned B, the MMA
 // reads B where it lies, as an MN-major operand: four TMA boxes of 64
 // columns x 64 k-rows per stage, each k-row a whole 128-byte line of B (the
-// tiles are 256 columns wide), so no encode pass runs at all.  With
-// checksums the data tile is 252 (e4m3: 248) columns wide, its boxes would
-// start off the 128-byte lines of B, and the kernel reads B^T (written by
-// the encode pass) K-major instead, as for e4m3 and unaligned B.
+// tiles are 256 columns wide), so no encode pass runs at all.  e4m3 and an
+// unaligned bf16 B without checksums: B^T, written by the encode pass, K-major.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -252,6 +253,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
   if constexpr (PAIR) cluster_sync();
   tc_fence_after();
   const uint32_t tmem = T.tmem_base;
+  pdl_wait();  // the encode pass, and whatever a direct call follows
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer: main boxes of A and B^T, then their tails ----------
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
       const int row0 = tm * DM, col0 = x.tn * DN;
       const TcProblem& Px = tc_problem(b, x.pi);
       const bool mn = !ABFT && DT == 0 && Px.b_mn;
+      constexpr bool packed = tc_packed_b(DT, ABFT);
       const bool off = Px.off;  // skipped: the stages are released unloaded
       for (int kb = 0; kb < x.nkb; ++kb, ++it) {
         const int s = it % S;
@@ -301,7 +304,10 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
           const uint32_t cbar = mapa_rank(&T.full[s], 0);
           if (leader) mbar_arrive_expect_tx(&T.full[s], 2 * Cfg::STAGE_BYTES);
           tma_load_2d_pair(sA(s), &mp->A, cbar, kb * BK, row0);
-          if (mn) {
+          if constexpr (packed) {
+            // this CTA's half of the tile's columns: one contiguous piece
+            tma_load_2d_pair(sB(s), &mp->B, cbar, 0, (x.tn * x.nkb + kb) * TC_PACK_ROWS + rank * (TC_PACK_ROWS / 2));
+          } else if (mn) {
 #pragma unroll
             for (int g = 0; g < BN / 128; ++g)
               tma_load_2d_pair(sB(s) + g * Cfg::MN_BOX, &mp->B, cbar, col0 + 128 * rank + 64 * g, kb * BK);
@@ -310,13 +316,15 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
           }
           if constexpr (ABFT) {
             tma_load_2d_pair(sA(s) + TC_AROWS * 128, &mp->V, cbar, kb * BK, tm * CSR);
-            if (rank) tma_load_2d_pair(sB(s) + (TC_BROWS - 128) * 128, &mp->W, cbar, kb * BK, x.tn * CSR);
+            if (!packed && rank) tma_load_2d_pair(sB(s) + (TC_BROWS - 128) * 128, &mp->W, cbar, kb * BK, x.tn * CSR);
           }
         } else {
           // the same byte count either way: an MN-major B is 4 boxes of 8 KB
           mbar_arrive_expect_tx(&T.full[s], Cfg::STAGE_BYTES);
           tma_load_2d(sA(s), &mp->A, &T.full[s], kb * BK, row0);
-          if (mn) {
+          if constexpr (packed) {
+            tma_load_2d(sB(s), &mp->B, &T.full[s], 0, (x.tn * x.nkb + kb) * TC_PACK_ROWS);
+          } else if (mn) {
 #pragma unroll
             for (int g = 0; g < BN / 64; ++g)
               tma_load_2d(sB(s) + g * Cfg::MN_BOX, &mp->B, &T.full[s], col0 + 64 * g, kb * BK);
@@ -325,7 +333,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
           }
           if constexpr (ABFT) {
             tma_load_2d(sA(s) + TC_AROWS * 128, &mp->V, &T.full[s], kb * BK, tm * CSR);
-            tma_load_2d(sB(s) + TC_BROWS * 128, &mp->W, &T.full[s], kb * BK, x.tn * CSR);
+            if (!packed) tma_load_2d(sB(s) + TC_BROWS * 128, &mp->W, &T.full[s], kb * BK, x.tn * CSR);
           }
         }
         // look one tile ahead while this tile's loads are in flight
@@ -348,7 +356,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
     TcTile nx = n_my > 0 ? tc_my_tile<PAIR>(b, my0, 0) : TcTile{0, 0, 0, 0};
     for (; lt < n_my && !dead; ++lt) {
       const int nkb = nx.nkb;
-      const bool mn = !ABFT && DT == 0 && tc_problem(b, nx.pi).b_mn;
+      const bool mn = tc_packed_b(DT, ABFT) || (!ABFT && DT == 0 && tc_problem(b, nx.pi).b_mn);
       const uint32_t id_t = mn ? (idesc | TC_IDESC_B_MN) : idesc;
       const int ab = lt & 1;
       if (lt >= 2 && !mbar_wait(&T.acc_empty[ab], ((lt >> 1) - 1) & 1)) {
@@ -461,9 +469,9 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
           nB_c[h] = (c < DN && gc < pN) ? P.nB[gc] : 0.f;
         }
 #pragma unroll
-        for (int q = 0; q < Cfg::NPIECE; ++q) {
-          wsc[q] = P.wscale[(size_t)x.tn * CSR + q];
-          vsc[q] = P.vscale[(size_t)tm * CSR + q];
+        for (int q = 0; q < Cfg::NPIECE; ++q) {  // (the bf16 pieces are the value itself)
+          wsc[q] = DT == 0 ? 1.f : P.wscale[(size_t)x.tn * CSR + q];
+          vsc[q] = DT == 0 ? 1.f : P.vscale[(size_t)tm * CSR + q];
         }
         // ----- threshold of this tile -----
         // analytic: lambda * u times the norms plus the growth term
@@ -894,25 +902,22 @@ cudaError_t launch_tc_impl(const TcBatch& b, const TcMapsBatch& mb, const TcRun&
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<DT, ABFT, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  if constexpr (!PAIR) {
-    tc_gemm_kernel<DT, ABFT, false><<<grid, Cfg::THREADS, smem, st>>>(b, mb, run);
-    return cudaGetLastError();
-  } else {
-    // clusters of two CTAs (an SM pair each)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(Cfg::THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<DT, ABFT, true>, b, mb, run);
-  }
+  // the set-up overlaps the encode pass; pairs: clusters of two CTAs (an SM pair each)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(Cfg::THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = PAIR ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<DT, ABFT, PAIR>, b, mb, run);
 }
 
 // Persistent launch over b.total_tiles tiles with `grid` CTAs (<= one per SM;

@@ -45,7 +45,10 @@ __device__ __forceinline__ float ld_elem(const void* base, long long idx) {
 // blocks of launch `kind` start at blk_start[kind].  A group passes `bmap`,
 // the problem of every block of the launch (built once, at group creation);
 // otherwise the problem is found by binary search.
+// What the launch before left is waited for first.
 #define TC_BLOCK_OF(KIND)                                                  \
+  pdl_wait();                                                              \
+  pdl_trigger();                                                           \
   const int pi = bmap ? bmap[blockIdx.x] : tc_find_block(b, KIND, blockIdx.x); \
   const TcProblem& P = tc_problem(b, pi);                                  \
   if (P.off) return; /* skipped by a device-array rebinding: not read */   \
@@ -138,15 +141,37 @@ __device__ __forceinline__ void cvt8(const uint4 q, float* v) {
   }
 }
 
+// Three bf16 values whose sum is x to 24 bits.
+__device__ __forceinline__ void tc_pieces3(float x, uint16_t p[3]) {
+  const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(hi);
+  const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+  p[0] = __bfloat16_as_ushort(hi);
+  p[1] = __bfloat16_as_ushort(mid);
+  p[2] = __bfloat16_as_ushort(__float2bfloat16_rn(r1 - __bfloat162float(mid)));
+}
+
 // A: block sums over DM-row blocks (-> Vf), squared row-norm partials over
 // 256-wide k-chunks (-> nA_part), and the copy of each block's rows
 // TC_AROWS .. DM - 1 into the first rows of its tail in Vt (the MMA reads a
-// tile's first TC_AROWS rows from A and the rest from the tail), one pass.
-// Block = (row block, chunk); warp w takes rows w, w+8, ..., lane l the 8
-// columns 8l..8l+7 of the chunk.
+// tile's first TC_AROWS rows from A and the rest from the tail); for bf16 the
+// rest of the tail too: zeros for rows past M and the pieces of the sums.  One
+// pass.  Block = (row block, chunk); warp w takes rows w, w+8, ..., lane l the
+// 8 columns 8l..8l+7 of the chunk.
+// It runs beside the B pass before it: it depends on nothing that pass writes,
+// and waits for it at its end, so that whatever waits for this pass waits for
+// both.
 template <int DT>
 __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
-  TC_BLOCK_OF(P_ENC_A);
+  // the B pass lets this one start once it has itself waited for what came before
+  pdl_trigger();
+  const int pi = bmap ? bmap[blockIdx.x] : tc_find_block(b, P_ENC_A, blockIdx.x);
+  const TcProblem& P = tc_problem(b, pi);
+  if (P.off) {  // skipped by a device-array rebinding: not read
+    pdl_wait();
+    return;
+  }
+  const int lb = (int)blockIdx.x - P.blk_start[P_ENC_A];
   constexpr int DM = tc_dm(DT, true);
   __shared__ float part[8][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -229,20 +254,110 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += part[w][t];
     P.Vf[(long long)blk * P.ldk + k0 + t] = s;
+    if constexpr (DT == 0) {
+      static_assert(DM - TC_AROWS + 3 == TC_TAIL, "data rows and pieces fill the tail");
+      uint16_t pc[3];
+      tc_pieces3(s, pc);
+#pragma unroll
+      for (int c = 0; c < DM - TC_AROWS; ++c)
+        if (r0 + TC_AROWS + c >= P.M) tail[(long long)c * P.ldk + k0 + t] = 0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) tail[(long long)(DM - TC_AROWS + c) * P.ldk + k0 + t] = pc[c];
+    }
+  }
+  pdl_wait();  // the B pass
+}
+
+// bf16 B (K x N, N contiguous) packed by tiles (tc_packed_b), with the tile's
+// block sums (-> Wf), their pieces in the tile's columns DN .. DN + 2, and the
+// squared column-norm partials (-> nB_part, one per block).  Block = (tile
+// column, enc_sub k-blocks of 64); warp w takes k-rows w, w + 8, ..., lane l
+// the 8 columns 8l .. 8l + 7 of the tile (two 8-byte loads: DN is a multiple of
+// 4, so every tile starts on an 8-byte boundary of B's rows), which it writes
+// as one 16-byte unit: whole 128-byte lines both ways, no transpose.
+// Bound: HBM, 4 bytes an element.  (Through a shared-memory transpose to
+// K-major rows this pass ran at 3.7 TB/s at 8192^2, 73 us, bound by its
+// shared-memory loads.)
+__global__ void __launch_bounds__(256) tc_pack_b_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
+  TC_BLOCK_OF(P_ENC_B);
+  constexpr int KC = 64, DN = tc_dn(0, true);
+  __shared__ float sqw[8][256];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nkc = (P.K + KC - 1) / KC, nkg = (nkc + P.enc_sub - 1) / P.enc_sub;
+  const int kg = lb % nkg, nb = lb / nkg;
+  const int n0 = nb * DN, c0 = n0 + lane * 8, ncols = min(P.N, n0 + DN);
+  const bool vec_ok = ((uintptr_t)P.B % 8 == 0) && ((P.ldb * 2) % 8 == 0);
+  // vector loads, columns past the tile or N read as zeros, unless some lane's
+  // 8 columns straddle the end otherwise than at an 8-byte half
+  const bool fast = vec_ok && !__any_sync(0xffffffffu, c0 < ncols && c0 + 8 > ncols && c0 + 4 != ncols);
+  float sq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int sub = 0; sub < P.enc_sub; ++sub) {
+    const int kc = kg * P.enc_sub + sub;
+    if (kc >= nkc) break;  // block-uniform
+    const int k0 = kc * KC;
+    uint16_t* const out = reinterpret_cast<uint16_t*>(P.Bt) + ((long long)nb * nkc + kc) * (TC_PACK_ROWS * 64) +
+                          (lane >> 3) * (KC * 64);
+    uint4 q[8];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const int k = min(k0 + warp + 8 * g, P.K - 1);
+      if (fast) {
+        q[g] = ldraw8_a8_upto<0>(P.B, P.ldb, k, c0, ncols);
+      } else {
+        float v[8];
+        uint16_t raw[8];
+        ld8<0>(P.B, P.ldb, k, c0, ncols, false, v, raw);
+        q[g] = make_uint4((uint32_t)raw[0] | (uint32_t)raw[1] << 16, (uint32_t)raw[2] | (uint32_t)raw[3] << 16,
+                          (uint32_t)raw[4] | (uint32_t)raw[5] << 16, (uint32_t)raw[6] | (uint32_t)raw[7] << 16);
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const int kl = warp + 8 * g, k = k0 + kl;
+      uint4 w = k < P.K ? q[g] : make_uint4(0u, 0u, 0u, 0u);
+      float v[8];
+      cvt8<0>(w, v);
+      float rs = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        rs += v[e];
+        sq[e] = fmaf(v[e], v[e], sq[e]);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
+      if (lane == 31) {
+        static_assert(DN == 252, "lane 31: four data columns, three pieces, a zero");
+        uint16_t pc[3];
+        tc_pieces3(rs, pc);
+        w.z = (uint32_t)pc[0] | (uint32_t)pc[1] << 16;
+        w.w = (uint32_t)pc[2];
+      }
+      if (lane == 0 && k < P.K) P.Wf[(long long)nb * P.ldk + k] = rs;
+      *reinterpret_cast<uint4*>(out + kl * 64 + (((lane & 7) ^ (kl & 7)) << 3)) = w;
+    }
+  }
+  // each warp saw 1/8 of the block's k rows: sum the warps' column partials
+#pragma unroll
+  for (int e = 0; e < 8; ++e) sqw[warp][lane * 8 + e] = sq[e];
+  __syncthreads();
+  const int c = threadIdx.x;
+  if (c < DN && n0 + c < P.N) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s += sqw[w][c];
+    P.nB_part[(long long)kg * P.N + n0 + c] = s;
   }
 }
 
 // B (K x N, N contiguous): B^T (N x ldk, K contiguous) in KC x NBW tiles
-// through shared memory, TC_ENC_B_SUB consecutive tiles along K per block;
+// through shared memory, enc_sub consecutive tiles along K per block;
 // KC is one 128-byte k-block of the operand type.  With checksums a block
 // covers one DN-column data block of B (NBW = DN) and also writes its block
 // sums (-> Wf), the squared column-norm partials (-> nB_part, one per
-// TC_ENC_B_SUB * KC rows of K) and the copy of B^T's rows TC_BROWS .. DN - 1
+// enc_sub * KC rows of K) and the copy of B^T's rows TC_BROWS .. DN - 1
 // of the block into the first rows of its tail in Wt.  DN being a multiple
 // of 4, every block starts on an 8-byte boundary of B's rows: lane l reads
 // columns 8l .. 8l + 7 of a k-row as two 8-byte loads (bf16) or one (e4m3).
-constexpr int TC_ENC_B_SUB = 4;
-
 template <int DT, bool ABFT>
 __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
   TC_BLOCK_OF(P_ENC_B);
@@ -253,7 +368,7 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
   constexpr int PITCH = 256 + (DT == 0 ? 10 : 20);  // elements; staggers the banks (a lane may store 8 past NBW)
   __shared__ __align__(16) E tile[KC][PITCH];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nkc = (P.K + KC - 1) / KC, nkg = (nkc + TC_ENC_B_SUB - 1) / TC_ENC_B_SUB;
+  const int nkc = (P.K + KC - 1) / KC, nkg = (nkc + P.enc_sub - 1) / P.enc_sub;
   const int kg = lb % nkg, nb = lb / nkg;
   const int n0 = nb * NBW;
   const int lim = min(8, NBW - lane * 8);  // this lane's columns inside the block (8, 4 or <= 0)
@@ -281,8 +396,8 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
   };
   E* Bt = reinterpret_cast<E*>(P.Bt);
   constexpr int EPV = 16 / (int)sizeof(E);  // elements per 16-byte vector
-  for (int sub = 0; sub < TC_ENC_B_SUB; ++sub) {
-    const int kc = kg * TC_ENC_B_SUB + sub;
+  for (int sub = 0; sub < P.enc_sub; ++sub) {
+    const int kc = kg * P.enc_sub + sub;
     if (kc >= nkc) break;  // block-uniform
     const int k0 = kc * KC;
     if (fast) {
@@ -387,7 +502,7 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
 // coherence ||v_I||_2 / (sqrt(|I|) ||A_I||_F) of each block (the same for
 // w_J and B_J), a feature of the learned threshold.
 template <int DT>
-__global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
+__global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap, int sink) {
   TC_BLOCK_OF(P_FIN);
   __shared__ float red[8], red2[8];
   __shared__ float sred[8][256];
@@ -397,7 +512,7 @@ __global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ T
   const bool side_a = lb < P.tiles_m;
   const int blk = side_a ? lb : lb - P.tiles_m;
   const int R = side_a ? P.M : P.N, bs = side_a ? DM : DN;
-  const int nparts = side_a ? (P.K + 255) / 256 : (P.K + KC * TC_ENC_B_SUB - 1) / (KC * TC_ENC_B_SUB);
+  const int nparts = side_a ? (P.K + 255) / 256 : (P.K + KC * P.enc_sub - 1) / (KC * P.enc_sub);
   const float* part = side_a ? P.nA_part : P.nB_part;
   float* nrm = side_a ? P.nA : P.nB;
   const int t = threadIdx.x, r = blk * bs + t, warp = t >> 5, lane = t & 31;
@@ -424,8 +539,10 @@ __global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ T
   // squared norm of the checksum vector of this block over K
   const float* S = (side_a ? P.Vf : P.Wf) + (long long)blk * P.ldk;
   float c = 0.f;
+  if (P.mlp || sink) {  // (only the learned threshold and the sink use it)
 #pragma unroll 8
-  for (int k = t; k < P.K; k += blockDim.x) c = fmaf(S[k], S[k], c);
+    for (int k = t; k < P.K; k += blockDim.x) c = fmaf(S[k], S[k], c);
+  }
   float f = s;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -450,63 +567,50 @@ __global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ T
   }
 }
 
-// s0[blk]: power of two with max_k |S[blk][k]| * s0 in (224, 448]  (fp8 only)
-__global__ void tc_blockscale_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
-  TC_BLOCK_OF(P_SCALE);
-  __shared__ float red[32];
-  const bool side_a = lb < P.tiles_m;
-  const int blk = side_a ? lb : lb - P.tiles_m;
-  const float* S = (side_a ? P.Vf : P.Wf) + (long long)blk * P.ldk;
-  float m = 0.f;
-  for (int k = threadIdx.x; k < P.K; k += blockDim.x) m = fmaxf(m, fabsf(S[k]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = fmaxf(t, red[w]);
-    float sc = 1.f;
-    if (t > 0.f) {
-      int e;
-      frexpf(448.f / t, &e);  // 448/t in [2^(e-1), 2^e)
-      sc = ldexpf(1.f, e - 1);
-    }
-    (side_a ? P.s0v : P.s0w)[blk] = sc;
-  }
-}
-
-// Pieces of S[blk][k] into the block's tail rows in Pc (rows blk*TC_TAIL ..
-// + 7) and their multipliers scale[blk*TC_TAIL + p] (piece p; 0 past the
-// pieces in use); row blocks of A first, then column blocks of B.  A tail's
-// rows 0 .. TC_TAIL - NP - 1 are rows TC_AROWS.. of the block of A (written
-// by tc_encode_a), a B tail's rows 0 .. DN - TC_BROWS - 1 the same rows of
-// B^T (tc_encode_b); those past M (N) are zeroed here; the NP pieces follow,
-// then zeros.
-template <int DT>
-__global__ void tc_pieces_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
+// e4m3: pieces of S[blk][k] into the block's tail rows in Pc (rows blk*TC_TAIL
+// .. + 7) and their multipliers scale[blk*TC_TAIL + p] (piece p; 0 past the
+// pieces in use); row blocks of A first, then column blocks of B.  The pieces'
+// base scale s0 is the power of two with max_k |S[blk][k]| * s0 in (224, 448],
+// found by every block of the row (one read of S, from L2).  A tail's rows 0 ..
+// TC_TAIL - NP - 1 are rows TC_AROWS.. of the block of A (written by
+// tc_encode_a), a B tail's rows 0 .. DN - TC_BROWS - 1 the same rows of B^T
+// (tc_encode_b); those past M (N) are zeroed here; the NP pieces follow, then
+// zeros.
+__global__ void __launch_bounds__(256) tc_pieces_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
   TC_BLOCK_OF(P_PIECES);
-  constexpr int NS = TC_TAIL, KPT = 8;  // k per thread: one 16-byte (bf16) / 8-byte (fp8) store per slot
-  constexpr int NP = tc_npiece(DT), DM = tc_dm(DT, true), DN = tc_dn(DT, true);
+  constexpr int NS = TC_TAIL, KPT = 8;  // k per thread: one 8-byte store per slot
+  constexpr int NP = tc_npiece(1), DM = tc_dm(1, true), DN = tc_dn(1, true);
+  __shared__ float red[8];
   const int nkx = (P.K + 256 * KPT - 1) / (256 * KPT);
   const int k0 = (lb % nkx) * 256 * KPT + threadIdx.x * KPT, bi = lb / nkx;
   const bool side_a = bi < P.tiles_m;
   const int blk = side_a ? bi : bi - P.tiles_m;
-  const float* S = side_a ? P.Vf : P.Wf;
+  const float* S = (side_a ? P.Vf : P.Wf) + (long long)blk * P.ldk;
   void* Pc = side_a ? P.Vt : P.Wt;
-  float* scale = side_a ? P.vscale : P.wscale;
-  const float* s0 = side_a ? P.s0v : P.s0w;
+  float m = 0.f;
+#pragma unroll 8
+  for (int k = threadIdx.x; k < P.K; k += 256) m = fmaxf(m, fabsf(S[k]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w]);
+  float s0 = 1.f;
+  if (m > 0.f) {
+    int e;
+    frexpf(448.f / m, &e);  // 448/m in [2^(e-1), 2^e)
+    s0 = ldexpf(1.f, e - 1);
+  }
   if (lb % nkx == 0 && threadIdx.x < NS) {
     const int c = threadIdx.x;
-    float m = 0.f;
-    if (DT == 0) {
-      m = c < 3 ? 1.f : 0.f;
-    } else if (c < 5) {
-      m = s0[blk];
-      for (int q = 0; q < c; ++q) m *= 16.f;
-      m = 1.f / m;
+    float q = 0.f;
+    if (c < NP) {
+      q = s0;
+      for (int i = 0; i < c; ++i) q *= 16.f;
+      q = 1.f / q;
     }
-    scale[blk * NS + c] = m;
+    (side_a ? P.vscale : P.wscale)[blk * NS + c] = q;
   }
   if (k0 >= P.K) return;
   // slot of piece c, and whether slot c is left alone (a data row of A's
@@ -519,66 +623,39 @@ __global__ void tc_pieces_kernel(const __grid_constant__ TcBatch b, const int* _
                                : max(0, min(first, P.N - (blk * DN + TC_BROWS)));
   float x[KPT];
   {
-    const float4* src = reinterpret_cast<const float4*>(S + (long long)blk * P.ldk + k0);
+    const float4* src = reinterpret_cast<const float4*>(S + k0);
     const float4 u = src[0], v = src[1];
     const float t[KPT] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < KPT; ++j) x[j] = k0 + j < P.K ? t[j] : 0.f;
   }
-  if constexpr (DT == 0) {
-    uint16_t q[3][KPT];
+  __nv_fp8_storage_t* out = reinterpret_cast<__nv_fp8_storage_t*>(Pc);
+  uint32_t lo4[NP], hi4[NP];
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(x[j]);
-      const float r1 = x[j] - __bfloat162float(hi);
-      const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-      const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-      q[0][j] = __bfloat16_as_ushort(hi);
-      q[1][j] = __bfloat16_as_ushort(mid);
-      q[2][j] = __bfloat16_as_ushort(lo);
+  for (int c = 0; c < NP; ++c) { lo4[c] = 0u; hi4[c] = 0u; }
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    float sc = s0, r = x[j];
+#pragma unroll
+    for (int c = 0; c < NP; ++c) {
+      const __nv_fp8_storage_t qv = __nv_cvt_float_to_fp8(r * sc, __NV_SATFINITE, __NV_E4M3);
+      __nv_fp8_e4m3 qq;
+      qq.__x = qv;
+      r -= float(qq) / sc;
+      sc *= 16.f;
+      if (j < 4) lo4[c] |= (uint32_t)qv << (8 * j);
+      else hi4[c] |= (uint32_t)qv << (8 * (j - 4));
     }
-    uint16_t* out = reinterpret_cast<uint16_t*>(Pc);
+  }
 #pragma unroll
-    for (int c = 0; c < NS; ++c) {
-      if (c < live_rows) continue;
-      const int pc = c - first;  // piece in this slot
-      uint4 w = make_uint4(0u, 0u, 0u, 0u);
+  for (int c = 0; c < NS; ++c) {
+    if (c < live_rows) continue;
+    const int pc = c - first;
+    uint2 w = make_uint2(0u, 0u);
 #pragma unroll
-      for (int p = 0; p < NP; ++p)
-        if (p == pc)
-          w = make_uint4((uint32_t)q[p][0] | ((uint32_t)q[p][1] << 16), (uint32_t)q[p][2] | ((uint32_t)q[p][3] << 16),
-                         (uint32_t)q[p][4] | ((uint32_t)q[p][5] << 16), (uint32_t)q[p][6] | ((uint32_t)q[p][7] << 16));
-      *reinterpret_cast<uint4*>(out + (long long)(blk * NS + c) * P.ldk + k0) = w;
-    }
-  } else {
-    __nv_fp8_storage_t* out = reinterpret_cast<__nv_fp8_storage_t*>(Pc);
-    uint32_t lo4[NS], hi4[NS];
-#pragma unroll
-    for (int c = 0; c < NS; ++c) { lo4[c] = 0u; hi4[c] = 0u; }
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      float sc = s0[blk], r = x[j];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const __nv_fp8_storage_t qv = __nv_cvt_float_to_fp8(r * sc, __NV_SATFINITE, __NV_E4M3);
-        __nv_fp8_e4m3 qq;
-        qq.__x = qv;
-        r -= float(qq) / sc;
-        sc *= 16.f;
-        if (j < 4) lo4[c] |= (uint32_t)qv << (8 * j);
-        else hi4[c] |= (uint32_t)qv << (8 * (j - 4));
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < NS; ++c) {
-      if (c < live_rows) continue;
-      const int pc = c - first;
-      uint2 w = make_uint2(0u, 0u);
-#pragma unroll
-      for (int p = 0; p < NP; ++p)
-        if (p == pc) w = make_uint2(lo4[p], hi4[p]);
-      *reinterpret_cast<uint2*>(out + (long long)(blk * NS + c) * P.ldk + k0) = w;
-    }
+    for (int p = 0; p < NP; ++p)
+      if (p == pc) w = make_uint2(lo4[p], hi4[p]);
+    *reinterpret_cast<uint2*>(out + (long long)(blk * NS + c) * P.ldk + k0) = w;
   }
 }
 
@@ -609,52 +686,58 @@ __global__ void cast_e4m3_kernel(const float* __restrict__ x, long long n, const
 
 // ---------------------------------------------------------------------------
 
-// Column-norm partials of B per column: one per encode_b block along K.
-int tc_nb_parts(int dt, long long K) {
-  const long long kr = (dt == 0 ? 64 : 128) * TC_ENC_B_SUB;
+// k-blocks per block of the B pass: 4 (fewer partials), or 1 when the launch
+// would not fill the GPU (300 x 500 x 256: two blocks walking four k-blocks
+// each took 15 us).
+int tc_enc_sub(int dt, long long K, long long tiles_n) {
+  const long long nkc = (K + (dt == 0 ? 63 : 127)) / (dt == 0 ? 64 : 128);
+  return (nkc + 3) / 4 * tiles_n >= 304 ? 4 : 1;
+}
+
+// Column-norm partials of B per column: one per block of the B pass along K.
+int tc_nb_parts(int dt, long long K, int sub) {
+  const long long kr = (dt == 0 ? 64 : 128) * sub;
   return (int)((K + kr - 1) / kr);
 }
 
 // Blocks each batched encode launch gives one problem.
 // An MN-major B (checksums off) needs no encode blocks at all.
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]) {
-  const int nkx = (P.K + 255) / 256, kc = dt == 0 ? 64 : 128;
+  const int nkx = (P.K + 255) / 256;
   out[P_ENC_A] = nkx * P.tiles_m;
-  out[P_ENC_B] = P.b_mn ? 0 : ((P.K + kc * TC_ENC_B_SUB - 1) / (kc * TC_ENC_B_SUB)) * P.tiles_n;
+  out[P_ENC_B] = P.b_mn ? 0 : tc_nb_parts(dt, P.K, P.enc_sub) * P.tiles_n;
   out[P_FIN] = P.tiles_m + P.tiles_n;
-  out[P_SCALE] = P.tiles_m + P.tiles_n;
-  out[P_PIECES] = ((P.K + 2047) / 2048) * (P.tiles_m + P.tiles_n);  // 8 k per thread
+  out[P_PIECES] = dt == 0 ? 0 : ((P.K + 2047) / 2048) * (P.tiles_m + P.tiles_n);  // 8 k per thread
 }
 
-// The encode pass of a batch: B^T for every problem that needs it; with checksums also
-// the block sums, norms, Frobenius norms and pieces.  total[kind] = blocks
-// of each launch over the batch.
-// bmap: null, or per launch kind the problem of each of its blocks.
-cudaError_t launch_tc_prep(int dt, bool abft, const TcBatch& b, const int total[P_KINDS],
+// The encode pass of a batch: B^T (bf16 with checksums: the packed B) for
+// every problem that needs it; with checksums also the block sums, norms,
+// Frobenius norms and pieces.  total[kind] = blocks of each launch over the
+// batch.  bmap: null, or per launch kind the problem of each of its blocks.
+// sink: the tiles' coherences are wanted whether or not a network is set.
+// The launches overlap (pdl_wait): the A pass runs beside the B pass, the
+// others' start-up behind the one before.
+cudaError_t launch_tc_prep(int dt, bool abft, bool sink, const TcBatch& b, const int total[P_KINDS],
                            const int* const* bmap, int* launches, cudaStream_t st) {
   auto mp = [&](int kind) -> const int* { return bmap ? bmap[kind] : nullptr; };
   if (!abft) {
     if (total[P_ENC_B] == 0) return cudaSuccess;  // every B is read in place
-    if (dt == 0) tc_encode_b_kernel<0, false><<<total[P_ENC_B], 256, 0, st>>>(b, mp(P_ENC_B));
-    else tc_encode_b_kernel<1, false><<<total[P_ENC_B], 256, 0, st>>>(b, mp(P_ENC_B));
     ++*launches;
-    return cudaGetLastError();
+    return launch_pdl(dt == 0 ? tc_encode_b_kernel<0, false> : tc_encode_b_kernel<1, false>, total[P_ENC_B], 256, 0, st,
+                      b, mp(P_ENC_B));
   }
-  if (dt == 0) {
-    tc_encode_b_kernel<0, true><<<total[P_ENC_B], 256, 0, st>>>(b, mp(P_ENC_B));
-    tc_encode_a_kernel<0><<<total[P_ENC_A], 256, 0, st>>>(b, mp(P_ENC_A));
-    tc_norms_kernel<0><<<total[P_FIN], 256, 0, st>>>(b, mp(P_FIN));
-  } else {
-    tc_encode_b_kernel<1, true><<<total[P_ENC_B], 256, 0, st>>>(b, mp(P_ENC_B));
-    tc_encode_a_kernel<1><<<total[P_ENC_A], 256, 0, st>>>(b, mp(P_ENC_A));
-    tc_norms_kernel<1><<<total[P_FIN], 256, 0, st>>>(b, mp(P_FIN));
-    tc_blockscale_kernel<<<total[P_SCALE], 256, 0, st>>>(b, mp(P_SCALE));
+  cudaError_t e = launch_pdl(dt == 0 ? tc_pack_b_kernel : tc_encode_b_kernel<1, true>, total[P_ENC_B], 256, 0, st, b,
+                             mp(P_ENC_B));
+  if (e == cudaSuccess)
+    e = launch_pdl(dt == 0 ? tc_encode_a_kernel<0> : tc_encode_a_kernel<1>, total[P_ENC_A], 256, 0, st, b, mp(P_ENC_A));
+  if (e == cudaSuccess)
+    e = launch_pdl(dt == 0 ? tc_norms_kernel<0> : tc_norms_kernel<1>, total[P_FIN], 256, 0, st, b, mp(P_FIN), (int)sink);
+  *launches += 3;
+  if (e == cudaSuccess && dt == 1) {
+    e = launch_pdl(tc_pieces_kernel, total[P_PIECES], 256, 0, st, b, mp(P_PIECES));
     ++*launches;
   }
-  if (dt == 0) tc_pieces_kernel<0><<<total[P_PIECES], 256, 0, st>>>(b, mp(P_PIECES));
-  else tc_pieces_kernel<1><<<total[P_PIECES], 256, 0, st>>>(b, mp(P_PIECES));
-  *launches += 4;
-  return cudaGetLastError();
+  return e;
 }
 
 // Rebinding of a group to a device array of problems (ftgemm_grouped_gemm_dev),
