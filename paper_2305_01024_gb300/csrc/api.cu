@@ -57,7 +57,8 @@ cudaError_t launch_tc_prep(int dt, bool abft, bool sink, const TcBatch& b, const
                            const int* const* bmap, int* launches, cudaStream_t st);
 cudaError_t launch_tc_gemm(int dt, bool abft, bool pair, const TcBatch& b, const TcMapsBatch& mb, const TcRun& run, int grid,
                            cudaStream_t st);
-cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, unsigned int* amax_bits, float* scale,
+int tc_quant_scratch();
+cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, float* part, float* scale_host,
                             int* launches, cudaStream_t st);
 cudaError_t launch_fault_bits(const Fault* f, int n, uint32_t* bits, size_t words, cudaStream_t st);
 cudaError_t launch_report_collect(DevReport* rep, const ftgemm_fault_record* recs, const int* flag, HostReport* out,
@@ -155,7 +156,7 @@ struct ftgemm_ctx {
   // checksum-growth term of the analytic threshold, mu * u * sqrt(k) * |c|
   double mu = kMu;
   float fp8_sa = 1.f, fp8_sb = 1.f;
-  float* qscratch = nullptr;  // amax bits + scale of ftgemm_quantize
+  float* qscratch = nullptr;  // block maxima of ftgemm_quantize
   // learned threshold (tensor-core path)
   float* mlp_theta = nullptr;  // device, FTGEMM_MLP_PARAMS floats
   bool mlp_on = false;
@@ -1325,17 +1326,17 @@ int ftgemm_quantize(ftgemm_handle_t h, int64_t n, const float* x, void* y, ftgem
   if (!h || !x || !y || n <= 0) FAIL(FTGEMM_ERR_ARG, "ftgemm_quantize: bad argument");
   if (dtype != FTGEMM_BF16 && dtype != FTGEMM_E4M3) FAIL(FTGEMM_ERR_UNSUPPORTED, "ftgemm_quantize: dtype %d", (int)dtype);
   CK(cudaSetDevice(h->device));
-  if (!h->qscratch) CK(cudaMalloc(&h->qscratch, 2 * sizeof(float)));
+  if (!h->qscratch && dtype == FTGEMM_E4M3) CK(cudaMalloc(&h->qscratch, sizeof(float) * tc_quant_scratch()));
   int launches = 0;
-  CK(launch_quantize(dtype == FTGEMM_BF16 ? 0 : 1, x, n, y, reinterpret_cast<unsigned int*>(h->qscratch),
-                     h->qscratch + 1, &launches, h->stream));
+  CK(launch_quantize(dtype == FTGEMM_BF16 ? 0 : 1, x, n, y, h->qscratch, scale_out ? &h->h_rep->scale : nullptr,
+                     &launches, h->stream));
   h->launches += launches;
   if (scale_out) {
     if (dtype == FTGEMM_BF16) {
       *scale_out = 1.f;
     } else {
-      CK(cudaMemcpyAsync(scale_out, h->qscratch + 1, sizeof(float), cudaMemcpyDeviceToHost, h->stream));
       CK(cudaStreamSynchronize(h->stream));
+      *scale_out = h->h_rep->scale;
     }
   }
   return FTGEMM_OK;

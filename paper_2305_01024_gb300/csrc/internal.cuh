@@ -37,7 +37,8 @@ static_assert(sizeof(ftgemm_fault_record) == 64, "record layout");
 struct HostReport {
   static constexpr int kRecords = 64;
   DevReport r;
-  int flag;  // a device flag read in the same go
+  int flag;     // a device flag read in the same go
+  float scale;  // the scale ftgemm_quantize hands back
   alignas(16) ftgemm_fault_record recs[kRecords];
 };
 

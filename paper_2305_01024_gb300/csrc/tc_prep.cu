@@ -365,8 +365,14 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
   constexpr int KC = 128 / (int)sizeof(E);
   constexpr int NBW = ABFT ? tc_dn(DT, true) : TC_BN;
   static_assert(NBW % 4 == 0 && NBW > 31 * 8 - 8 && NBW <= 256, "block columns: 8-byte aligned, 31 or 32 lanes");
-  constexpr int PITCH = 256 + (DT == 0 ? 10 : 20);  // elements; staggers the banks (a lane may store 8 past NBW)
+  // bf16: the pitch staggers the banks (a lane may store 8 past NBW).  e4m3:
+  // 64 words a k-row, word c of row kk at c ^ 4 (kk / 16 % 8), so that both the
+  // rows' 8-byte stores and the 4 words x 8 row groups of a warp's reads hit
+  // distinct banks; the reads are words, turned by byte permutes (one byte at a
+  // time this pass took 62 us for 8192 x 4096).
+  constexpr int PITCH = DT == 0 ? 256 + 10 : 256;  // elements
   __shared__ __align__(16) E tile[KC][PITCH];
+  auto word_at = [](int kk, int c) { return c ^ (((kk >> 4) & 7) << 2); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkc = (P.K + KC - 1) / KC, nkg = (nkc + P.enc_sub - 1) / P.enc_sub;
   const int kg = lb % nkg, nb = lb / nkg;
@@ -420,12 +426,14 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
           if (in_cols) {
             // row pitch and column offset are multiples of 4 bytes; a lane
             // past the block's last column writes inside the padded row
-            uint32_t* t = reinterpret_cast<uint32_t*>(&tile[kk][lane * 8]);
-            t[0] = w.x;
-            t[1] = w.y;
             if constexpr (DT == 0) {
+              uint32_t* t = reinterpret_cast<uint32_t*>(&tile[kk][lane * 8]);
+              t[0] = w.x;
+              t[1] = w.y;
               t[2] = w.z;
               t[3] = w.w;
+            } else {
+              *reinterpret_cast<uint2*>(&tile[kk][4 * word_at(kk, lane * 2)]) = make_uint2(w.x, w.y);
             }
           }
           float v[8];
@@ -444,7 +452,8 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
         if (k < P.K && in_cols) ld8<DT>(P.B, P.ldb, k, n0 + lane * 8, ncols, false, v, raw);
         if (in_cols) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) tile[kk][lane * 8 + e] = (E)raw[e];
+          for (int e = 0; e < 8; ++e)
+            tile[kk][DT == 0 ? lane * 8 + e : 4 * word_at(kk, lane * 2 + (e >> 2)) + (e & 3)] = (E)raw[e];
         }
         take(v, k);
       }
@@ -453,29 +462,50 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
     // B^T rows n0..n0+NBW-1, k0..k0+KC-1: 8 threads write one 128-byte row
     // segment (the k-range past K is zero, inside the padded row); with
     // checksums the block's rows TC_BROWS.. also go to its tail
-    for (int i = threadIdx.x; i < NBW * 8; i += 256) {
-      const int nn = i >> 3, vq = i & 7;
-      const int n = n0 + nn;
-      if (n >= P.N) continue;
-      E o[EPV];
+    if constexpr (DT == 0) {
+      for (int i = threadIdx.x; i < NBW * 8; i += 256) {
+        const int nn = i >> 3, vq = i & 7;
+        const int n = n0 + nn;
+        if (n >= P.N) continue;
+        E o[EPV];
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) o[e] = tile[vq * EPV + e][nn];
-      uint4 w;
-      if constexpr (DT == 0) {
+        for (int e = 0; e < EPV; ++e) o[e] = tile[vq * EPV + e][nn];
+        uint4 w;
         w.x = (uint32_t)o[0] | ((uint32_t)o[1] << 16); w.y = (uint32_t)o[2] | ((uint32_t)o[3] << 16);
         w.z = (uint32_t)o[4] | ((uint32_t)o[5] << 16); w.w = (uint32_t)o[6] | ((uint32_t)o[7] << 16);
-      } else {
-        uint32_t q[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          q[j] = (uint32_t)o[4 * j] | ((uint32_t)o[4 * j + 1] << 8) | ((uint32_t)o[4 * j + 2] << 16) |
-                 ((uint32_t)o[4 * j + 3] << 24);
-        w = make_uint4(q[0], q[1], q[2], q[3]);
+        *reinterpret_cast<uint4*>(Bt + (long long)n * P.ldk + k0 + vq * EPV) = w;
       }
-      *reinterpret_cast<uint4*>(Bt + (long long)n * P.ldk + k0 + vq * EPV) = w;
-      if (ABFT && nn >= TC_BROWS)
-        *reinterpret_cast<uint4*>(reinterpret_cast<E*>(P.Wt) + ((long long)nb * TC_TAIL + nn - TC_BROWS) * P.ldk + k0 +
-                                  vq * EPV) = w;
+    } else {
+      // thread: 16 k-rows (vq) of one word of columns (c), four rows of B^T
+      for (int i = threadIdx.x; i < (NBW / 4) * 8; i += 256) {
+        const int vq = i & 7, c = i >> 3, n = n0 + 4 * c;
+        if (n >= P.N) continue;
+        uint32_t r[4][4];  // [row of B^T][4 k each]
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int kk = vq * 16 + g * 4 + e;
+            w[e] = reinterpret_cast<const uint32_t*>(&tile[kk][0])[word_at(kk, c)];
+          }
+          const uint32_t a0 = __byte_perm(w[0], w[1], 0x5140), a1 = __byte_perm(w[0], w[1], 0x7362);
+          const uint32_t b0 = __byte_perm(w[2], w[3], 0x5140), b1 = __byte_perm(w[2], w[3], 0x7362);
+          r[0][g] = __byte_perm(a0, b0, 0x5410);
+          r[1][g] = __byte_perm(a0, b0, 0x7632);
+          r[2][g] = __byte_perm(a1, b1, 0x5410);
+          r[3][g] = __byte_perm(a1, b1, 0x7632);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (n + j >= P.N) break;
+          const uint4 w = make_uint4(r[j][0], r[j][1], r[j][2], r[j][3]);
+          *reinterpret_cast<uint4*>(Bt + (long long)(n + j) * P.ldk + k0 + vq * EPV) = w;
+          if (ABFT && 4 * c + j >= TC_BROWS)
+            *reinterpret_cast<uint4*>(reinterpret_cast<E*>(P.Wt) + ((long long)nb * TC_TAIL + 4 * c + j - TC_BROWS) * P.ldk +
+                                      k0 + vq * EPV) = w;
+        }
+      }
     }
     __syncthreads();  // the tile is refilled by the next chunk
   }
@@ -661,27 +691,94 @@ __global__ void __launch_bounds__(256) tc_pieces_kernel(const __grid_constant__ 
 
 // ---- quantizer ------------------------------------------------------------
 
-__global__ void amax_kernel(const float* __restrict__ x, long long n, unsigned int* __restrict__ amax_bits) {
-  float m = 0.f;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    m = fmaxf(m, fabsf(x[i]));
+// Bound: HBM; both kernels read four float4 per thread and round (one float
+// at a time 4096 x 8192 values took 33 us + 57 us).
+constexpr int kQuantBlocks = 152 * 8;  // most blocks: as many block maxima
+
+// f(i, x[i .. i + 3]) over all whole groups of four, f1(i, x[i]) over the rest.
+template <class F, class F1>
+__device__ __forceinline__ void for_each4(const float* __restrict__ x, long long n, F f, F1 f1) {
+  const long long stride = (long long)gridDim.x * blockDim.x, t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long n4 = ((uintptr_t)x & 15) == 0 ? n / 4 : 0;
+  const float4* x4 = reinterpret_cast<const float4*>(x);
+  long long i = t;
+  for (; i + 3 * stride < n4; i += 4 * stride) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __ldg(x4 + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) f(4 * (i + u * stride), v[u]);
+  }
+  for (; i < n4; i += stride) f(4 * i, __ldg(x4 + i));
+  for (i = 4 * n4 + t; i < n; i += stride) f1(i, x[i]);
+}
+
+// Largest of a value over the block (256 threads), in every thread.
+__device__ __forceinline__ float block_max(float m) {
+  __shared__ float red[8];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax_bits, __float_as_uint(m));  // |x| >= 0: bits order as values
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w]);
+  return m;
 }
 
-__global__ void cast_bf16_kernel(const float* __restrict__ x, long long n, __nv_bfloat16* __restrict__ y) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16_rn(x[i]);
+// part[block] = the largest |x| of the block's share
+__global__ void __launch_bounds__(256) amax_kernel(const float* __restrict__ x, long long n, float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
+  float m = 0.f;
+  for_each4(
+      x, n,
+      [&](long long, float4 v) { m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); },
+      [&](long long, float v) { m = fmaxf(m, fabsf(v)); });
+  m = block_max(m);
+  if (threadIdx.x == 0) part[blockIdx.x] = m;
 }
 
-__global__ void cast_e4m3_kernel(const float* __restrict__ x, long long n, const unsigned int* __restrict__ amax_bits,
-                                 __nv_fp8_storage_t* __restrict__ y, float* __restrict__ scale_out) {
-  const float amax = __uint_as_float(*amax_bits);
+__global__ void __launch_bounds__(256) cast_bf16_kernel(const float* __restrict__ x, long long n, __nv_bfloat16* __restrict__ y) {
+  const bool vec = ((uintptr_t)y & 7) == 0;
+  for_each4(
+      x, n,
+      [&](long long i, float4 v) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), c = __floats2bfloat162_rn(v.z, v.w);
+        if (vec) {
+          *reinterpret_cast<uint2*>(y + i) =
+              make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&c));
+        } else {
+          y[i] = a.x; y[i + 1] = a.y; y[i + 2] = c.x; y[i + 3] = c.y;
+        }
+      },
+      [&](long long i, float v) { y[i] = __float2bfloat16_rn(v); });
+}
+
+// The scale also goes to scale_host (page-locked host memory) if given.
+__global__ void __launch_bounds__(256) cast_e4m3_kernel(const float* __restrict__ x, long long n,
+                                                        const float* __restrict__ part, int parts,
+                                                        __nv_fp8_storage_t* __restrict__ y, float* scale_host) {
+  pdl_wait();
+  float m = 0.f;
+  for (int i = threadIdx.x; i < parts; i += 256) m = fmaxf(m, part[i]);
+  const float amax = block_max(m);
   const float scale = amax > 0.f ? amax / 448.f : 1.f;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = scale;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = __nv_cvt_float_to_fp8(x[i] / scale, __NV_SATFINITE, __NV_E4M3);
+  if (scale_host && blockIdx.x == 0 && threadIdx.x == 0) *scale_host = scale;
+  const bool vec = ((uintptr_t)y & 3) == 0;
+  for_each4(
+      x, n,
+      [&](long long i, float4 v) {
+        const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v.x / scale, v.y / scale), __NV_SATFINITE, __NV_E4M3);
+        const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(v.z / scale, v.w / scale), __NV_SATFINITE, __NV_E4M3);
+        const uint32_t w = lo | hi << 16;
+        if (vec) {
+          *reinterpret_cast<uint32_t*>(y + i) = w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[i + e] = (__nv_fp8_storage_t)(w >> (8 * e));
+        }
+      },
+      [&](long long i, float v) { y[i] = __nv_cvt_float_to_fp8(v / scale, __NV_SATFINITE, __NV_E4M3); });
 }
 
 // ---------------------------------------------------------------------------
@@ -794,20 +891,21 @@ cudaError_t launch_fault_bits(const Fault* f, int n, uint32_t* bits, size_t word
   return cudaGetLastError();
 }
 
-cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, unsigned int* amax_bits, float* scale,
+// part: tc_quant_scratch() floats of scratch (e4m3).
+int tc_quant_scratch() { return kQuantBlocks; }
+cudaError_t launch_quantize(int dt, const float* x, long long n, void* y, float* part, float* scale_host,
                             int* launches, cudaStream_t st) {
-  const int grid = (int)std::min<long long>((n + 255) / 256, 152 * 8);
+  const int grid = (int)std::max<long long>(1, std::min<long long>((n + 4095) / 4096, kQuantBlocks));
   if (dt == 0) {
     cast_bf16_kernel<<<grid, 256, 0, st>>>(x, n, (__nv_bfloat16*)y);
     ++*launches;
     return cudaGetLastError();
   }
-  cudaError_t e = cudaMemsetAsync(amax_bits, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  amax_kernel<<<grid, 256, 0, st>>>(x, n, amax_bits);
-  cast_e4m3_kernel<<<grid, 256, 0, st>>>(x, n, amax_bits, (__nv_fp8_storage_t*)y, scale);
+  cudaError_t e = launch_pdl(amax_kernel, grid, 256, 0, st, x, n, part);
+  if (e == cudaSuccess)
+    e = launch_pdl(cast_e4m3_kernel, grid, 256, 0, st, x, n, part, grid, (__nv_fp8_storage_t*)y, scale_host);
   *launches += 2;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace ftg
