@@ -41,7 +41,11 @@ cudaError_t launch_encode_kmajor(const float*, long long, int, int, int, float*,
                                  float*, int*, cudaStream_t);
 cudaError_t launch_splitk_reduce(const float*, int, int, int, float, float, float*, long long,
                                  cudaStream_t);
-cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long lda, int M, int K, float* At,
+bool encode_small_fits(int M, int N, int K, int m_u, int n_u);
+cudaError_t launch_encode_small(const float* A, long long lda, int M, int K, float* At, long long ldt, int m_u, float* V,
+                                long long ldv, float* nA, const float* B, long long ldb, int N, int n_u, float* Bp,
+                                long long ldbp, float* W, float* nB, int* launches, cudaStream_t st);
+cudaError_t launch_kmajor_operands_if(const int* gate, int epoch, const float* A, long long lda, int M, int K, float* At,
                                       long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
                                       int* launches, cudaStream_t st);
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
@@ -137,6 +141,7 @@ struct ftgemm_ctx {
   ftgemm_fault_record* recs = nullptr;
   int rep_cap = 1 << 16;
   HostReport* h_rep = nullptr;  // page-locked: where a fetch reads the report
+  int epoch = 0;                // number of the fp32 tensor-core call (never 0 in one)
   bool rep_clean = true;        // nothing that may report was enqueued since the counters were last zero
   bool rep_replayed = false;    // a captured call reports here whenever its graph is replayed: never clean
   // fault table
@@ -1581,7 +1586,7 @@ static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, doub
   p.partial = partial;
   p.faults = nf > 0 ? h->d_faults : nullptr; p.nfaults = nf;
   p.rep = h->rep; p.recs = h->recs;
-  p.bad = e.bad;
+  p.bad = e.bad; p.epoch = e.epoch;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
   if (h->timing) {
     rc = take_events(h, &ev);
@@ -1721,6 +1726,8 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     e.pa = ws + oTc[2]; e.pb = ws + oTc[3];
     e.nA = ws + oNa; e.nB = ws + oNb; e.sq16a = ws + oTc[4]; e.sq16b = ws + oTc[5];
     e.bad = (int*)(ws + oTc[8]);
+    h->epoch = h->epoch % 0x7fffffff + 1;
+    e.epoch = h->epoch;
     CK(launch_f32tc_split(Af, lda, Bf, ldb, e, &launches, h->stream));
     int rc = f32tc_run(h, tc, e, alpha, beta, C, ldc, al16(C), level, s, split, ks_per_split, cadence, ksteps, tiles_n,
                        nf, ws + oTc[6], ws + oTc[7], ws + oTc[9], split > 1 ? ws + oPart : nullptr, &launches);
@@ -1733,12 +1740,16 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
       h->launches += launches;
       launches = 0;
       rc = fetch_report(h, report, e.bad, &bad);
-      if (rc || !bad) return rc;
+      if (rc || bad != e.epoch) return rc;
       gate = nullptr;
       h->rep_clean = false;
     }
-    CK(launch_kmajor_operands_if(gate, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
+    CK(launch_kmajor_operands_if(gate, e.epoch, Af, lda, M, K, ws + oAt, ldt, Bf, ldb, N, b_ok ? nullptr : ws + oBp, ldbp,
                                  &launches, h->stream));
+  } else if (!At_given && !detect && encode_small_fits(M, N, K, need_vw ? m_u : 0, n_u)) {
+    CK(launch_encode_small(Af, lda, M, K, ws + oAt, ldt, need_vw ? m_u : 0, need_vw ? ws + oV : nullptr, ldv,
+                           abft ? ws + oNa : nullptr, Bf, ldb, N, need_vw ? n_u : 0, b_ok ? nullptr : ws + oBp, ldbp,
+                           need_vw ? ws + oW : nullptr, abft ? ws + oNb : nullptr, &launches, h->stream));
   } else {
     // A^T, with the A side of the encoding (block sums, row norms) in the same pass
     if (!At_given)
@@ -1799,6 +1810,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   p.sink_lam = sink ? h->sink_lam : nullptr;
   p.sink_x = sink ? h->sink_x : nullptr;
   p.only_if = gate;
+  p.epoch = h->epoch;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
   const bool timed = h->timing && !gate;  // (the tensor-core kernels were timed themselves)
   if (timed) {

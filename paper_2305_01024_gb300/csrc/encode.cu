@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "internal.cuh"
+#include "ptx.cuh"
 
 namespace ftg {
 
@@ -45,8 +46,8 @@ __global__ void __launch_bounds__(256) transpose_encode_kernel(const float* __re
                                                                int K, float* __restrict__ At, long long ldt,
                                                                int m_u, float* __restrict__ V, long long ldv,
                                                                float* __restrict__ part,
-                                                               const int* __restrict__ gate) {
-  if (gate && !*gate) return;  // only run if *gate is set
+                                                               const int* __restrict__ gate, int epoch) {
+  if (gate && *gate != epoch) return;  // only run if *gate holds this call's number
   __shared__ float tile[128][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * 32, m0 = blockIdx.y * 128;
@@ -109,8 +110,8 @@ __global__ void __launch_bounds__(256) transpose_encode_kernel(const float* __re
 }
 
 __global__ void copy_pad_kernel(const float* __restrict__ X, long long ldx, int R, int Cn,
-                                float* __restrict__ Y, long long ldy, const int* __restrict__ gate) {
-  if (gate && !*gate) return;  // only run if *gate is set
+                                float* __restrict__ Y, long long ldy, const int* __restrict__ gate, int epoch) {
+  if (gate && *gate != epoch) return;  // only run if *gate holds this call's number
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)R * Cn) return;
   const int r = (int)(idx / Cn), c = (int)(idx % Cn);
@@ -205,6 +206,110 @@ __global__ void __launch_bounds__(256) encode_kmajor_kernel(const float* __restr
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (c0 + q < L) part[(long long)blockIdx.y * L + c0 + q] = sq[q];
+  }
+}
+
+// The whole encode pass of a small problem in one launch (units of at most 32
+// rows and 128 columns): the first blocks take 32 rows of A each, over all of
+// K: A^T, e^T A per unit of m_u rows, row norms; the others 128 columns of B:
+// B e per unit of n_u columns, column norms, and the padded copy of B if Bp is
+// given.  m_u = 0: layout and norms only.  256 elements of K a step, every load
+// of a step in flight at once; bound by the latency of a step or two.
+// (256 x 256 x 256: the four launches it stands for took 20 us with the gaps.)
+__global__ void __launch_bounds__(1024) encode_small_kernel(const float* __restrict__ A, long long lda, int M, int K,
+                                                            float* __restrict__ At, long long ldt, int m_u,
+                                                            float* __restrict__ V, long long ldv, float* __restrict__ nA,
+                                                            const float* __restrict__ B, long long ldb, int N, int n_u,
+                                                            int vec, float* __restrict__ Bp, long long ldbp,
+                                                            float* __restrict__ W, float* __restrict__ nB, int a_blocks) {
+  __shared__ float sh[32 * 257];  // A: a 32 x 256 tile; B: 32 warps' column norms
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
+  if ((int)blockIdx.x < a_blocks) {
+    const int m0 = blockIdx.x * 32, m = m0 + warp;
+    float sq = 0.f;
+    for (int k0 = 0; k0 < K; k0 += 256) {
+      float v[8];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const int k = k0 + 32 * h + lane;
+        v[h] = m < M && k < K ? __ldg(A + (long long)m * lda + k) : 0.f;
+      }
+      __syncthreads();  // the previous tile is written out
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        sh[warp * 257 + 32 * h + lane] = v[h];
+        sq = fmaf(v[h], v[h], sq);
+      }
+      __syncthreads();
+      // rows k0 + warp + 32 q of A^T, lane = row of A
+      float s[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = k0 + warp + 32 * q;
+        s[q] = sh[lane * 257 + warp + 32 * q];
+        if (k < K && m0 + lane < M) At[(long long)k * ldt + m0 + lane] = s[q];
+      }
+      for (int o = 1; o < m_u; o <<= 1) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+      }
+      if (m_u && (lane & (m_u - 1)) == 0 && m0 + lane < M) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (k0 + warp + 32 * q < K) V[(long long)((m0 + lane) / m_u) * ldv + k0 + warp + 32 * q] = s[q];
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (nA && lane == 0 && m < M) nA[m] = sqrtf(sq);
+  } else {
+    const int n0 = ((int)blockIdx.x - a_blocks) * 128, c = n0 + lane * 4;
+    float sq[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k0 = warp; k0 < K; k0 += 256) {
+      float x[8][4], s[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = k0 + 32 * i;
+        const float* row = B + (long long)min(k, K - 1) * ldb + c;
+        const int cols = k < K ? N - c : 0;
+        if (vec && cols >= 4) {
+          const float4 u = __ldg(reinterpret_cast<const float4*>(row));
+          x[i][0] = u.x; x[i][1] = u.y; x[i][2] = u.z; x[i][3] = u.w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[i][e] = e < cols ? __ldg(row + e) : 0.f;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (Bp && c < N && k0 + 32 * i < K)
+          *reinterpret_cast<float4*>(Bp + (long long)(k0 + 32 * i) * ldbp + c) =
+              make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sq[e] = fmaf(x[i][e], x[i][e], sq[e]);
+        s[i] = (x[i][0] + x[i][1]) + (x[i][2] + x[i][3]);
+      }
+      for (int o = 1; o < n_u / 4; o <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+      }
+      if (n_u && (lane & (n_u / 4 - 1)) == 0 && c < N) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (k0 + 32 * i < K) W[(long long)(c / n_u) * ldv + k0 + 32 * i] = s[i];
+      }
+    }
+    if (!nB) return;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) sh[warp * 128 + lane * 4 + e] = sq[e];
+    __syncthreads();
+    if (threadIdx.x < 128 && n0 + (int)threadIdx.x < N) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < 32; ++w) s += sh[w * 128 + threadIdx.x];
+      nB[n0 + threadIdx.x] = sqrtf(s);
+    }
   }
 }
 
@@ -323,7 +428,7 @@ cudaError_t launch_transpose_encode(const float* A, long long lda, int M, int K,
   if (V && (m_u < 2 || m_u > 128 || (m_u & (m_u - 1)))) return cudaErrorInvalidValue;
   dim3 g((K + 31) / 32, (M + 127) / 128);
   transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, V ? m_u : 0, V, ldv, nrm ? scratch : nullptr,
-                                          nullptr);
+                                          nullptr, 0);
   ++*launches;
   if (nrm) {
     colnorm_finish_kernel<<<(M + 31) / 32, 256, 0, st>>>(scratch, (K + 31) / 32, M, nrm);
@@ -332,24 +437,39 @@ cudaError_t launch_transpose_encode(const float* A, long long lda, int M, int K,
   return cudaGetLastError();
 }
 
+// Whether launch_encode_small takes the problem (units 0: none): small enough
+// for the launches to count more than the bandwidth.
+bool encode_small_fits(int M, int N, int K, int m_u, int n_u) {
+  return K <= 1024 && ((long long)M + N) * K <= 3000000 && (m_u == 0 || (m_u >= 2 && m_u <= 32 && n_u >= 4 && n_u <= 128));
+}
+cudaError_t launch_encode_small(const float* A, long long lda, int M, int K, float* At, long long ldt, int m_u, float* V,
+                                long long ldv, float* nA, const float* B, long long ldb, int N, int n_u, float* Bp,
+                                long long ldbp, float* W, float* nB, int* launches, cudaStream_t st) {
+  const int vec = ldb % 4 == 0 && ((uintptr_t)B & 15) == 0;
+  const int ab = (M + 31) / 32, bb = (W || nB || Bp) ? (N + 127) / 128 : 0;
+  ++*launches;
+  return launch_pdl(encode_small_kernel, ab + bb, 1024, 0, st, A, lda, M, K, At, ldt, m_u, V, ldv, nA, B, ldb, N, n_u, vec,
+                    Bp, ldbp, W, nB, ab);
+}
+
 cudaError_t launch_copy_pad(const float* X, long long ldx, int R, int Cn, float* Y, long long ldy,
                             cudaStream_t st) {
   const long long total = (long long)R * Cn;
-  copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(X, ldx, R, Cn, Y, ldy, nullptr);
+  copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(X, ldx, R, Cn, Y, ldy, nullptr, 0);
   return cudaGetLastError();
 }
 
-// The operand layout of the CUDA-core kernel, produced only if *gate is set
+// The operand layout of the CUDA-core kernel, produced only if *gate == epoch
 // when the kernels run (null: always): A^T, and (Bp not null) B with padded rows.
-cudaError_t launch_kmajor_operands_if(const int* gate, const float* A, long long lda, int M, int K, float* At,
+cudaError_t launch_kmajor_operands_if(const int* gate, int epoch, const float* A, long long lda, int M, int K, float* At,
                                       long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
                                       int* launches, cudaStream_t st) {
   dim3 g((K + 31) / 32, (M + 127) / 128);
-  transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, 0, nullptr, 0, nullptr, gate);
+  transpose_encode_kernel<<<g, 256, 0, st>>>(A, lda, M, K, At, ldt, 0, nullptr, 0, nullptr, gate, epoch);
   ++*launches;
   if (Bp) {
     const long long total = (long long)K * N;
-    copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, ldb, K, N, Bp, ldbp, gate);
+    copy_pad_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, ldb, K, N, Bp, ldbp, gate, epoch);
     ++*launches;
   }
   return cudaGetLastError();

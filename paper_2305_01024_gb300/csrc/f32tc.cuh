@@ -59,7 +59,9 @@ struct F32TcParams {
   float* partial;              // [split][M][N], or null
   const Fault* faults; int nfaults;
   DevReport* rep; ftgemm_fault_record* recs;
-  const int* bad;              // set by the encode pass when an operand is outside the split's range
+  // the encode pass sets *bad to `epoch` (the call's own number) when an operand
+  // is outside the split's range: nothing to clear before a call
+  const int* bad; int epoch;
 };
 
 // The encode pass: operand planes, and (um > 0) checksum vectors and norms.
@@ -72,7 +74,7 @@ struct F32TcPrep {
   uint16_t* Vp; uint16_t* Wp;   // their planes, as A's
   float* pa; float* pb;         // squared-norm partials [ceil(K / 128)][M], [ceil(K / 128)][N]
   float* nA; float* nB; float* sq16a; float* sq16b;
-  int* bad;
+  int* bad; int epoch;
 };
 
 // 2-D maps over the planes as rows of 128 bytes, no swizzle (the planes are

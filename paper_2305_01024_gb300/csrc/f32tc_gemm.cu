@@ -216,7 +216,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     f32tc_kernel(const __grid_constant__ F32TcMaps maps, const __grid_constant__ F32TcParams p) {
   using Cfg = F32TcCfg<BN>;
   constexpr int S = Cfg::STAGES, NBUF = Cfg::NBUF, CPT = Cfg::CPT, KC = Cfg::KC, EPI_T = Cfg::EPI_T;
-  if (*p.bad) return;  // an operand outside the split's range: the CUDA-core kernel runs instead
+  pdl_wait();
+  pdl_trigger();
+  if (*p.bad == p.epoch) return;  // an operand outside the split's range: the CUDA-core kernel runs instead
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = smem_raw + (-smem_u32(smem_raw) & 1023u);  // (shared address space kept)
   F32TcTail<BN>& T = *reinterpret_cast<F32TcTail<BN>*>(base + S * Cfg::STAGE_BYTES);
@@ -759,8 +761,7 @@ static cudaError_t f32tc_launch(const F32TcMaps& maps, const F32TcParams& p, int
     if (fa.numRegs != F32TcCfg<BN>::REGS) return cudaErrorInvalidConfiguration;
   }
   const int workers = items < sms / 2 ? items : sms / 2;
-  f32tc_kernel<BN, ABFT, SUMS><<<2 * workers, F32TcCfg<BN>::THREADS, smem, st>>>(maps, p);
-  return cudaGetLastError();
+  return launch_pdl(f32tc_kernel<BN, ABFT, SUMS>, 2 * workers, F32TcCfg<BN>::THREADS, smem, st, maps, p);
 }
 
 // The segments (checksums; the product too if it goes by segments), then the

@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 
 #include "f32tc.cuh"
+#include "ptx.cuh"
 
 namespace ftg {
 
@@ -77,6 +78,8 @@ __global__ void __launch_bounds__(256) f32tc_split_kernel(const float* __restric
                                                           const F32TcPrep e, int veca, int vecb, int a_blocks) {
   __shared__ __align__(16) float usum[8][128];  // unit sums per element of K (units of 128: two halves)
   __shared__ float sq4[4][128];                 // squared norms per chunk
+  pdl_wait();
+  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool side_a = (int)blockIdx.x < a_blocks;
   const int blk = side_a ? blockIdx.x : blockIdx.x - a_blocks;
@@ -171,7 +174,7 @@ __global__ void __launch_bounds__(256) f32tc_split_kernel(const float* __restric
       }
     }
   }
-  if (__any_sync(0xffffffffu, out) && lane == 0) *e.bad = 1;
+  if (__any_sync(0xffffffffu, out) && lane == 0) *e.bad = e.epoch;
   if (!us) return;
   __syncthreads();
   const int chunks = min(4, nch - kb * 4);
@@ -209,6 +212,8 @@ __global__ void __launch_bounds__(1024) f32tc_norms_kernel(const float* __restri
                                                            float* __restrict__ nA, float* __restrict__ nB,
                                                            float* __restrict__ sq16a, float* __restrict__ sq16b) {
   __shared__ float red[32][16];
+  pdl_wait();
+  pdl_trigger();
   const int ba = (M + 15) / 16;
   const bool side_a = (int)blockIdx.x < ba;
   const int b = side_a ? blockIdx.x : blockIdx.x - ba;
@@ -236,20 +241,18 @@ __global__ void __launch_bounds__(1024) f32tc_norms_kernel(const float* __restri
 
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
                                int* launches, cudaStream_t st) {
-  cudaError_t er = cudaMemsetAsync(e.bad, 0, sizeof(int), st);
-  if (er != cudaSuccess) return er;
   const int veca = lda % 4 == 0 && ((uintptr_t)A & 15) == 0, vecb = ldb % 4 == 0 && ((uintptr_t)B & 15) == 0;
   const int kgroups = (e.K + 127) / 128;
   const long long ab = (long long)kgroups * ((e.M + 127) / 128), bb = (long long)kgroups * ((e.N + 127) / 128);
   if (ab + bb > 0x7fffffff) return cudaErrorInvalidValue;
-  f32tc_split_kernel<<<(unsigned)(ab + bb), 256, 0, st>>>(A, lda, B, ldb, e, veca, vecb, (int)ab);
+  cudaError_t er = launch_pdl(f32tc_split_kernel, (unsigned)(ab + bb), 256, 0, st, A, lda, B, ldb, e, veca, vecb, (int)ab);
   *launches += 1;
-  if (e.um) {
-    f32tc_norms_kernel<<<(e.M + 15) / 16 + (e.N + 15) / 16, 1024, 0, st>>>(e.pa, kgroups, e.M, e.pb, kgroups, e.N, e.nA,
-                                                                            e.nB, e.sq16a, e.sq16b);
+  if (er == cudaSuccess && e.um) {
+    er = launch_pdl(f32tc_norms_kernel, (e.M + 15) / 16 + (e.N + 15) / 16, 1024, 0, st, e.pa, kgroups, e.M, e.pb, kgroups,
+                    e.N, e.nA, e.nB, e.sq16a, e.sq16b);
     *launches += 1;
   }
-  return cudaGetLastError();
+  return er;
 }
 
 }  // namespace ftg

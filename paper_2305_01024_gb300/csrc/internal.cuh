@@ -118,7 +118,7 @@ struct SimtParams {
   // / (u * norm product) over its rows, columns and periods (float bits,
   // combined with atomicMax; zeroed by the host), and its 5 features
   float* sink_lam; float* sink_x;
-  const int* only_if;  // device flag: the kernel returns at once unless it is set (null: always run)
+  const int* only_if; int epoch;  // the kernel returns at once unless *only_if == epoch (null: always run)
 };
 
 struct SimtMaps {

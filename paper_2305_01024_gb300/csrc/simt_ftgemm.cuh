@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(T::NTHR, T::MINB)
   using L = SimtLayout<T, LEVEL>;
   using Aux = SimtAux<T, LEVEL>;
   constexpr int NV = L::NV, NW = L::NW;
-  if (p.only_if && !*p.only_if) return;
+  pdl_wait();
+  if (p.only_if && *p.only_if != p.epoch) return;
 
   extern __shared__ unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1225,8 +1226,7 @@ cudaError_t launch_simt_inj(const SimtMaps& maps, const SimtParams& p, int split
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((p.N + T::NT - 1) / T::NT, (p.M + T::MT - 1) / T::MT, split);
-  simt_ftgemm_kernel<T, LEVEL, INJ><<<grid, T::NTHR, smem, st>>>(maps.A, maps.B, maps.V, maps.W, p);
-  return cudaGetLastError();
+  return launch_pdl(simt_ftgemm_kernel<T, LEVEL, INJ>, grid, T::NTHR, smem, st, maps.A, maps.B, maps.V, maps.W, p);
 }
 
 template <class T, int LEVEL>
