@@ -2297,7 +2297,7 @@ static int f64_gemm(ftgemm_ctx* h, bool cplx, int64_t m, int64_t n, int64_t k, c
     if (rc) return rc;
     CK(cudaEventRecord(ev2.first, h->stream));
   }
-  CK(launch_f64_gemm(cplx, abft, p, h->stream));
+  CK(launch_f64_gemm(cplx, abft, p, h->num_sms > 0 ? h->num_sms : 148, h->stream));
   ++launches;
   if (h->timing) {
     CK(cudaEventRecord(ev2.second, h->stream));

@@ -10,11 +10,14 @@
 // and corrected (Section 4.2.1).  Complex values use |d| for the comparison.
 //
 // This part of GB300 has a low FP64 rate and no fast FP64 tensor path, so
-// the kernel is a CUDA-core (DFMA) kernel: 256 threads, register tiles of
-// 8 x 8 doubles (128 x 128 output tile) or 4 x 4 complex values (64 x 64),
-// k-steps of 8 staged through shared memory with a register prefetch.  The
-// checksum row and column cost one multiply-add per thread per k (1/64 of
-// the data work for doubles, 1/32 for complex).
+// the kernel is a CUDA-core (DFMA) kernel bound by that rate: a checksum unit
+// of 128 x 128 doubles (64 x 64 complex values) is computed by one CTA with
+// 8 x 8 (4 x 4) values a thread, or by a cluster of 4 or 8 CTAs that share its
+// checksums, whichever fills the GPU's waves better (f64_launch_g).  k-steps of
+// 8 are staged through shared memory with a register prefetch.  2048^3 with
+// BLOCK checksums: 17.4 ms with one CTA a unit, 16.3 ms with four; the FP64
+// units alone need 13.7 ms.  300 x 260 x 520: 2.28 ms, now 0.36 ms.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,6 +25,7 @@
 #include <type_traits>
 
 #include "fp64.cuh"
+#include "ptx.cuh"
 
 namespace ftg {
 
@@ -132,6 +136,12 @@ __global__ void __launch_bounds__(256) f64_reduce_rows_kernel(const T* __restric
 
 // ---- the GEMM --------------------------------------------------------------
 
+// A shared variable of the cluster's CTA `rank` (this CTA's own without one).
+template <bool CL, class V>
+__device__ __forceinline__ V* f64_peer(V* v, int rank) {
+  if constexpr (CL) return cooperative_groups::this_cluster().map_shared_rank(v, rank);
+  else return v;
+}
 
 // The report of one verification event; the record's `reserved` field
 // carries its slot so that the host can pair it with the imaginary parts.
@@ -152,33 +162,54 @@ __device__ void f64_report(const F64Params& p, ftgemm_fault_record r, double di,
   }
 }
 
-template <bool CPLX, bool ABFT>
-__global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
+// A GM x GN cluster computes one unit tile, each CTA a (1/GM x 1/GN) piece of
+// it (1 x 1: one CTA, no cluster), with 256 threads of (TM / GM) x (TN / GN)
+// elements.  The fp64 units take 64 cycles per warp instruction, so smaller
+// fragments cost nothing, while smaller pieces fill the GPU and even out its
+// last wave.  One CTA per row of pieces keeps that row's checksums, one per
+// column the column's, all different CTAs; at a verification they add up the
+// pieces' sums through distributed shared memory, and CTA 0 decides.
+template <bool CPLX, bool ABFT, int GM, int GN>
+__global__ void __launch_bounds__(256, GM * GN == 1 ? 1 : 2) f64_gemm_kernel(const F64Params p) {
   using Cfg = F64Cfg<CPLX>;
   using T = typename Cfg::T;
-  constexpr int BM = Cfg::BM, BN = Cfg::BN, TM = Cfg::TM, TN = Cfg::TN, BK = F64_BK;
+  constexpr int UM = Cfg::BM, UN = Cfg::BN;  // the unit
+  constexpr int BM = UM / GM, BN = UN / GN, TM = Cfg::TM / GM, TN = Cfg::TN / GN, BK = F64_BK;
   constexpr int LA = BM * BK / 256, LB = BN * BK / 256;  // elements each thread stages per k-step
-  static_assert(BM == 16 * TM && BN == 16 * TN && BN + BM <= 256, "thread layout");
+  constexpr int VM = TM < 4 ? TM : 4, VN = TN < 4 ? TN : 4;
+  constexpr bool CL = ABFT && GM * GN > 1;  // the CTAs of a unit talk to one another
+  static_assert(TM >= 1 && LA >= 1 && BM == 16 * TM && BN == 16 * TN && BN + BM <= 256, "thread layout");
   __shared__ __align__(16) T As[2][BK][BM];
   __shared__ __align__(16) T Bs[2][BK][BN];
   __shared__ T vs[2][BK], ws[2][BK];
-  __shared__ T rowsum[BM], colpart[8][BN], dres_r[BM], dres_c[BN];
-  __shared__ double tau_r[BM], tau_c[BN], red[16];
+  __shared__ T rowsum[BM], colsum[BN], colpart[8][BN];
+  __shared__ double red[16], growth;
+  // this piece's flagged rows and columns, and the unit's decision (CTA 0's is used)
   __shared__ unsigned long long best_r, best_c;
-  __shared__ int nr, nc, ib, jb;
+  __shared__ int any[2], nr, nc, ib, jb;
+  __shared__ T d_r, d_c, fix_v;
+  __shared__ double tau_r, tau_c;
   __shared__ int fix_kind, fix_i, fix_j;  // 0 none, 1 correct acc, 2 reset row checksum, 3 reset column checksum
-  __shared__ T fix_v;
 
   const T* A = reinterpret_cast<const T*>(p.A);
   const T* B = reinterpret_cast<const T*>(p.B);
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
-  const int tn = blockIdx.x, tm = blockIdx.y, tiles_n = gridDim.x;
-  const int m0 = tm * BM, n0 = tn * BN;
-  const int rows = min(BM, p.M - m0), cols = min(BN, p.N - n0);
+  const int tn = blockIdx.x / GN, cc = blockIdx.x % GN, tm = blockIdx.y / GM, cr = blockIdx.y % GM;
+  const int tiles_n = gridDim.x / GN;
+  const int u0 = tm * UM, v0 = tn * UN;                // the unit's first row and column
+  const int m0 = u0 + cr * BM, n0 = v0 + cc * BN;      // this piece's
+  const int rows = min(BM, p.M - m0), cols = min(BN, p.N - n0);  // may be <= 0 in the last unit
   const int nks = (p.K + BK - 1) / BK;
-  // the checksum element this thread carries: column checksum of column
-  // `tid` (tid < BN) or row checksum of row `tid - BN` (BN <= tid < BN + BM)
-  const bool own_c = tid < BN, own_r = tid >= BN && tid < BN + BM;
+  auto frow = [&](int i) { return (i / VM) * (16 * VM) + ty * VM + i % VM; };
+  auto fcol = [&](int j) { return (j / VN) * (16 * VN) + tx * VN + j % VN; };
+  // the checksum element this thread carries: column checksum of column `tid`
+  // (tid < BN) or row checksum of row `tid - BN` of the piece
+  const bool own_c = (GM == 1 || cr == (cc + 1) % GM) && tid < BN;
+  const bool own_r = cc == cr % GN && tid >= BN && tid < BN + BM;
+  auto sync = [&]() {
+    if constexpr (CL) cluster_sync();
+    else __syncthreads();
+  };
 
   T acc[TM][TN];
 #pragma unroll
@@ -187,13 +218,15 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
     for (int j = 0; j < TN; ++j) acc[i][j] = f64_zero(T{});
   T csum = f64_zero(T{});
   double tau_own = 0.0;
+  [[maybe_unused]] int odd = 0;  // verifications take turns with any[2]
+  if (CL && tid == 0) any[0] = any[1] = 0;
 
   if constexpr (ABFT) {
-    // Frobenius norms of the tile's rows of A and columns of B, then the
+    // Frobenius norms of the unit's rows of A and columns of B, then the
     // thresholds lambda*u*||A(i,:)||*||B(:,J)||_F and lambda*u*||A(I,:)||_F*||B(:,j)||
     double a2 = 0.0, b2 = 0.0;
-    if (tid < rows) a2 = p.nA[m0 + tid] * p.nA[m0 + tid];
-    if (tid < cols) b2 = p.nB[n0 + tid] * p.nB[n0 + tid];
+    if (tid < UM && u0 + tid < p.M) a2 = p.nA[u0 + tid] * p.nA[u0 + tid];
+    if (tid < UN && v0 + tid < p.N) b2 = p.nB[v0 + tid] * p.nB[v0 + tid];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       a2 += __shfl_xor_sync(0xffffffffu, a2, o);
@@ -214,11 +247,9 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
     fb = sqrt(fb);
     if (own_c) tau_own = tid < cols ? p.lam_u * fa * p.nB[n0 + tid] : 0.0;
     if (own_r) tau_own = tid - BN < rows ? p.lam_u * p.nA[m0 + tid - BN] * fb : 0.0;
-    if (own_c) tau_c[tid] = tau_own;
-    if (own_r) tau_r[tid - BN] = tau_own;
   }
 
-  // this tile's faults: [f_next, f_end) of the table sorted by (tile, k-step)
+  // this unit's faults: [f_next, f_end) of the table sorted by (tile, k-step)
   int f_next = 0, f_end = 0, f_ks = INT_MAX;
   if (p.nfaults > 0) {
     const int tile = tm * tiles_n + tn;
@@ -277,9 +308,9 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
     for (int kk = 0; kk < BK; ++kk) {
       T a[TM], b[TN];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][(i >> 2) * 64 + ty * 4 + (i & 3)];
+      for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][frow(i)];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][(j >> 2) * 64 + tx * 4 + (j & 3)];
+      for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][fcol(j)];
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -294,25 +325,19 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
     while (f_ks == s) {
       const Fault F = p.faults[f_next];
       const bool imag = (F.target & 4) != 0;
-      const int tg = F.target & 3;
+      const int tg = F.target & 3, fr = F.row - cr * BM, fc = F.col - cc * BN;  // inside the piece
       const T off = f64_offset(T{}, (double)F.delta, imag);
       if (tg == T_ACC) {
-        if (ty == (F.row & 63) >> 2 && tx == (F.col & 63) >> 2) {
-          // every element takes w * off with w = 1 only at the target: no
-          // indexed access, so the accumulators stay in registers
+        // (no indexed access, so the accumulators stay in registers)
 #pragma unroll
-          for (int i = 0; i < TM; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < TN; ++j) {
-              const double w = ((i >> 2) * 64 + (i & 3) == (F.row & ~63) + (F.row & 3) &&
-                                (j >> 2) * 64 + (j & 3) == (F.col & ~63) + (F.col & 3)) ? 1.0 : 0.0;
-              acc[i][j] = f64_axpy(w, off, acc[i][j]);
-            }
-        }
+          for (int j = 0; j < TN; ++j)
+            if (frow(i) == fr && fcol(j) == fc) acc[i][j] = f64_add(acc[i][j], off);
       } else if (ABFT && tg == T_ROWSUM) {
-        if (own_r && tid - BN == F.row) csum = f64_add(csum, off);
+        if (own_r && tid - BN == fr) csum = f64_add(csum, off);
       } else if (ABFT && tg == T_COLSUM) {
-        if (own_c && tid == F.col) csum = f64_add(csum, off);
+        if (own_c && tid == fc) csum = f64_add(csum, off);
       }
       ++f_next;
       f_ks = f_next < f_end ? p.faults[f_next].kstep : INT_MAX;
@@ -320,7 +345,7 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
 
     if constexpr (ABFT) {
       if ((s + 1) % p.cadence == 0 || s == nks - 1) {
-        // row sums: across the 16 threads of a half-warp (tx), xor tree
+        // the piece's row sums: across the 16 threads of a half-warp (tx), xor tree
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
           T r = acc[i][0];
@@ -328,7 +353,7 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
           for (int j = 1; j < TN; ++j) r = f64_add(r, acc[i][j]);
 #pragma unroll
           for (int o = 1; o < 16; o <<= 1) r = f64_add(r, f64_shfl(r, o));
-          if (tx == 0) rowsum[(i >> 2) * 64 + ty * 4 + (i & 3)] = r;
+          if (tx == 0) rowsum[frow(i)] = r;
         }
         // column sums: the two half-warps of a warp, then the 8 warps in order
 #pragma unroll
@@ -337,9 +362,12 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
 #pragma unroll
           for (int i = 1; i < TM; ++i) c = f64_add(c, acc[i][j]);
           c = f64_add(c, f64_shfl(c, 16));
-          if (lane < 16) colpart[warp][(j >> 2) * 64 + tx * 4 + (j & 3)] = c;
+          if (lane < 16) colpart[warp][fcol(j)] = c;
         }
         if (tid == 0) {
+          // growth term of this verification's threshold, per |checksum|, after
+          // k elements of K
+          growth = p.mu_u * sqrt((double)min((s + 1) * BK, p.K));
           nr = 0;
           nc = 0;
           best_r = 0ull;
@@ -349,29 +377,40 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
           fix_kind = 0;
         }
         __syncthreads();
-        T d = f64_zero(T{});
-        bool flag = false;
-        // this verification's threshold: the norm term plus the growth term
-        // mu * u * sqrt(k) * |checksum| after k elements of K
-        const double tau_now = tau_own + p.mu_u * sqrt((double)min((s + 1) * BK, p.K)) * f64_abs(csum);
-        if (own_c) {
+        if (tid < BN) {
           T c = colpart[0][tid];
 #pragma unroll
           for (int w = 1; w < 8; ++w) c = f64_add(c, colpart[w][tid]);
-          colpart[0][tid] = c;  // the column sum, kept for a checksum reset
-          d = f64_sub(c, csum);
-          flag = tid < cols && f64_abs(d) > tau_now;
-          dres_c[tid] = d;
-          tau_c[tid] = tid < cols ? tau_now : 0.0;
-        } else if (own_r) {
-          d = f64_sub(rowsum[tid - BN], csum);
-          flag = tid - BN < rows && f64_abs(d) > tau_now;
-          dres_r[tid - BN] = d;
-          tau_r[tid - BN] = tid - BN < rows ? tau_now : 0.0;
+          colsum[tid] = c;
         }
-        if (__syncthreads_or(flag)) {
+        sync();
+        T d = f64_zero(T{}), tot = f64_zero(T{});  // residual and data sum of this thread's entry
+        bool flag = false;
+        double tau_now = 0.0;  // this verification's threshold: the norm term plus the growth term
+        const int ui = own_c ? cc * BN + tid : cr * BM + tid - BN;  // the entry's index in the unit
+        if (own_c || own_r) {
+          const T* src = own_c ? &colsum[tid] : &rowsum[tid - BN];
+          tau_now = tau_own + growth * f64_abs(csum);
+          tot = *f64_peer<CL>(src, own_c ? cc : cr * GN);
+          for (int g = 1; g < (own_c ? GM : GN); ++g)
+            tot = f64_add(tot, *f64_peer<CL>(src, own_c ? g * GN + cc : cr * GN + g));
+          d = f64_sub(tot, csum);
+          flag = (own_c ? tid < cols : tid - BN < rows) && f64_abs(d) > tau_now;
+        }
+        bool found;
+        if constexpr (CL) {
+          if (flag) *f64_peer<CL>(&any[odd], 0) = 1;
+          cluster_sync();
+          found = *f64_peer<CL>(&any[odd], 0) != 0;
+          odd ^= 1;
+          // for the next one; its last readers have passed this verification's first barrier
+          if (tid == 0) any[odd] = 0;
+        } else {
+          found = __syncthreads_or(flag);
+        }
+        if (found) {
           // rare path: count, then the largest |d|/tau (exact in double;
-          // ties to the smaller index)
+          // ties to the smaller index), first inside each piece
           double score = 0.0;
           if (flag) {
             const double a = f64_abs(d);
@@ -381,26 +420,58 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
           }
           __syncthreads();
           if (flag && (unsigned long long)__double_as_longlong(score) == (own_c ? best_c : best_r))
-            atomicMin(own_c ? &jb : &ib, own_c ? tid : tid - BN);
+            atomicMin(own_c ? &jb : &ib, ui);
           __syncthreads();
-          if (tid == 0) {
-            const int ir = nr ? ib : -1, jc = nc ? jb : -1;
-            const T dR = ir >= 0 ? dres_r[ir] : f64_zero(T{});
-            const T dC = jc >= 0 ? dres_c[jc] : f64_zero(T{});
-            const double tR = ir >= 0 ? tau_r[ir] : 0.0, tC = jc >= 0 ? tau_c[jc] : 0.0;
+          if (flag && ui == (own_c ? jb : ib)) {  // the located row's / column's residual
+            *(own_c ? &d_c : &d_r) = d;
+            *(own_c ? &tau_c : &tau_r) = tau_now;
+          }
+          sync();
+          if (tid == 0 && cr == 0 && cc == 0) {
+            // then over the pieces (not by atomics on CTA 0's memory: a 64-bit
+            // maximum taken so from several CTAs located the wrong column)
+            int nr_u = 0, nc_u = 0, ir = -1, jc = -1;
+            unsigned long long best_ru = 0ull, best_cu = 0ull;
+            T dR = f64_zero(T{}), dC = f64_zero(T{});
+            double tR = 0.0, tC = 0.0;
+            for (int g = 0; g < GM * GN; ++g) {
+              const int gr = *f64_peer<CL>(&nr, g), gc = *f64_peer<CL>(&nc, g);
+              if (gr) {
+                const unsigned long long v = *f64_peer<CL>(&best_r, g);
+                const int i = *f64_peer<CL>(&ib, g);
+                if (!nr_u || v > best_ru || (v == best_ru && i < ir)) {
+                  best_ru = v;
+                  ir = i;
+                  dR = *f64_peer<CL>(&d_r, g);
+                  tR = *f64_peer<CL>(&tau_r, g);
+                }
+                nr_u += gr;
+              }
+              if (gc) {
+                const unsigned long long v = *f64_peer<CL>(&best_c, g);
+                const int j = *f64_peer<CL>(&jb, g);
+                if (!nc_u || v > best_cu || (v == best_cu && j < jc)) {
+                  best_cu = v;
+                  jc = j;
+                  dC = *f64_peer<CL>(&d_c, g);
+                  tC = *f64_peer<CL>(&tau_c, g);
+                }
+                nc_u += gc;
+              }
+            }
             ftgemm_fault_record rec;
             rec.tile_m = tm;
             rec.tile_n = tn;
             rec.kstep = s;
-            rec.row = ir >= 0 ? m0 + ir : -1;
-            rec.col = jc >= 0 ? n0 + jc : -1;
+            rec.row = ir >= 0 ? u0 + ir : -1;
+            rec.col = jc >= 0 ? v0 + jc : -1;
             rec.problem = 0;
             rec.reserved = 0;
             rec.residual_r = f64_re(dR);
             rec.residual_c = f64_re(dC);
             rec.tau = tR + tC;
             T delta = f64_zero(T{});
-            if (nr == 1 && nc == 1) {
+            if (nr_u == 1 && nc_u == 1) {
               if (f64_abs(f64_sub(dR, dC)) <= tR + tC) {
                 rec.kind = K_CORRECTED;
                 delta = dR;
@@ -411,12 +482,11 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
               } else {
                 rec.kind = K_UNCORRECTABLE;
               }
-            } else if ((nr == 1 && nc == 0) || (nr == 0 && nc == 1)) {
+            } else if ((nr_u == 1 && nc_u == 0) || (nr_u == 0 && nc_u == 1)) {
               // the checksum itself was hit: reset it from the data, C untouched
               rec.kind = K_CHECKSUM;
-              delta = f64_zero(T{});
-              delta = f64_sub(delta, nr ? dR : dC);  // checksum - data sum
-              fix_kind = nr ? 2 : 3;
+              delta = f64_sub(delta, nr_u ? dR : dC);  // checksum - data sum
+              fix_kind = nr_u ? 2 : 3;
               fix_i = ir;
               fix_j = jc;
             } else {
@@ -425,25 +495,22 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
             rec.delta = f64_re(delta);
             f64_report(p, rec, f64_im(delta), f64_im(dR), f64_im(dC));
           }
-          __syncthreads();
-          if (fix_kind == 1) {
-            const int fr = fix_i, fc = fix_j;
-            if (ty == (fr & 63) >> 2 && tx == (fc & 63) >> 2) {
-              const T fv = fix_v;
+          sync();
+          const int kind = *f64_peer<CL>(&fix_kind, 0);
+          const int fi = *f64_peer<CL>(&fix_i, 0), fj = *f64_peer<CL>(&fix_j, 0);
+          if (kind == 1) {
+            const T fv = *f64_peer<CL>(&fix_v, 0);
 #pragma unroll
-              for (int i = 0; i < TM; ++i)
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                  const double w = ((i >> 2) * 64 + (i & 3) == (fr & ~63) + (fr & 3) &&
-                                    (j >> 2) * 64 + (j & 3) == (fc & ~63) + (fc & 3)) ? -1.0 : 0.0;
-                  acc[i][j] = f64_axpy(w, fv, acc[i][j]);
-                }
-            }
-          } else if (fix_kind == 2) {
-            if (own_r && tid - BN == fix_i) csum = rowsum[fix_i];
-          } else if (fix_kind == 3) {
-            if (own_c && tid == fix_j) csum = colpart[0][fix_j];
+              for (int j = 0; j < TN; ++j)
+                if (cr * BM + frow(i) == fi && cc * BN + fcol(j) == fj) acc[i][j] = f64_sub(acc[i][j], fv);
+          } else if (kind == 2) {
+            if (own_r && ui == fi) csum = tot;
+          } else if (kind == 3) {
+            if (own_c && ui == fj) csum = tot;
           }
+          sync();  // CTA 0's decision is read
         }
       }
     }
@@ -455,11 +522,11 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
   T* Cp = reinterpret_cast<T*>(p.C);
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    const int r = m0 + (i >> 2) * 64 + ty * 4 + (i & 3);
+    const int r = m0 + frow(i);
     if (r >= p.M) continue;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int c = n0 + (j >> 2) * 64 + tx * 4 + (j & 3);
+      const int c = n0 + fcol(j);
       if (c >= p.N) continue;
       T* dst = Cp + (long long)r * p.ldc + c;
       if constexpr (CPLX) {
@@ -477,6 +544,7 @@ __global__ void __launch_bounds__(256, 1) f64_gemm_kernel(const F64Params p) {
       }
     }
   }
+  if constexpr (CL) cluster_sync();  // no CTA leaves while another may read its shared memory
 }
 
 // ---- launchers ---------------------------------------------------------------
@@ -509,18 +577,59 @@ cudaError_t launch_f64_encode(bool cplx, const void* A, long long lda, const voi
   return cudaGetLastError();
 }
 
-cudaError_t launch_f64_gemm(bool cplx, bool abft, const F64Params& p, cudaStream_t st) {
-  const int T = f64_tile(cplx);
-  const dim3 grid((p.N + T - 1) / T, (p.M + T - 1) / T);
-  if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
-  if (cplx) {
-    if (abft) f64_gemm_kernel<true, true><<<grid, 256, 0, st>>>(p);
-    else f64_gemm_kernel<true, false><<<grid, 256, 0, st>>>(p);
-  } else {
-    if (abft) f64_gemm_kernel<false, true><<<grid, 256, 0, st>>>(p);
-    else f64_gemm_kernel<false, false><<<grid, 256, 0, st>>>(p);
+template <bool CPLX, bool ABFT, int GM, int GN>
+static cudaError_t f64_launch(const F64Params& p, int tiles_m, int tiles_n, cudaStream_t st) {
+  const dim3 grid(tiles_n * GN, tiles_m * GM);
+  if (!ABFT || GM * GN == 1) {
+    f64_gemm_kernel<CPLX, ABFT, GM, GN><<<grid, 256, 0, st>>>(p);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = GN;
+  attr[0].val.clusterDim.y = GM;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, f64_gemm_kernel<CPLX, ABFT, GM, GN>, p);
+}
+
+template <bool CPLX, bool ABFT>
+static cudaError_t f64_launch_g(const F64Params& p, int sms, cudaStream_t st) {
+  const int T = f64_tile(CPLX), tiles_m = (p.M + T - 1) / T, tiles_n = (p.N + T - 1) / T;
+  if (tiles_m > 65535) return cudaErrorInvalidConfiguration;
+  // The pieces whose waves end first.  With checksums a cluster costs a few
+  // per cent: its barriers, and SMs that a GPC's clusters leave over.  Measured,
+  // ms, 1 / 4 / 8 pieces: BLOCK 2048^3 17.7 / 16.2 / 17.1, 4096x4096x2048 61.7 /
+  // 62.0 / 66.4, 1024^3 4.45 / 2.25 / 2.43, 300x260x520 2.28 / 0.62 / 0.36; OFF
+  // 2048^3 16.6 / 14.4 / 14.3, 512^3 2.08 / 0.54 / 0.29; complex BLOCK 1024^3 8.78 /
+  // 8.07, 200x150x96 0.45 / 0.15.
+  const long long units = (long long)tiles_m * tiles_n;
+  auto waves = [&](int pieces) { return (double)((units * pieces + sms - 1) / sms) / pieces; };
+  int g = 1;
+  double best = waves(1);
+  auto take = [&](int pieces, double cost) {
+    if (tiles_m <= 16383 && tiles_n <= 1 << 28 && waves(pieces) * cost < best) {
+      best = waves(pieces) * cost;
+      g = pieces;
+    }
+  };
+  take(4, ABFT ? 1.05 : 1.0);
+  if (!CPLX) take(8, ABFT ? 1.12 : 1.0);
+  if (g == 4) return f64_launch<CPLX, ABFT, 2, 2>(p, tiles_m, tiles_n, st);
+  if constexpr (!CPLX) {
+    if (g == 8) return f64_launch<CPLX, ABFT, 4, 2>(p, tiles_m, tiles_n, st);
+  }
+  return f64_launch<CPLX, ABFT, 1, 1>(p, tiles_m, tiles_n, st);
+}
+
+cudaError_t launch_f64_gemm(bool cplx, bool abft, const F64Params& p, int sms, cudaStream_t st) {
+  if (cplx) return abft ? f64_launch_g<true, true>(p, sms, st) : f64_launch_g<true, false>(p, sms, st);
+  return abft ? f64_launch_g<false, true>(p, sms, st) : f64_launch_g<false, false>(p, sms, st);
 }
 
 }  // namespace ftg

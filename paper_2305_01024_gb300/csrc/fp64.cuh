@@ -33,6 +33,6 @@ struct F64Params {
 int f64_tile(bool cplx);
 cudaError_t launch_f64_encode(bool cplx, const void* A, long long lda, const void* B, long long ldb, int M, int N,
                               int K, void* V, void* W, double* nA, double* nB, int* launches, cudaStream_t st);
-cudaError_t launch_f64_gemm(bool cplx, bool abft, const F64Params& p, cudaStream_t st);
+cudaError_t launch_f64_gemm(bool cplx, bool abft, const F64Params& p, int sms, cudaStream_t st);
 
 }  // namespace ftg
