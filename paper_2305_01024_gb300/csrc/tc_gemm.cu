@@ -60,8 +60,9 @@ namespace ftg {
 // tile with checksums) and half of B's 256 columns, and its tensor
 // memory holds its 128 rows of the accumulator, so the epilogue is the same
 // as a single CTA's.  Per SM a k-block then moves 32 KB of operands into
-// shared memory instead of 48 KB, and the ring holds 6 stages instead of 4.
-constexpr int TC_PAIR_STAGES = 6, TC_MAX_STAGES = 6;
+// shared memory instead of 48 KB, and the ring holds 6 stages instead of 4 (5
+// with checksums, whose epilogue stages 32 KB of C; 6 measured no faster).
+constexpr int TC_MAX_STAGES = 6;
 
 template <int DT, bool ABFT, bool PAIR = false>
 struct TcCfg {
@@ -71,7 +72,10 @@ struct TcCfg {
   static constexpr int ELEM = DT == 0 ? 2 : 1;        // bytes per operand element
   static constexpr int BK = 128 / ELEM;               // one 128-byte row per k-block
   static constexpr int UK = 32 / ELEM;                // K per MMA instruction
-  static constexpr int STAGES = PAIR ? TC_PAIR_STAGES : 4;
+  // columns a warp of the epilogue stages at a time: runs of 128 bytes of C
+  // where a pair's smaller stages leave room for them, else of 64
+  static constexpr int SC = PAIR ? 32 : 16;
+  static constexpr int STAGES = PAIR ? (ABFT ? 5 : 6) : 4;
   static constexpr int A_BYTES = BM * 128;                   // 16 KB
   static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * 128;  // 32 KB, or 16 KB a CTA of a pair
   static constexpr int MMA_M = PAIR ? 2 * BM : BM;            // rows of one MMA
@@ -81,6 +85,7 @@ struct TcCfg {
   static constexpr int EW = ABFT ? 8 : 4;
   static constexpr int THREADS = 64 + 32 * EW;
   static constexpr int MN_BOX = 64 * 128;  // bytes of one 64-column x 64-row box of an MN-major B
+  static constexpr int STG_BYTES = EW * 32 * SC * 4;  // the epilogue's staging tiles
   static constexpr uint32_t TMEM_COLS = 2 * BN;       // two fp32 accumulators
   static_assert(NPIECE == tc_npiece(DT) && NPIECE <= TC_MAX_PIECES, "column-checksum piece rows in shared memory");
   static_assert(!ABFT || (DM == TC_BM - NPIECE && DN + NPIECE <= TC_BN), "pieces inside the MMA tile");
@@ -131,7 +136,7 @@ struct TcSmemTail {
   double fix_delta[2];
   unsigned int sink_max;           // residual sink: largest residual / (u * norms) of the tile
   alignas(16) float colpart[4][256];  // per TMEM lane quarter partial column sums (data rows); float4 stores
-  float ccp[TC_MAX_PIECES][256];   // column-checksum pieces, TMEM lanes 128 - NP ..
+  alignas(16) float ccp[TC_MAX_PIECES][256];  // column-checksum pieces, TMEM lanes 128 - NP ..
   float crow[128];                 // row checksums
   float ccol[256];                 // column checksums
   // thresholds; before the threshold is formed, the same entry holds the
@@ -142,19 +147,17 @@ struct TcSmemTail {
   uint8_t flag_r[128], flag_c[256];
   double sum_r[128], sum_c[256];   // fp64 confirmation sums
   double sum_rp[128];              // fp64 row sums of the second half of the columns
-  // per epilogue warp: its 32 rows x 16 columns of one accumulator chunk,
-  // 64-byte rows with the 16-byte column groups XOR-swizzled by (row / 2) % 4
-  // (16-byte writes of 8 consecutive rows, and the read-back of 4 column
-  // groups of 2 rows, hit distinct banks), read back row-segment-wise so
-  // that C is written in 64-byte runs
-  alignas(16) float stg[8][32][16];
-};
+};  // the epilogue's staging tiles follow, SC columns of 32 rows per warp
 
-static_assert(offsetof(TcSmemTail, colpart) % 16 == 0 && offsetof(TcSmemTail, stg) % 16 == 0,
+static_assert(offsetof(TcSmemTail, colpart) % 16 == 0 && offsetof(TcSmemTail, ccp) % 16 == 0 &&
+                  sizeof(TcSmemTail) % 16 == 0,
               "vector stores into the epilogue's shared arrays");
-static_assert(1024 + TcCfg<0, true>::STAGES * TcCfg<0, true>::STAGE_BYTES + sizeof(TcSmemTail) <= 227 * 1024 &&
-                  1024 + TcCfg<0, true, true>::STAGES * TcCfg<0, true, true>::STAGE_BYTES + sizeof(TcSmemTail) <=
-                      227 * 1024,
+template <class Cfg>
+constexpr size_t tc_smem_bytes() {
+  return 1024 + (size_t)Cfg::STAGES * Cfg::STAGE_BYTES + sizeof(TcSmemTail) + Cfg::STG_BYTES;
+}
+static_assert(tc_smem_bytes<TcCfg<0, true>>() <= 227 * 1024 && tc_smem_bytes<TcCfg<0, true, true>>() <= 227 * 1024 &&
+                  tc_smem_bytes<TcCfg<0, false, true>>() <= 227 * 1024,
               "dynamic shared memory within the 227 KB a CTA may use");
 
 // Named barrier 1 over the N epilogue threads (128 or 256).
@@ -220,6 +223,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                          ~uintptr_t(1023));
   TcSmemTail& T = *reinterpret_cast<TcSmemTail*>(base + S * Cfg::STAGE_BYTES);
+  float* const stg = reinterpret_cast<float*>(&T + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = PAIR ? (int)cluster_ctarank() : 0;  // CTA of the pair (0 issues the MMAs)
   const bool leader = rank == 0;
@@ -446,7 +450,6 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
       // load latency hides behind the tile's main loop.
       const int pM = P.M, pN = P.N;
       const float sc = P.alpha * P.acc_scale;  // fp8: product of the per-tensor scales
-      const bool unit_sc = sc == 1.f;           // skip the scaling multiplies
       const float beta = P.beta;
       const int c_vec = P.c_vec;
       const long long ldc = P.ldc;
@@ -506,66 +509,87 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
       tc_fence_after();
       const bool row_ok = ok && data_row && gr < pM;
       float* crow_ptr = Cp + (long long)(row_ok ? gr : 0) * ldc + col0;
-      // alpha * acc + beta * C of one 16-column chunk of the warp's 32 rows,
-      // rows and columns inside the matrix only.  The chunk goes through the
-      // warp's staging tile: lane l then writes 16 bytes of row 8s + l/4
-      // (s = 0..3), so each store instruction covers 8 rows x 64 bytes
-      // instead of 32 rows x 16 bytes.  All lanes call it.
-      // With checksums it also leaves, in T.colpart[lq], the sums of the
-      // chunk's 16 columns over the warp's data rows: each lane adds its 4
-      // rows of 4 columns, then an xor tree over the 8 lanes of a column
-      // group.
-      auto store16w = [&](int ch, const float* v) {
-        float(*S)[16] = T.stg[ew];
+      // alpha * acc + beta * C of SC columns of the warp's 32 rows, rows and
+      // columns inside the matrix only.  They go through the warp's staging
+      // tile (16-byte column groups XOR-swizzled by the row, so that 8
+      // consecutive rows' writes and a read's rows hit distinct banks): a lane
+      // then writes 16 bytes of row RP s + lane / G, so that a store
+      // instruction covers RP rows x 4 SC bytes instead of 32 rows x 16 bytes.
+      // All lanes call it.  The usual tile (whole 16-byte groups, beta = 0) has
+      // straight-line code, loads before stores.  8192 x 8192 x K, us, with
+      // runs of 64 bytes and a branch a store / now: OFF K = 512 113 / 83, 1024
+      // 119 / 103; TILE 130 / 118, 141 / 127; from K = 2048 on the main loop
+      // bounds a tile.  (TILE's pass: 8000 cycles, 4900 without the stores.)
+      // With checksums it also leaves, in T.colpart[lq], the columns' sums
+      // over the warp's data rows: each lane adds its rows of 4 columns, then
+      // an xor tree over the lanes of a column group.
+      constexpr int SC = Cfg::SC, G = SC / 4, RP = 32 / G;
+      const bool whole = ok && c_vec && beta == 0.f && (col0 + DN <= pN || pN % 4 == 0);
+      const int srows = ok ? min(DM, pM - row0) - lq * 32 : 0;  // rows of the warp that are stored
+      auto store_cols = [&](int c0, const float* v) {
+        float* const S = stg + ew * 32 * SC;
+        auto swz = [](int row, int g) { return row * SC + 4 * (g ^ (G == 8 ? row & 7 : (row >> 1) & 3)); };
 #pragma unroll
-        for (int g = 0; g < 4; ++g)
-          *reinterpret_cast<float4*>(&S[lane][4 * (g ^ ((lane >> 1) & 3))]) =
+        for (int g = 0; g < G; ++g)
+          *reinterpret_cast<float4*>(&S[swz(lane, g)]) =
               make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
         __syncwarp();
-        float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int cq = lane % G, r0 = lane / G, c = c0 + 4 * cq, gc = col0 + c;
+        float4 x[G];
 #pragma unroll
-        for (int sgrp = 0; sgrp < 4; ++sgrp) {
-          const int rr = 8 * sgrp + (lane >> 2), cq = lane & 3;
-          const int tr_ = lq * 32 + rr, gr_ = row0 + tr_;  // tile row, matrix row
-          const float4 x = *reinterpret_cast<const float4*>(&S[rr][4 * (cq ^ ((rr >> 1) & 3))]);
-          if constexpr (ABFT) {
-            if (tr_ < DM) {
-              cs.x += x.x; cs.y += x.y; cs.z += x.z; cs.w += x.w;
-            }
-          }
-          const int c = ch * 16 + 4 * cq, gc = col0 + c;
-          if (!ok || tr_ >= DM || gr_ >= pM || c >= DN) continue;
-          float* dst = Cp + (long long)gr_ * ldc + gc;
-          if (c_vec && c + 3 < DN && gc + 3 < pN) {
-            float4 o = unit_sc ? x : make_float4(sc * x.x, sc * x.y, sc * x.z, sc * x.w);
-            if (beta != 0.f) {
-              const float4 ci = *reinterpret_cast<const float4*>(dst);
-              o.x = fmaf(beta, ci.x, o.x); o.y = fmaf(beta, ci.y, o.y);
-              o.z = fmaf(beta, ci.z, o.z); o.w = fmaf(beta, ci.w, o.w);
-            }
-            *reinterpret_cast<float4*>(dst) = o;
-          } else {
-            const float xs[4] = {x.x, x.y, x.z, x.w};
+        for (int s = 0; s < G; ++s) x[s] = *reinterpret_cast<const float4*>(&S[swz(RP * s + r0, cq)]);
+        float* dst = Cp + (long long)(row0 + lq * 32 + r0) * ldc + gc;
+        const int lim = c < DN && gc < pN ? srows - r0 : 0;
+        if (whole) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              if (c + e < DN && gc + e < pN) {
-                const float o = sc * xs[e];
-                dst[e] = beta != 0.f ? fmaf(beta, dst[e], o) : o;
+          for (int s = 0; s < G; ++s)
+            if (RP * s < lim)
+              *reinterpret_cast<float4*>(dst + (long long)(RP * s) * ldc) =
+                  make_float4(sc * x[s].x, sc * x[s].y, sc * x[s].z, sc * x[s].w);
+        } else {
+#pragma unroll 1
+          for (int s = 0; s < G; ++s, dst += (long long)RP * ldc) {
+            if (RP * s >= lim) break;
+            const float4 y = *reinterpret_cast<const float4*>(&S[swz(RP * s + r0, cq)]);
+            if (c_vec && c + 3 < DN && gc + 3 < pN) {
+              float4 o = make_float4(sc * y.x, sc * y.y, sc * y.z, sc * y.w);
+              if (beta != 0.f) {
+                const float4 ci = *reinterpret_cast<const float4*>(dst);
+                o.x = fmaf(beta, ci.x, o.x); o.y = fmaf(beta, ci.y, o.y);
+                o.z = fmaf(beta, ci.z, o.z); o.w = fmaf(beta, ci.w, o.w);
+              }
+              *reinterpret_cast<float4*>(dst) = o;
+            } else {
+              const float ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                if (c + e < DN && gc + e < pN) {
+                  const float o = sc * ys[e];
+                  dst[e] = beta != 0.f ? fmaf(beta, dst[e], o) : o;
+                }
               }
             }
           }
         }
         if constexpr (ABFT) {
+          float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int o = 4; o < 32; o <<= 1) {
+          for (int s = 0; s < G; ++s) {
+            // (only the last quarter's last rows hold pieces)
+            if (96 + RP * s + RP <= DM || lq * 32 + RP * s + r0 < DM) {
+              cs.x += x[s].x; cs.y += x[s].y; cs.z += x[s].z; cs.w += x[s].w;
+            }
+          }
+#pragma unroll
+          for (int o = G; o < 32; o <<= 1) {
             cs.x += __shfl_xor_sync(0xffffffffu, cs.x, o);
             cs.y += __shfl_xor_sync(0xffffffffu, cs.y, o);
             cs.z += __shfl_xor_sync(0xffffffffu, cs.z, o);
             cs.w += __shfl_xor_sync(0xffffffffu, cs.w, o);
           }
-          if (lane < 4) *reinterpret_cast<float4*>(&T.colpart[lq][ch * 16 + 4 * lane]) = cs;
+          if (r0 == 0) *reinterpret_cast<float4*>(&T.colpart[lq][c]) = cs;
         }
-        __syncwarp();  // the tile is refilled by the next chunk
+        __syncwarp();  // the tile is refilled by the next columns
       };
 
       if constexpr (ABFT) {
@@ -619,13 +643,15 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
         // ----- alpha * acc + beta * C, store -----
         // every lane reads tensor memory (the loads are warp-collective);
         // only rows inside the matrix store
-        // 32 columns per tensor-memory load: half the load-and-wait round trips
-        for (int c2 = 0; c2 < BN / 32; ++c2) {
-          float v2[32];
-          tmem_ld32(tl + c2 * 32, v2);
-          tmem_wait_ld();
+        // 32 columns per tensor-memory load, the next one in flight meanwhile
+        float v2[2][32];
+        tmem_ld32(tl, v2[0]);
 #pragma unroll
-          for (int hh = 0; hh < 2; ++hh) store16w(2 * c2 + hh, v2 + 16 * hh);
+        for (int c2 = 0; c2 < BN / 32; ++c2) {
+          tmem_wait_ld();
+          if (c2 + 1 < BN / 32) tmem_ld32(tl + (c2 + 1) * 32, v2[(c2 + 1) & 1]);
+#pragma unroll
+          for (int hh = 0; hh < 32 / SC; ++hh) store_cols(c2 * 32 + hh * SC, v2[c2 & 1] + SC * hh);
         }
       } else {
         epi_bar<EPI_T>();
@@ -634,15 +660,19 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
         // patched in place (a single element, below).  Each warp covers its
         // lane quarter's rows over its half of the columns.
         float rs = 0.f, rc = 0.f, crow = 0.f;
-        // 32 columns per tensor-memory load, processed as two 16-column chunks
-        for (int c2 = eh * CH2; c2 < (eh + 1) * CH2; ++c2) {
-          float v2[32];
-          tmem_ld32(tl + c2 * 32, v2);
+        // 32 columns per tensor-memory load (the next one in flight meanwhile),
+        // summed as two 16-column chunks
+        float v2[2][32];
+        tmem_ld32(tl + eh * CH2 * 32, v2[0]);
+#pragma unroll
+        for (int i2 = 0; i2 < CH2; ++i2) {
+          const int c2 = eh * CH2 + i2;
           tmem_wait_ld();
+          if (i2 + 1 < CH2) tmem_ld32(tl + (c2 + 1) * 32, v2[(i2 + 1) & 1]);
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
             const int ch = 2 * c2 + hh;
-            const float* v = v2 + 16 * hh;
+            const float* v = v2[i2 & 1] + 16 * hh;
             // row sum over the data columns: a pairwise tree over the chunk,
             // then a compensated (two-term) add of the chunk's sum; the row
             // checksum pieces sit in columns DN..DN+NPIECE-1 of the last chunk
@@ -679,9 +709,12 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
             // the column checksum pieces sit in lanes DM..DM+NPIECE-1
             if (r >= DM && r - DM < Cfg::NPIECE) {
 #pragma unroll
-              for (int e = 0; e < 16; ++e) T.ccp[r - DM][ch * 16 + e] = v[e];
+              for (int g = 0; g < 4; ++g)
+                *reinterpret_cast<float4*>(&T.ccp[r - DM][ch * 16 + 4 * g]) =
+                    make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
             }
-            store16w(ch, v);  // also the warp's column partial sums of the chunk
+            // also the warp's column partial sums
+            if (SC == 16 || hh == 1) store_cols(ch * 16 + 16 - SC, v2[i2 & 1] + (SC == 16 ? 16 * hh : 0));
           }
         }
         T.rsp[eh][r] = rs;
@@ -777,7 +810,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
           double sr = 0.0;
           for (unsigned frows = __ballot_sync(0xffffffffu, T.flag_r[r] != 0); frows; frows &= frows - 1u) {
             const int l0 = __ffs(frows) - 1;
-            float* srow = T.stg[ew][0];
+            float* srow = stg + ew * 32 * SC;
             double part = 0.0;
             for (int ch = eh * 2 * CH2; ch < (eh + 1) * 2 * CH2; ++ch) {
               float v[16];
@@ -898,7 +931,7 @@ __global__ void __launch_bounds__(TcCfg<DT, ABFT, PAIR>::THREADS, 1)
 template <int DT, bool ABFT, bool PAIR>
 cudaError_t launch_tc_impl(const TcBatch& b, const TcMapsBatch& mb, const TcRun& run, int grid, cudaStream_t st) {
   using Cfg = TcCfg<DT, ABFT, PAIR>;
-  const size_t smem = 1024 + (size_t)Cfg::STAGES * Cfg::STAGE_BYTES + sizeof(TcSmemTail);
+  const size_t smem = tc_smem_bytes<Cfg>();
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<DT, ABFT, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
