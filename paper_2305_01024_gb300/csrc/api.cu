@@ -51,7 +51,7 @@ cudaError_t launch_kmajor_operands_if(const int* gate, int epoch, const float* A
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
                                int* launches, cudaStream_t st);
 bool f32tc_scan_units(int um, int un);
-cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
+cudaError_t launch_f32tc(int bn, int tail, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]);
 int tc_nb_parts(int dt, long long K, int sub);
 int tc_enc_sub(int dt, long long K, long long tiles_n);
@@ -1451,6 +1451,7 @@ int ftgemm_gemm(ftgemm_handle_t h, int64_t m, int64_t n, int64_t k, double alpha
 struct F32TcPlan {
   int nch;                  // 32-element chunks of K
   int bn;                   // columns of a CTA pair's tile: 256 or 128
+  int tail;                 // of the 256-column tiles, those run as two of 128 after the others
   long long ldc_d, ldr_d;   // row strides of the checksum segments
   int seg, segs_per_period, segs_per_split;
   long long segs;           // over all splits
@@ -1489,14 +1490,29 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
   // rows of 128 bytes are addressed by 32-bit coordinates
   if (((long long)std::max(M, N) + 127) / 128 * t.nch * 192 > INT32_MAX) return false;
   t.bn = 128;
+  t.tail = 0;
   if (!abft || (um >= 64 && un >= 64)) {
     // waves of CTA-pair tiles times the measured SM cycles (in tens) of a chunk
     // of K: 256 x 256 tiles keep the tensor cores busier, 256 x 128 ones fill
     // a small grid (BLOCK 1024^3: 83 us on the former, 66 on the latter)
-    auto waves = [&](int bn) {
-      return (int64_t)split * (((int64_t)M + 255) / 256) * (((int64_t)N + bn - 1) / bn) + pairs - 1;
-    };
-    t.bn = waves(256) / pairs * (abft ? 210 : 156) <= waves(128) / pairs * (abft ? 127 : 107) ? 256 : 128;
+    // The last wave of the former may run as halves, in a launch of its own
+    // (some 3 us).  Without / with that, us per call, BLOCK: 4096^3 (3 waves and 28
+    // tiles) 712 / 678, 2560x2304x512 99 / 95, 2560x2304x2048 228 / 206,
+    // 3000x3500x1000 192 / 185, 5120x5120x1024 350 / 354; OFF 545 / 530, 75 / 71,
+    // 162 / 155, 138 / 135, 249 / 251.
+    auto tiles = [&](int bn) { return (int64_t)split * (((int64_t)M + 255) / 256) * (((int64_t)N + bn - 1) / bn); };
+    auto waves = [&](int64_t items) { return (items + pairs - 1) / pairs; };
+    const int64_t c256 = abft ? 210 : 156, c128 = abft ? 127 : 107, nch = t.nch;
+    const int64_t t256 = tiles(256), left = t256 % pairs;
+    int64_t best = waves(tiles(128)) * c128 * nch;
+    if (waves(t256) * c256 * nch <= best) {
+      t.bn = 256;
+      best = waves(t256) * c256 * nch;
+    }
+    if (left > 0 && t256 > left && (t256 / pairs * c256 + waves(2 * left) * c128) * nch + 600 < best) {
+      t.bn = 256;
+      t.tail = (int)left;
+    }
   }
   t.ldc_d = ((long long)N + 3) / 4 * 4;
   t.ldr_d = ((long long)M + 3) / 4 * 4;
@@ -1534,6 +1550,7 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
     if (segs > 1 && 4.0 * segs * M * t.ldp <= 536870912.0 && scan * 20 < direct * 19) {
       t.by_segments = true;
       t.bn = 128;
+      t.tail = 0;
       t.seg = seg;
       t.segs = t.segs_per_split = segs;
       if (!abft) t.segs_per_period = segs;
@@ -1593,7 +1610,7 @@ static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, doub
     if (rc) return rc;
     CK(cudaEventRecord(ev.first, h->stream));
   }
-  CK(launch_f32tc(bn, abft, maps, p, h->num_sms > 0 ? h->num_sms : 148, launches, h->stream));
+  CK(launch_f32tc(bn, t.tail, abft, maps, p, h->num_sms > 0 ? h->num_sms : 148, launches, h->stream));
   if (h->timing) {
     CK(cudaEventRecord(ev.second, h->stream));
     h->pending.push_back(ev);

@@ -40,6 +40,9 @@ struct F32TcParams {
   int M, N, K;
   int tiles_m2, tiles_n;       // CTA-pair tile rows (2 * F32TC_BM each), tile columns
   int group_m;                 // pair tile rows per raster group
+  // MAIN: tiles of the launch; half_first > 0: tiles of 256 columns from that
+  // one on, in halves of 128 (what the 256-column launch before it leaves over)
+  int tiles, half_first;
   int nsplit, k_per_split;     // splits of K and their length in elements
   int seg, segs_per_period, segs_per_split;
   // verification units and the schedule's tiling (what records and faults refer to)

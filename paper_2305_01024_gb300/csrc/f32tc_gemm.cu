@@ -171,7 +171,7 @@ __host__ __device__ __forceinline__ F32TcSums f32tc_sums(const F32TcParams& p) {
 
 template <int BN, bool SUMS>
 __device__ __forceinline__ int f32tc_items(const F32TcParams& p) {
-  if constexpr (!SUMS) return p.nsplit * p.tiles_m2 * p.tiles_n;
+  if constexpr (!SUMS) return p.tiles;
   const F32TcSums t = f32tc_sums<BN>(p);
   return p.nsplit * p.segs_per_split * (t.n[0] + t.n[1] + t.n[2]);
 }
@@ -181,6 +181,12 @@ __device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
   F32TcItem t;
   if constexpr (!SUMS) {
     const int tiles = p.tiles_m2 * p.tiles_n;
+    int width = BN, half = 0;
+    if (BN == 128 && p.half_first > 0) {
+      width = 256;
+      half = id % 2 * 128;
+      id = p.half_first + id / 2;
+    }
     t.z = id / tiles;
     id -= t.z * tiles;
     const int per_group = p.group_m * p.tiles_n, first = id / per_group * p.group_m;
@@ -188,7 +194,7 @@ __device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
     t.type = 0;
     t.seg = 0;
     t.row0 = (first + in % gsize) * 256;
-    t.col0 = in / gsize * BN;
+    t.col0 = in / gsize * width + half;
     t.k0 = t.z * p.k_per_split;
     t.klen = min(p.k_per_split, p.K - t.k0);
   } else {
@@ -764,10 +770,21 @@ static cudaError_t f32tc_launch(const F32TcMaps& maps, const F32TcParams& p, int
   return launch_pdl(f32tc_kernel<BN, ABFT, SUMS>, 2 * workers, F32TcCfg<BN>::THREADS, smem, st, maps, p);
 }
 
-// The segments (checksums; the product too if it goes by segments), then the
-// product in one pass or its scan.  bn: columns per tile.
+// The product's tiles in one pass over K.
 template <int BN>
-static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st) {
+static cudaError_t f32tc_product(bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches,
+                                 cudaStream_t st) {
+  ++*launches;
+  return abft ? f32tc_launch<BN, true, false>(maps, p, p.tiles, sms, st)
+              : f32tc_launch<BN, false, false>(maps, p, p.tiles, sms, st);
+}
+
+// The segments (checksums; the product too if it goes by segments), then the
+// product in one pass or its scan.  bn: columns per tile; tail: tiles of 256
+// columns left to a second launch.
+template <int BN>
+static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, F32TcParams p, int tail, int sms, int* launches,
+                                cudaStream_t st) {
   // the tile's shared arrays hold units of GC rows and columns or more
   if (abft && (p.um < F32TcCfg<BN>::GC || p.un < F32TcCfg<BN>::GC || p.um > 128 || p.un > 128)) return cudaErrorInvalidValue;
   if (abft || p.P) {
@@ -780,16 +797,19 @@ static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, const F32TcPar
   }
   if (p.P) return launch_f32tc_scan(abft, p, launches, st);
   const long long items = (long long)p.nsplit * p.tiles_m2 * p.tiles_n;
-  if (items > INT_MAX) return cudaErrorInvalidValue;
-  ++*launches;
-  return abft ? f32tc_launch<BN, true, false>(maps, p, (int)items, sms, st)
-              : f32tc_launch<BN, false, false>(maps, p, (int)items, sms, st);
+  if (items > INT_MAX || tail < 0 || tail >= items || (tail && BN != 256)) return cudaErrorInvalidValue;
+  p.tiles = (int)items - tail;
+  cudaError_t e = f32tc_product<BN>(abft, maps, p, sms, launches, st);
+  if (e != cudaSuccess || !tail) return e;
+  p.half_first = p.tiles;
+  p.tiles = 2 * tail;
+  return f32tc_product<128>(abft, maps, p, sms, launches, st);
 }
 
-cudaError_t launch_f32tc(int bn, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches,
-                         cudaStream_t st) {
-  return bn == 256 ? f32tc_run_bn<256>(abft, maps, p, sms, launches, st)
-                   : f32tc_run_bn<128>(abft, maps, p, sms, launches, st);
+cudaError_t launch_f32tc(int bn, int tail, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms,
+                         int* launches, cudaStream_t st) {
+  return bn == 256 ? f32tc_run_bn<256>(abft, maps, p, tail, sms, launches, st)
+                   : f32tc_run_bn<128>(abft, maps, p, tail, sms, launches, st);
 }
 
 }  // namespace ftg
