@@ -1594,6 +1594,7 @@ static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, doub
   p.m_tb = s.m_tb; p.n_tb = s.n_tb; p.k_tb = s.k_tb;
   p.tiles_n_sched = tiles_n; p.ks_per_split = ks_per_split; p.cadence = std::max(1, std::min(cadence, ks_per_split)); p.ksteps = ksteps;
   p.nA = e.nA; p.nB = e.nB; p.sq16a = e.sq16a; p.sq16b = e.sq16b;
+  p.pa = abft ? e.pa : nullptr; p.pb = abft ? e.pb : nullptr;
   p.Dc = abft ? Dc : nullptr; p.Dr = abft ? Dr : nullptr; p.P = t.by_segments ? P : nullptr; p.ldp = t.ldp;
   p.ldc_d = t.ldc_d; p.ldr_d = t.ldr_d;
   p.lam_u = (float)(h->lambda * std::ldexp(1.0, -24));

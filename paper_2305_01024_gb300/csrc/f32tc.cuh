@@ -49,8 +49,11 @@ struct F32TcParams {
   int um, un;                  // unit rows / columns (powers of two, 16 .. 128)
   int nv, nw;                  // units along M and N
   int m_tb, n_tb, k_tb, tiles_n_sched, ks_per_split, cadence, ksteps;
-  const float* nA; const float* nB;      // row norms of A, column norms of B
-  const float* sq16a; const float* sq16b;  // sums of squares of every 16 rows of A / columns of B
+  float* nA; float* nB;        // row norms of A, column norms of B
+  float* sq16a; float* sq16b;  // sums of squares of every 16 rows of A / columns of B
+  // what the SUMS launch forms them from: squared-norm partials
+  // [ceil(K / 128)][M] and [ceil(K / 128)][N], or null (no checksums)
+  const float* pa; const float* pb;
   float* Dc; float* Dr;        // checksum segments: [seg][nv][ldc_d] and [seg][nw][ldr_d]
   long long ldc_d, ldr_d;
   // the product itself by segments, [seg][M][ldp] (f32tc_scan.cu adds them

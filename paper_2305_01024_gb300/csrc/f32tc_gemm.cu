@@ -49,8 +49,9 @@ struct F32TcCfg {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = 4;
   static constexpr int NBUF = 512 / BN;                  // tensor-memory accumulators
-  // warps: TMA, MMA, two idle (register hand-over works on groups of four),
-  // then the epilogue's, EW / 4 per tensor-memory lane quarter
+  // warps: TMA, MMA, two more (the SUMS launch's norms; register hand-over
+  // works on groups of four), then the epilogue's, EW / 4 per tensor-memory
+  // lane quarter
   static constexpr int EW0 = 4, EW = BN == 256 ? 16 : 8, EPI_T = 32 * EW, THREADS = 32 * (EW0 + EW);
   static constexpr int CPT = BN / (EW / 4);              // columns per epilogue warp
   static constexpr int GC = BN == 256 ? 64 : 16;         // columns per row partial: the smallest unit
@@ -217,6 +218,32 @@ __device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
   return t;
 }
 
+// Norms from the encode pass's squared partials, a line (row of A, column of B)
+// per lane, and the sums of squares of each 16 lines; eight partial sums a line
+// in a fixed order, so results repeat.  Two warps of every CTA of the SUMS launch,
+// which have nothing else to do: a kernel of its own took 6-14 us of every call
+// (256 .. 4096 rows) before the checksum products could start.
+__device__ __forceinline__ void f32tc_norms(const F32TcParams& p, int w, int nw, int lane) {
+  const int ga = (p.M + 31) / 32, gb = (p.N + 31) / 32, parts = (p.K + 127) / 128;
+  for (int g = w; g < ga + gb; g += nw) {
+    const bool side_a = g < ga;
+    const int L = side_a ? p.M : p.N, line = (side_a ? g : g - ga) * 32 + lane;
+    const float* part = (side_a ? p.pa : p.pb) + line;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (line < L) {
+      for (int c = 0; c < parts; c += 8)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c + u < parts) s[u] += part[(long long)(c + u) * L];
+    }
+    float t = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+    if (line < L) (side_a ? p.nA : p.nB)[line] = sqrtf(t);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (line < L && lane % 16 == 0) (side_a ? p.sq16a : p.sq16b)[line / 16] = t;
+  }
+}
+
 template <int BN, bool ABFT, bool SUMS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREADS, 1)
     f32tc_kernel(const __grid_constant__ F32TcMaps maps, const __grid_constant__ F32TcParams p) {
@@ -224,7 +251,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
   constexpr int S = Cfg::STAGES, NBUF = Cfg::NBUF, CPT = Cfg::CPT, KC = Cfg::KC, EPI_T = Cfg::EPI_T;
   pdl_wait();
   pdl_trigger();
-  if (*p.bad == p.epoch) return;  // an operand outside the split's range: the CUDA-core kernel runs instead
+  if (*p.bad == p.epoch) {  // an operand outside the split's range: the CUDA-core kernel runs instead
+    if (SUMS && p.pa && threadIdx.x / 32 - 2 < 2u)  // (with the same norms)
+      f32tc_norms(p, blockIdx.x * 2 + threadIdx.x / 32 - 2, gridDim.x * 2, threadIdx.x & 31);
+    return;
+  }
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = smem_raw + (-smem_u32(smem_raw) & 1023u);  // (shared address space kept)
   F32TcTail<BN>& T = *reinterpret_cast<F32TcTail<BN>*>(base + S * Cfg::STAGE_BYTES);
@@ -298,6 +329,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     // let the last loads land before the CTAs may exit (bounded)
     if (leader)
       for (uint32_t q = it > (uint32_t)S ? it - S : 0; q < it; ++q) mbar_wait(&T.full[q % S], (q / S) & 1u);
+  } else if (SUMS && warp >= 2) {
+    if (p.pa) f32tc_norms(p, blockIdx.x * 2 + warp - 2, gridDim.x * 2, lane);
   } else if (warp == 1 && lane == 0 && leader) {
     // ---- MMA issuer: per chunk the six plane products, smallest first ----
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((256u >> 4) << 24);

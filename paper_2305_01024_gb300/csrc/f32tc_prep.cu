@@ -204,41 +204,6 @@ __global__ void __launch_bounds__(256) f32tc_split_kernel(const float* __restric
   store_planes8(P + row_unit(unit, k, nch), F32TC_APLANE, s);
 }
 
-// Norms from the squared partials, 16 lines (rows of A, then columns of B)
-// per block and 64 threads a line, and the sums of squares of each 16 lines.
-// Fixed-order sums: results repeat.
-__global__ void __launch_bounds__(1024) f32tc_norms_kernel(const float* __restrict__ pa, int na_parts, int M,
-                                                           const float* __restrict__ pb, int nb_parts, int N,
-                                                           float* __restrict__ nA, float* __restrict__ nB,
-                                                           float* __restrict__ sq16a, float* __restrict__ sq16b) {
-  __shared__ float red[32][16];
-  pdl_wait();
-  pdl_trigger();
-  const int ba = (M + 15) / 16;
-  const bool side_a = (int)blockIdx.x < ba;
-  const int b = side_a ? blockIdx.x : blockIdx.x - ba;
-  const int L = side_a ? M : N, parts = side_a ? na_parts : nb_parts;
-  const float* part = side_a ? pa : pb;
-  const int l = threadIdx.x & 15, slice = threadIdx.x >> 4, line = b * 16 + l;
-  float s = 0.f;
-  if (line < L) {
-#pragma unroll 4
-    for (int c = slice; c < parts; c += 64) s += part[(long long)c * L + line];
-  }
-  s += __shfl_xor_sync(0xffffffffu, s, 16);
-  if ((threadIdx.x & 31) < 16) red[threadIdx.x >> 5][l] = s;
-  __syncthreads();
-  if (threadIdx.x >= 32) return;
-  float t = 0.f;
-#pragma unroll
-  for (int w = 0; w < 32; ++w) t += red[w][l];
-  if (threadIdx.x < 16 && line < L) (side_a ? nA : nB)[line] = sqrtf(t);
-  float f = line < L ? t : 0.f;
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-  if (threadIdx.x == 0) (side_a ? sq16a : sq16b)[b] = f;
-}
-
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
                                int* launches, cudaStream_t st) {
   const int veca = lda % 4 == 0 && ((uintptr_t)A & 15) == 0, vecb = ldb % 4 == 0 && ((uintptr_t)B & 15) == 0;
@@ -247,11 +212,6 @@ cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, lo
   if (ab + bb > 0x7fffffff) return cudaErrorInvalidValue;
   cudaError_t er = launch_pdl(f32tc_split_kernel, (unsigned)(ab + bb), 256, 0, st, A, lda, B, ldb, e, veca, vecb, (int)ab);
   *launches += 1;
-  if (er == cudaSuccess && e.um) {
-    er = launch_pdl(f32tc_norms_kernel, (e.M + 15) / 16 + (e.N + 15) / 16, 1024, 0, st, e.pa, kgroups, e.M, e.pb, kgroups,
-                    e.N, e.nA, e.nB, e.sq16a, e.sq16b);
-    *launches += 1;
-  }
   return er;
 }
 
