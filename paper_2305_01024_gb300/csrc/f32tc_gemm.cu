@@ -40,7 +40,7 @@ cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cu
 // What bounds it at BN = 256: the tensor cores without checksums (16384^3
 // 29.4-30.6 ms, 290 TFLOP/s = 1740 of bf16 MMAs, the power cap); with block
 // checksums the verification, which stops the MMAs once both accumulators are
-// full (34-36 ms; the CUDA-core kernel 133.8).
+// full (33.3-35 ms; the CUDA-core kernel 133.8).
 template <int BN>
 struct F32TcCfg {
   static constexpr int BM = F32TC_BM, KC = F32TC_KC;
@@ -49,8 +49,7 @@ struct F32TcCfg {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = 4;
   static constexpr int NBUF = 512 / BN;                  // tensor-memory accumulators
-  // warps: TMA, MMA, two more (the SUMS launch's norms; register hand-over
-  // works on groups of four), then the epilogue's, EW / 4 per tensor-memory
+  // warps: TMA, MMA, two that keep the checksums (the SUMS launch: norms), then the epilogue's, EW / 4 per tensor-memory
   // lane quarter
   static constexpr int EW0 = 4, EW = BN == 256 ? 16 : 8, EPI_T = 32 * EW, THREADS = 32 * (EW0 + EW);
   static constexpr int CPT = BN / (EW / 4);              // columns per epilogue warp
@@ -76,11 +75,11 @@ struct F32TcTail {
   float rowpart[BN / Cfg::GC][128];     // row sums of GC columns
   double sum64[Cfg::MAXE];
   uint8_t eflag[Cfg::MAXE];
-  float c[Cfg::MAXE];                   // running checksums: rows per column unit, then columns per row unit
-  float d[Cfg::MAXE];                   // the coming period's checksum segments, copied ahead
+  float c[Cfg::MAXE];                   // checksums at the end of the period: rows per column unit, then columns per row unit
   float tn[Cfg::MAXE];                  // norm term of each entry's threshold
   float sFA[128 / Cfg::GC], sFB[BN / Cfg::GC];
   uint64_t full[Cfg::STAGES], empty[Cfg::STAGES], acc_full[Cfg::NBUF], acc_empty[Cfg::NBUF];
+  uint64_t chk_full, chk_empty;         // c (and tn) of a period ready, verified
   unsigned long long bestr[Cfg::MAXU], bestc[Cfg::MAXU];
   double fix_delta[Cfg::MAXU];
   int nr[Cfg::MAXU], nc[Cfg::MAXU], fix_row[Cfg::MAXU], fix_col[Cfg::MAXU];
@@ -276,6 +275,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       mbar_init(&T.acc_full[a], 1);
       mbar_init(&T.acc_empty[a], 2 * Cfg::EW);  // one arrival per epilogue warp of both CTAs
     }
+    mbar_init(&T.chk_full, 2);
+    mbar_init(&T.chk_empty, Cfg::EW);
     T.abort = 0;
     fence_mbar_init();
   }
@@ -331,6 +332,88 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       for (uint32_t q = it > (uint32_t)S ? it - S : 0; q < it; ++q) mbar_wait(&T.full[q % S], (q / S) & 1u);
   } else if (SUMS && warp >= 2) {
     if (p.pa) f32tc_norms(p, blockIdx.x * 2 + warp - 2, gridDim.x * 2, lane);
+  } else if (ABFT && warp >= 2) {
+    // ---- the checksums of the epilogue's entries, a period ahead ------------
+    // Their segments of the coming period are loaded while the current one
+    // runs and added once it is verified; a tile's first period also forms the
+    // thresholds' norm terms.  Done by the epilogue itself this kept the MMAs
+    // waiting: the 256-column tiles of 8192^3 took 3.54 ms, now 3.35, those of
+    // 4096^3's three full waves 430 us, now 407.
+    const int hq = (warp - 2) * 32 + lane;
+    const int um_sh = 31 - __clz(p.um), un_sh = 31 - __clz(p.un);
+    const int nRow = 128 * (BN >> un_sh), nE = nRow + BN * (128 >> um_sh);
+    constexpr int AHEAD = 4;  // entries a thread loads ahead (more would spill)
+    uint32_t checks = 0;
+    bool dead = false;
+    auto both = [] { asm volatile("bar.sync 2, 64;" ::: "memory"); };
+    for (int id = worker; id < items; id += workers) {
+      const F32TcItem x = f32tc_item<BN, SUMS>(p, id);
+      const int row0 = x.row0 + rank * 128, col0 = x.col0;
+      const int ks0 = x.z * p.ks_per_split, nks = min(p.ks_per_split, p.ksteps - ks0);
+      // Frobenius norms of the units' rows and columns
+      auto fro = [](const float* sq16, int first, int per, int count) {
+        float s = 0.f;
+        for (int g = 0; g < per && first + g < count; ++g) s += sq16[first + g];
+        return sqrtf(s);
+      };
+      both();  // the other warp is done with the tile before
+      if (hq < 128 >> um_sh) T.sFA[hq] = fro(p.sq16a, row0 / 16 + hq * (p.um / 16), p.um / 16, (p.M + 15) / 16);
+      if (hq < BN >> un_sh) T.sFB[hq] = fro(p.sq16b, col0 / 16 + hq * (p.un / 16), p.un / 16, (p.N + 15) / 16);
+      both();
+      for (int period = 0, done = 0; done < nks; ++period, done += p.cadence) {
+        // segment g of this period at entry e: its address (null outside the
+        // matrix) for g = 0 and the distance to the next
+        const int s0 = x.z * p.segs_per_split + period * p.segs_per_period;
+        auto seg_of = [&](int e, long long* stride) -> const float* {
+          if (e < nRow) {
+            const int J = (col0 >> un_sh) + (e >> 7), gr = row0 + (e & 127);
+            *stride = (long long)p.nw * p.ldr_d;
+            return J < p.nw && gr < p.M ? p.Dr + ((long long)s0 * p.nw + J) * p.ldr_d + gr : nullptr;
+          }
+          const int I = (row0 >> um_sh) + (e - nRow) / BN, gc = col0 + (e - nRow) % BN;
+          *stride = (long long)p.nv * p.ldc_d;
+          return I < p.nv && gc < p.N ? p.Dc + ((long long)s0 * p.nv + I) * p.ldc_d + gc : nullptr;
+        };
+        const int segs = min(p.segs_per_period, p.segs_per_split - period * p.segs_per_period);
+        auto first = [&](int e) {
+          long long stride;
+          const float* src = e < nE ? seg_of(e, &stride) : nullptr;
+          return src ? __ldg(src) : 0.f;
+        };
+        auto enter = [&](int e, float d) {  // entry e, d its first segment
+          float c = (period > 0 ? T.c[e] : 0.f) + d;
+          if (segs > 1) {  // periods longer than a segment
+            long long stride;
+            const float* src = seg_of(e, &stride);
+            for (int g = 1; src && g < segs; ++g) c += __ldg(src + g * stride);
+          }
+          T.c[e] = c;
+          if (period == 0) {
+            // lambda * u times the norms, rounded as ft_tau does
+            const int gr = row0 + (e & 127), gc = col0 + (e - nRow) % BN;
+            T.tn[e] = e < nRow ? __fmul_rn(__fmul_rn(p.lam_u, gr < p.M ? p.nA[gr] : 0.f), T.sFB[e >> 7])
+                               : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), gc < p.N ? p.nB[gc] : 0.f);
+          }
+        };
+        float d[AHEAD];
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) d[i] = first(hq + 64 * i);
+        if (checks > 0 && !dead && !mbar_wait(&T.chk_empty, (checks - 1) & 1u)) {
+          dead = true;
+          atomicExch(&T.abort, 1);
+        }
+#pragma unroll 1
+        for (int e = hq; e < nE; e += 64) {
+          enter(e, d[0]);
+#pragma unroll
+          for (int i = 1; i < AHEAD; ++i) d[i - 1] = d[i];
+          d[AHEAD - 1] = first(e + 64 * AHEAD);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&T.chk_full);
+        ++checks;
+      }
+    }
   } else if (warp == 1 && lane == 0 && leader) {
     // ---- MMA issuer: per chunk the six plane products, smallest first ----
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((256u >> 4) << 24);
@@ -389,7 +472,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     constexpr int NJ = CPT / 8;
     const int lq = warp & 3, eh = (warp - Cfg::EW0) >> 2, q = (warp - Cfg::EW0) * 32 + lane;
     const int rbase = lq * 32 + (lane >> 2), cbase = eh * CPT + 2 * (lane & 3);
-    uint32_t it = 0;
+    uint32_t it = 0, checks = 0;
     bool dead = false;
     float acc[4][NJ][2];
     // Hand a chunk's accumulator back to the MMA thread (in the leader CTA).
@@ -433,10 +516,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       const int ks0 = x.z * p.ks_per_split, ks1 = min(ks0 + p.ks_per_split, p.ksteps);
       const int um_sh = 31 - __clz(p.um), un_sh = 31 - __clz(p.un);
       const int nRow = ABFT ? 128 * (BN >> un_sh) : 0, nE = ABFT ? nRow + BN * (128 >> um_sh) : 0;
-      int period = 0, next_ks = INT_MAX;  // next_ks: k-step that ends the current period
+      // the k-step that ends the current period, and the elements of K up to it
+      int period = 0, next_ks = INT_MAX, k_end = INT_MAX;
       bool has_fault = false;
       if constexpr (!SUMS) {
         next_ks = min(ks0 + (ABFT ? p.cadence : p.ks_per_split), ks1) - 1;
+        k_end = min(x.klen, (next_ks + 1 - ks0) * p.k_tb);
         if (p.nfaults > 0) {
           // any scheduled fault in the schedule tiles this CTA tile covers?
           const int tm0 = row0 / p.m_tb, tn0 = col0 / p.n_tb;
@@ -450,50 +535,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           }
           has_fault = __any_sync(0xffffffffu, mine);
         }
-      }
-      // the checksum segment g of the current period at entry e: its address
-      // (null outside the matrix) for g = 0 and the distance to the next
-      auto seg_of = [&](int e, long long* stride) -> const float* {
-        const int s0 = x.z * p.segs_per_split + period * p.segs_per_period;
-        if (e < nRow) {
-          const int J = (col0 >> un_sh) + (e >> 7), gr = row0 + (e & 127);
-          *stride = (long long)p.nw * p.ldr_d;
-          return J < p.nw && gr < p.M ? p.Dr + ((long long)s0 * p.nw + J) * p.ldr_d + gr : nullptr;
-        }
-        const int I = (row0 >> um_sh) + (e - nRow) / BN, gc = col0 + (e - nRow) % BN;
-        *stride = (long long)p.nv * p.ldc_d;
-        return I < p.nv && gc < p.N ? p.Dc + ((long long)s0 * p.nv + I) * p.ldc_d + gc : nullptr;
-      };
-      // start copying the first segment of the current period for this
-      // thread's entries; it lands while the period's MMAs run
-      auto fetch_segments = [&]() {
-        for (int e = q; e < nE; e += EPI_T) {
-          long long stride;
-          const float* src = seg_of(e, &stride);
-          if (src)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(&T.d[e])), "l"(src) : "memory");
-          else
-            T.d[e] = 0.f;
-        }
-      };
-      if constexpr (ABFT) {
-        // Frobenius norms of the units' rows and columns
-        auto fro = [](const float* sq16, int first, int per, int count) {
-          float s = 0.f;
-          for (int g = 0; g < per && first + g < count; ++g) s += sq16[first + g];
-          return sqrtf(s);
-        };
-        if (q < 128 >> um_sh) T.sFA[q] = fro(p.sq16a, row0 / 16 + q * (p.um / 16), p.um / 16, (p.M + 15) / 16);
-        if (q < BN >> un_sh) T.sFB[q] = fro(p.sq16b, col0 / 16 + q * (p.un / 16), p.un / 16, (p.N + 15) / 16);
-        bar_red_or(1, EPI_T, 0);
-        for (int e = q; e < nE; e += EPI_T) {
-          T.c[e] = 0.f;
-          // lambda * u times the norms, rounded as ft_tau does
-          const int gr = row0 + (e & 127), gc = col0 + (e - nRow) % BN;
-          T.tn[e] = e < nRow ? __fmul_rn(__fmul_rn(p.lam_u, gr < p.M ? p.nA[gr] : 0.f), T.sFB[e >> 7])
-                             : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), gc < p.N ? p.nB[gc] : 0.f);
-        }
-        fetch_segments();
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -534,10 +575,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
         if (lane == 0) acc_release(ab);
 
         if constexpr (!SUMS) {
-          // the last schedule k-step complete after this chunk
-          const int done = k + KC >= x.klen ? ks1 - 1 : ks0 + (k + KC) / p.k_tb - 1;
-          if (done < next_ks) continue;
+          if (k + KC < k_end) continue;
           const int ks = next_ks, ks_first = ks0 + period * (ABFT ? p.cadence : p.ks_per_split);
+          if constexpr (ABFT) {  // the checksums through this period
+            if (!dead && !mbar_wait(&T.chk_full, checks & 1u)) {
+              dead = true;
+              atomicExch(&T.abort, 1);
+            }
+            ++checks;
+          }
           // ----- faults scheduled in this period (Section 5.3): additive
           // offsets on the accumulators or the running checksums -----
           if (has_fault) {
@@ -569,18 +615,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
             // ----- verification: partial sums of GC columns of each row and
             // of GR rows of each column -----
             constexpr int GC = Cfg::GC, GR = Cfg::GR;
-            // this thread's running checksums through the period
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            const int segs = min(p.segs_per_period, p.segs_per_split - period * p.segs_per_period);
-            for (int e = q; e < nE; e += EPI_T) {
-              float c = T.c[e] + T.d[e];
-              if (segs > 1) {  // periods longer than a segment
-                long long stride;
-                const float* src = seg_of(e, &stride);
-                for (int g = 1; src && g < segs; ++g) c += __ldg(src + g * stride);
-              }
-              T.c[e] = c;
-            }
             {
               // rows: this thread's columns of each group, then its quad's
               constexpr int NG = CPT / GC, JG = GC / 8;
@@ -648,10 +682,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
               const int sh = is_row ? 7 : BN == 256 ? 8 : 7;  // entries of a line of partial sums
               const int per = is_row ? row_per : col_per, at = is_row ? e : e - nRow;
               const float* src = (is_row ? &T.rowpart[0][0] : &T.colpart[0][0]) + ((at >> sh) * per << sh) + (at & ((1 << sh) - 1));
-              float s = 0.f;
+              float w[128 / (GC < GR ? GC : GR)], s = 0.f;
 #pragma unroll
-              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g)
-                if (g < per) s += src[g << sh];
+              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) w[g] = src[(g < per ? g : 0) << sh];
+#pragma unroll
+              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) s += g < per ? w[g] : 0.f;
               if (ok && fabsf(s - c) > kScreen * tau_of(e, c)) flags |= 1u << i;
             }
             if (bar_red_or(1, EPI_T, flags != 0u)) {
@@ -757,8 +792,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           }
           ++period;
           next_ks = min(next_ks + (ABFT ? p.cadence : p.ks_per_split), ks1 - 1);
+          k_end = min(x.klen, (next_ks + 1 - ks0) * p.k_tb);
           if constexpr (ABFT) {
-            if (k + KC < x.klen) fetch_segments();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&T.chk_empty);
           }
         }
       }
