@@ -701,26 +701,75 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
                 T.nr[q] = 0; T.nc[q] = 0; T.bestr[q] = 0ull; T.bestc[q] = 0ull; T.fix_row[q] = -1;
               }
               bar_red_or(1, EPI_T, 0);
+              constexpr int RG = CPT / GC, CG = 32 / GR;  // entries of a row, of a column
+              if constexpr (BN == 128) {
+                // Which of the warp's entries are flagged first, then one at a
+                // time in a loop: a branch around every entry's own code took
+                // most of an event's time fetching code (777 x 1531 x 2049, the
+                // kernel with one fault 72 us, now 68, without 58).  256-column
+                // tiles have no registers for that.
+                unsigned rm = 0u;
 #pragma unroll
-              for (int i2 = 0; i2 < 4; ++i2) {
-                const int r = rbase + 8 * i2;
+                for (int u = 0; u < 4 * RG; ++u)
+                  rm |= (unsigned)T.eflag[((eh * CPT + GC * (u % RG)) >> un_sh) * 128 + rbase + 8 * (u / RG)] << u;
+                for (unsigned m = __reduce_or_sync(0xffffffffu, rm); m; m &= m - 1u) {
+                  const int u0 = __ffs(m) - 1;
+                  double sum = 0.0;
 #pragma unroll
-                for (int g = 0; g < CPT / GC; ++g) {
-                  const int e = ((eh * CPT + GC * g) >> un_sh) * 128 + r;
-                  if (T.eflag[e]) {
-                    double s = 0.0;
+                  for (int j = 0; j < GC / 4; ++j) {
+                    float v = 0.f;
 #pragma unroll
-                    for (int j = 0; j < GC / 8; ++j) s += (double)acc[i2][g * (GC / 8) + j][0] + (double)acc[i2][g * (GC / 8) + j][1];
-                    atomicAdd(&T.sum64[e], s);
+                    for (int u = 0; u < 4 * RG; ++u)
+                      if (u == u0) v = acc[u / RG][u % RG * (GC / 8) + j / 2][j % 2];
+                    sum += (double)v;
                   }
+#pragma unroll
+                  for (int o = 1; o < 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                  if ((rm >> u0 & 1u) && (lane & 3) == 0)
+                    atomicAdd(&T.sum64[((eh * CPT + GC * (u0 % RG)) >> un_sh) * 128 + rbase + 8 * (u0 / RG)], sum);
                 }
+                unsigned cm = 0u;
 #pragma unroll
-                for (int j = 0; j < NJ; ++j)
+                for (int u = 0; u < CG * NJ * 2; ++u)
+                  cm |= (unsigned)T.eflag[nRow + ((lq * 32 + GR * (u / (NJ * 2))) >> um_sh) * BN + cbase + u % (NJ * 2) / 2 * 8 + u % 2] << u;
+                for (unsigned m = __reduce_or_sync(0xffffffffu, cm); m; m &= m - 1u) {
+                  const int u0 = __ffs(m) - 1;
+                  double sum = 0.0;
 #pragma unroll
-                  for (int b = 0; b < 2; ++b) {
-                    const int e = nRow + (r >> um_sh) * BN + cbase + 8 * j + b;
-                    if (T.eflag[e]) atomicAdd(&T.sum64[e], (double)acc[i2][j][b]);
+                  for (int r = 0; r < GR / 8; ++r) {
+                    float v = 0.f;
+#pragma unroll
+                    for (int u = 0; u < CG * NJ * 2; ++u)
+                      if (u == u0) v = acc[u / (NJ * 2) * (GR / 8) + r][u % (NJ * 2) / 2][u % 2];
+                    sum += (double)v;
                   }
+#pragma unroll
+                  for (int o = 4; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                  if ((cm >> u0 & 1u) && lane < 4)
+                    atomicAdd(&T.sum64[nRow + ((lq * 32 + GR * (u0 / (NJ * 2))) >> um_sh) * BN + cbase + u0 % (NJ * 2) / 2 * 8 + u0 % 2], sum);
+                }
+              } else {
+#pragma unroll
+                for (int i2 = 0; i2 < 4; ++i2) {
+                  const int r = rbase + 8 * i2;
+#pragma unroll
+                  for (int g = 0; g < CPT / GC; ++g) {
+                    const int e = ((eh * CPT + GC * g) >> un_sh) * 128 + r;
+                    if (T.eflag[e]) {
+                      double s = 0.0;
+#pragma unroll
+                      for (int j = 0; j < GC / 8; ++j) s += (double)acc[i2][g * (GC / 8) + j][0] + (double)acc[i2][g * (GC / 8) + j][1];
+                      atomicAdd(&T.sum64[e], s);
+                    }
+                  }
+#pragma unroll
+                  for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                      const int e = nRow + (r >> um_sh) * BN + cbase + 8 * j + b;
+                      if (T.eflag[e]) atomicAdd(&T.sum64[e], (double)acc[i2][j][b]);
+                    }
+                }
               }
               bar_red_or(1, EPI_T, 0);
               i = 0;
