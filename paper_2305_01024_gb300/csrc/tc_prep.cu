@@ -46,13 +46,13 @@ __device__ __forceinline__ float ld_elem(const void* base, long long idx) {
 // the problem of every block of the launch (built once, at group creation);
 // otherwise the problem is found by binary search.
 // What the launch before left is waited for first.
-#define TC_BLOCK_OF(KIND)                                                  \
+#define TC_BLOCK_OF(KIND, BLOCK)                                           \
   pdl_wait();                                                              \
   pdl_trigger();                                                           \
-  const int pi = bmap ? bmap[blockIdx.x] : tc_find_block(b, KIND, blockIdx.x); \
+  const int pi = bmap ? bmap[BLOCK] : tc_find_block(b, KIND, BLOCK);       \
   const TcProblem& P = tc_problem(b, pi);                                  \
   if (P.off) return; /* skipped by a device-array rebinding: not read */   \
-  const int lb = (int)blockIdx.x - P.blk_start[KIND]
+  const int lb = (int)(BLOCK) - P.blk_start[KIND]
 
 // Eight consecutive elements of row `row` (columns c0..c0+7, zero past
 // `ncols`) as floats, and their raw codes; one vector load when aligned.
@@ -183,16 +183,14 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
   using E = typename std::conditional<DT == 0, uint16_t, uint8_t>::type;
   E* const tail = reinterpret_cast<E*>(P.Vt) + (long long)blk * TC_TAIL * P.ldk;
   float cs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  auto take = [&](const float* v, int r) {
+  auto take = [&](const float* v) {  // a row's 8 columns: into the sums, and their squares
     float sq = 0.f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       cs[e] += v[e];
       sq = fmaf(v[e], v[e], sq);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0) P.nA_part[(long long)kx * P.M + r] = sq;
+    return sq;
   };
   const int kl = k0 + lane * 8;
   if (vec_ok && !__any_sync(0xffffffffu, kl < P.K && kl + 8 > P.K)) {
@@ -211,13 +209,15 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
       for (int gi = 0; gi < GRP; ++gi)
         q[gi] = in_k ? ldraw8<DT>(P.A, P.lda, min(r0 + min(warp + 8 * (g0 + gi), DM - 1), P.M - 1), kl)
                      : make_uint4(0u, 0u, 0u, 0u);
+      float sq[GRP];
 #pragma unroll
       for (int gi = 0; gi < GRP; ++gi) {
         const int lr = warp + 8 * (g0 + gi), r = r0 + lr;
+        sq[gi] = 0.f;
         if (lr < DM && r < P.M) {
           float v[8];
           cvt8<DT>(q[gi], v);
-          take(v, r);
+          sq[gi] = take(v);
           // one 16-byte (bf16) / 8-byte (e4m3) store of the codes
           if (lr >= TC_AROWS && in_k) {
             E* dst = tail + (long long)(lr - TC_AROWS) * P.ldk + kl;
@@ -226,6 +226,21 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
           }
         }
       }
+      // the 8 rows' sums over the warp at once: halve the rows with each of
+      // three exchanges, then two more over the lanes left (9 shuffles, not 40:
+      // the pass over 128 problems' 578 MB of A 165 us, now 132)
+      static_assert(GRP == 8, "three halvings");
+#pragma unroll
+      for (int n = 4, o = 16; n > 0; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i)
+          sq[i] = (up ? sq[n + i] : sq[i]) + __shfl_xor_sync(0xffffffffu, up ? sq[i] : sq[n + i], o);
+      }
+      sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 2);
+      sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 1);
+      const int lr = warp + 8 * (g0 + (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1)), r = r0 + lr;
+      if ((lane & 3) == 0 && lr < DM && r < P.M) P.nA_part[(long long)kx * P.M + r] = sq[0];
     }
   } else {
     for (int lr = warp; lr < DM; lr += 8) {
@@ -234,7 +249,10 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
       float v[8];
       uint16_t raw[8];
       ld8<DT>(P.A, P.lda, r, k0 + lane * 8, P.K, vec_ok, v, raw);
-      take(v, r);
+      float sq = take(v);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      if (lane == 0) P.nA_part[(long long)kx * P.M + r] = sq;
       if (lr >= TC_AROWS) {
         E* dst = tail + (long long)(lr - TC_AROWS) * P.ldk;
 #pragma unroll
@@ -279,7 +297,7 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
 // K-major rows this pass ran at 3.7 TB/s at 8192^2, 73 us, bound by its
 // shared-memory loads.)
 __global__ void __launch_bounds__(256) tc_pack_b_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
-  TC_BLOCK_OF(P_ENC_B);
+  TC_BLOCK_OF(P_ENC_B, blockIdx.x);
   constexpr int KC = 64, DN = tc_dn(0, true);
   __shared__ float sqw[8][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -360,7 +378,7 @@ __global__ void __launch_bounds__(256) tc_pack_b_kernel(const __grid_constant__ 
 // columns 8l .. 8l + 7 of a k-row as two 8-byte loads (bf16) or one (e4m3).
 template <int DT, bool ABFT>
 __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
-  TC_BLOCK_OF(P_ENC_B);
+  TC_BLOCK_OF(P_ENC_B, blockIdx.x);
   using E = typename std::conditional<DT == 0, uint16_t, uint8_t>::type;
   constexpr int KC = 128 / (int)sizeof(E);
   constexpr int NBW = ABFT ? tc_dn(DT, true) : TC_BN;
@@ -532,8 +550,8 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
 // coherence ||v_I||_2 / (sqrt(|I|) ||A_I||_F) of each block (the same for
 // w_J and B_J), a feature of the learned threshold.
 template <int DT>
-__global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap, int sink) {
-  TC_BLOCK_OF(P_FIN);
+__device__ __forceinline__ void tc_norms(const TcBatch& b, const int* __restrict__ bmap, int block, int sink) {
+  TC_BLOCK_OF(P_FIN, block);
   __shared__ float red[8], red2[8];
   __shared__ float sred[8][256];
   constexpr int KC = DT == 0 ? 64 : 128;
@@ -606,8 +624,8 @@ __global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ T
 // tc_encode_a), a B tail's rows 0 .. DN - TC_BROWS - 1 the same rows of B^T
 // (tc_encode_b); those past M (N) are zeroed here; the NP pieces follow, then
 // zeros.
-__global__ void __launch_bounds__(256) tc_pieces_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
-  TC_BLOCK_OF(P_PIECES);
+__device__ __forceinline__ void tc_pieces(const TcBatch& b, const int* __restrict__ bmap, int block) {
+  TC_BLOCK_OF(P_PIECES, block);
   constexpr int NS = TC_TAIL, KPT = 8;  // k per thread: one 8-byte store per slot
   constexpr int NP = tc_npiece(1), DM = tc_dm(1, true), DN = tc_dn(1, true);
   __shared__ float red[8];
@@ -665,14 +683,15 @@ __global__ void __launch_bounds__(256) tc_pieces_kernel(const __grid_constant__ 
   for (int c = 0; c < NP; ++c) { lo4[c] = 0u; hi4[c] = 0u; }
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    float sc = s0, r = x[j];
+    float sc = s0, inv = 1.f / s0, r = x[j];  // (powers of two: a multiply is the division)
 #pragma unroll
     for (int c = 0; c < NP; ++c) {
       const __nv_fp8_storage_t qv = __nv_cvt_float_to_fp8(r * sc, __NV_SATFINITE, __NV_E4M3);
       __nv_fp8_e4m3 qq;
       qq.__x = qv;
-      r -= float(qq) / sc;
+      r -= float(qq) * inv;
       sc *= 16.f;
+      inv *= 0.0625f;
       if (j < 4) lo4[c] |= (uint32_t)qv << (8 * j);
       else hi4[c] |= (uint32_t)qv << (8 * (j - 4));
     }
@@ -687,6 +706,19 @@ __global__ void __launch_bounds__(256) tc_pieces_kernel(const __grid_constant__ 
       if (p == pc) w = make_uint2(lo4[p], hi4[p]);
     *reinterpret_cast<uint2*>(out + (long long)(blk * NS + c) * P.ldk + k0) = w;
   }
+}
+
+__global__ void __launch_bounds__(256) tc_norms_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap, int sink) {
+  tc_norms<0>(b, bmap, blockIdx.x, sink);
+}
+
+// e4m3: the norms' blocks, then the pieces'.  Neither needs the other's results
+// and both are bound by latency: in one launch the encode pass of 4096 x 4096 x
+// 8192 takes 42 us, one after the other 50.
+__global__ void __launch_bounds__(256) tc_norms_pieces_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ fmap,
+                                                              const int* __restrict__ pmap, int nfin, int sink) {
+  if ((int)blockIdx.x < nfin) tc_norms<1>(b, fmap, blockIdx.x, sink);
+  else tc_pieces(b, pmap, (int)blockIdx.x - nfin);
 }
 
 // ---- quantizer ------------------------------------------------------------
@@ -828,12 +860,10 @@ cudaError_t launch_tc_prep(int dt, bool abft, bool sink, const TcBatch& b, const
   if (e == cudaSuccess)
     e = launch_pdl(dt == 0 ? tc_encode_a_kernel<0> : tc_encode_a_kernel<1>, total[P_ENC_A], 256, 0, st, b, mp(P_ENC_A));
   if (e == cudaSuccess)
-    e = launch_pdl(dt == 0 ? tc_norms_kernel<0> : tc_norms_kernel<1>, total[P_FIN], 256, 0, st, b, mp(P_FIN), (int)sink);
+    e = dt == 0 ? launch_pdl(tc_norms_kernel, total[P_FIN], 256, 0, st, b, mp(P_FIN), (int)sink)
+                : launch_pdl(tc_norms_pieces_kernel, total[P_FIN] + total[P_PIECES], 256, 0, st, b, mp(P_FIN),
+                             mp(P_PIECES), total[P_FIN], (int)sink);
   *launches += 3;
-  if (e == cudaSuccess && dt == 1) {
-    e = launch_pdl(tc_pieces_kernel, total[P_PIECES], 256, 0, st, b, mp(P_PIECES));
-    ++*launches;
-  }
   return e;
 }
 
