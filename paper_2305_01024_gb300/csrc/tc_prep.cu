@@ -151,6 +151,21 @@ __device__ __forceinline__ void tc_pieces3(float x, uint16_t p[3]) {
   p[2] = __bfloat16_as_ushort(__float2bfloat16_rn(r1 - __bfloat162float(mid)));
 }
 
+// Eight rows' sums over the warp at once: row lane / 4's, in each lane.  Three
+// exchanges halve the rows, two add over the four lanes left (9 shuffles, not
+// 40; the same additions, so the same bits).
+__device__ __forceinline__ float rows8_sum(float* s, int lane) {
+#pragma unroll
+  for (int n = 4, o = 16; n > 0; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n; ++i)
+      s[i] = (up ? s[n + i] : s[i]) + __shfl_xor_sync(0xffffffffu, up ? s[i] : s[n + i], o);
+  }
+  s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+  return s[0] + __shfl_xor_sync(0xffffffffu, s[0], 1);
+}
+
 // A: block sums over DM-row blocks (-> Vf), squared row-norm partials over
 // 256-wide k-chunks (-> nA_part), and the copy of each block's rows
 // TC_AROWS .. DM - 1 into the first rows of its tail in Vt (the MMA reads a
@@ -226,21 +241,11 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
           }
         }
       }
-      // the 8 rows' sums over the warp at once: halve the rows with each of
-      // three exchanges, then two more over the lanes left (9 shuffles, not 40:
-      // the pass over 128 problems' 578 MB of A 165 us, now 132)
-      static_assert(GRP == 8, "three halvings");
-#pragma unroll
-      for (int n = 4, o = 16; n > 0; n >>= 1, o >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < n; ++i)
-          sq[i] = (up ? sq[n + i] : sq[i]) + __shfl_xor_sync(0xffffffffu, up ? sq[i] : sq[n + i], o);
-      }
-      sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 2);
-      sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 1);
-      const int lr = warp + 8 * (g0 + (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1)), r = r0 + lr;
-      if ((lane & 3) == 0 && lr < DM && r < P.M) P.nA_part[(long long)kx * P.M + r] = sq[0];
+      // (a reduction per row: 165 us for 128 problems' 578 MB of A, now 132)
+      static_assert(GRP == 8, "rows8_sum");
+      const float sum = rows8_sum(sq, lane);
+      const int lr = warp + 8 * (g0 + (lane >> 2)), r = r0 + lr;
+      if ((lane & 3) == 0 && lr < DM && r < P.M) P.nA_part[(long long)kx * P.M + r] = sum;
     }
   } else {
     for (int lr = warp; lr < DM; lr += 8) {
@@ -295,7 +300,8 @@ __global__ void __launch_bounds__(256) tc_encode_a_kernel(const __grid_constant_
 // as one 16-byte unit: whole 128-byte lines both ways, no transpose.
 // Bound: HBM, 4 bytes an element.  (Through a shared-memory transpose to
 // K-major rows this pass ran at 3.7 TB/s at 8192^2, 73 us, bound by its
-// shared-memory loads.)
+// shared-memory loads; with a warp reduction and its pieces per k-row 55 us, bound
+// by instructions; now 46.  128 problems, 1321 MB in and out: 204 us, 6.5 TB/s.)
 __global__ void __launch_bounds__(256) tc_pack_b_kernel(const __grid_constant__ TcBatch b, const int* __restrict__ bmap) {
   TC_BLOCK_OF(P_ENC_B, blockIdx.x);
   constexpr int KC = 64, DN = tc_dn(0, true);
@@ -329,29 +335,36 @@ __global__ void __launch_bounds__(256) tc_pack_b_kernel(const __grid_constant__ 
                           (uint32_t)raw[4] | (uint32_t)raw[5] << 16, (uint32_t)raw[6] | (uint32_t)raw[7] << 16);
       }
     }
+    float rs[8];
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
-      const int kl = warp + 8 * g, k = k0 + kl;
-      uint4 w = k < P.K ? q[g] : make_uint4(0u, 0u, 0u, 0u);
+      if (k0 + warp + 8 * g >= P.K) q[g] = make_uint4(0u, 0u, 0u, 0u);
       float v[8];
-      cvt8<0>(w, v);
-      float rs = 0.f;
+      cvt8<0>(q[g], v);
+      rs[g] = 0.f;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        rs += v[e];
+        rs[g] += v[e];
         sq[e] = fmaf(v[e], v[e], sq[e]);
       }
+    }
+    // the row sums and their pieces, k-row warp + 8 (lane / 4) in each lane; lane
+    // 31 then puts every row's beside its four data columns
+    static_assert(DN == 252, "lane 31: four data columns, three pieces, a zero");
+    const float sum = rows8_sum(rs, lane);
+    if ((lane & 3) == 0 && k0 + warp + 2 * lane < P.K) P.Wf[(long long)nb * P.ldk + k0 + warp + 2 * lane] = sum;
+    uint16_t pc[3];
+    tc_pieces3(sum, pc);
+    const uint32_t p01 = (uint32_t)pc[0] | (uint32_t)pc[1] << 16, p2 = pc[2];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
+    for (int g = 0; g < 8; ++g) {
+      const uint32_t z = __shfl_sync(0xffffffffu, p01, 4 * g), w = __shfl_sync(0xffffffffu, p2, 4 * g);
       if (lane == 31) {
-        static_assert(DN == 252, "lane 31: four data columns, three pieces, a zero");
-        uint16_t pc[3];
-        tc_pieces3(rs, pc);
-        w.z = (uint32_t)pc[0] | (uint32_t)pc[1] << 16;
-        w.w = (uint32_t)pc[2];
+        q[g].z = z;
+        q[g].w = w;
       }
-      if (lane == 0 && k < P.K) P.Wf[(long long)nb * P.ldk + k] = rs;
-      *reinterpret_cast<uint4*>(out + kl * 64 + (((lane & 7) ^ (kl & 7)) << 3)) = w;
+      const int kl = warp + 8 * g;
+      *reinterpret_cast<uint4*>(out + kl * 64 + (((lane & 7) ^ (kl & 7)) << 3)) = q[g];
     }
   }
   // each warp saw 1/8 of the block's k rows: sum the warps' column partials
@@ -404,19 +417,15 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
   const bool fast = vec_ok && !__any_sync(0xffffffffu, in_cols && c0 < P.N && c0 + 8 > P.N &&
                                                             (DT != 0 || c0 + 4 != P.N));
   float sq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  auto take = [&](const float* v, int k) {
-    if constexpr (ABFT) {
-      float rs = 0.f;
+  auto take = [&](const float* v) {  // a k-row's 8 columns: its part of the row sum
+    float rs = 0.f;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float x = e < lim ? v[e] : 0.f;  // columns of the next block do not count
-        rs += x;
-        sq[e] = fmaf(x, x, sq[e]);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-      if (lane == 0 && k < P.K) P.Wf[(long long)nb * P.ldk + k] = rs;
+    for (int e = 0; e < 8; ++e) {
+      const float x = e < lim ? v[e] : 0.f;  // columns of the next block do not count
+      rs += x;
+      sq[e] = fmaf(x, x, sq[e]);
     }
+    return rs;
   };
   E* Bt = reinterpret_cast<E*>(P.Bt);
   constexpr int EPV = 16 / (int)sizeof(E);  // elements per 16-byte vector
@@ -433,6 +442,7 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
       static_assert(RPW % GRP == 0, "row groups");
       for (int g0 = 0; g0 < RPW; g0 += GRP) {
         uint4 q[GRP];
+        [[maybe_unused]] float rs[GRP];
 #pragma unroll
         for (int gi = 0; gi < GRP; ++gi)
           q[gi] = in_cols ? ldraw8_a8_upto<DT>(P.B, P.ldb, min(k0 + warp + 8 * (g0 + gi), P.K - 1), c0, P.N)
@@ -454,9 +464,17 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
               *reinterpret_cast<uint2*>(&tile[kk][4 * word_at(kk, lane * 2)]) = make_uint2(w.x, w.y);
             }
           }
-          float v[8];
-          cvt8<DT>(w, v);
-          take(v, k);
+          if constexpr (ABFT) {
+            float v[8];
+            cvt8<DT>(w, v);
+            rs[gi] = take(v);
+          }
+        }
+        if constexpr (ABFT) {
+          static_assert(GRP == 8, "rows8_sum");
+          const float sum = rows8_sum(rs, lane);
+          const int k = k0 + warp + 8 * (g0 + (lane >> 2));
+          if ((lane & 3) == 0 && k < P.K) P.Wf[(long long)nb * P.ldk + k] = sum;
         }
       }
     } else {
@@ -473,7 +491,12 @@ __global__ void __launch_bounds__(256) tc_encode_b_kernel(const __grid_constant_
           for (int e = 0; e < 8; ++e)
             tile[kk][DT == 0 ? lane * 8 + e : 4 * word_at(kk, lane * 2 + (e >> 2)) + (e & 3)] = (E)raw[e];
         }
-        take(v, k);
+        if constexpr (ABFT) {
+          float rs = take(v);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
+          if (lane == 0 && k < P.K) P.Wf[(long long)nb * P.ldk + k] = rs;
+        }
       }
     }
     __syncthreads();
