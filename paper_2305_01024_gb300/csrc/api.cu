@@ -51,6 +51,7 @@ cudaError_t launch_kmajor_operands_if(const int* gate, int epoch, const float* A
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
                                int* launches, cudaStream_t st);
 bool f32tc_scan_units(int um, int un);
+bool f32tc_scan_groups(int M, int N, int um, int un, int periods);
 cudaError_t launch_f32tc(int bn, int tail, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
 void tc_prep_blocks(const TcProblem& P, int dt, int out[P_KINDS]);
 int tc_nb_parts(int dt, long long K, int sub);
@@ -1527,7 +1528,7 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
     // Few tiles and a long K leave most CTA pairs idle in a pass over K; the
     // segments of K run side by side and a scan adds them up.  Both routes in
     // tens of SM cycles: a chunk 107 (127 with verification), the scan 135 a
-    // segment with verification, 300 for its launch, and 21 KB of segments
+    // segment with verification (20 by shares), 300 for its launch, and 21 KB of segments
     // written and read.  Measured, us per call, one pass / by segments: BLOCK
     // 256x256x65536 1890 / 383, 512x512x8192 (32 x 32 units) 190 / 126, but
     // 777x1531x2049 114 / 125, 2543x700x3717 189 / 197; OFF 640x640x4096 98 / 53.
@@ -1545,7 +1546,8 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
     auto waves = [&](long long items) { return (items + pairs - 1) / pairs; };
     const long long per = seg / F32TC_KC;
     const long long direct = waves(tiles) * t.nch * (abft ? 127 : 107) + waves(sums * segs) * per * 107;
-    const long long scan = waves((tiles + sums) * segs) * per * 107 + (abft ? 135 : 0) * segs + 300 +
+    const bool groups = abft && f32tc_scan_groups(M, N, um, un, (segs + t.segs_per_period - 1) / t.segs_per_period);
+    const long long scan = waves((tiles + sums) * segs) * per * 107 + (!abft ? 0 : groups ? 20 : 135) * segs + 300 +
                            8LL * segs * M * N / 21000;
     if (segs > 1 && 4.0 * segs * M * t.ldp <= 536870912.0 && scan * 20 < direct * 19) {
       t.by_segments = true;

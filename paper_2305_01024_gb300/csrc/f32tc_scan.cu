@@ -5,12 +5,13 @@
 // verification unit, a warp holding a 32 x 32 (16 x 16, 16 x 32) piece of it in
 // registers; at the end of each period it injects the scheduled faults
 // (Section 5.3), verifies, locates and corrects (Section 4.2.1) exactly as the
-// one-pass kernel does, so results and records do not depend on the route.
+// one-pass kernel does.
 //
 // Bound: the chain of one period (copy, sums, barriers, comparison: 0.7 us
-// with one warp a unit); units run side by side.  256 x 256 x 65536 with 16 x 16
-// units: 182 us after 124 us for the segments; one pass over K kept 2 of 76 CTA
-// pairs busy for 1780 us.
+// with one warp a unit); units run side by side, and units of one warp walk
+// shares of their periods side by side (f32tc_scan_groups_kernel).  256 x 256 x
+// 65536 with 16 x 16 units: 50 us after 128 us for the segments; one pass over K
+// kept 2 of 76 CTA pairs busy for 1780 us.
 #include "f32tc.cuh"
 
 namespace ftg {
@@ -24,6 +25,48 @@ __device__ __forceinline__ void scan_fold(float* v, int lane, int o) {
     const float lo = v[e], hi = v[N / 2 + e];
     v[e] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
   }
+}
+
+// Row and column sums of the piece a warp holds (the layout of the kernels
+// below): rowp[UR], colp[CW].
+template <int UR, int CW>
+__device__ __forceinline__ void scan_sums(const float* acc, int lane, float* rowp, float* colp) {
+  constexpr int EPT = UR * CW / 32;
+  float t[EPT];
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) t[i] = acc[i];
+  // rows: over the CW lanes of a row
+  if constexpr (EPT == 32) {
+    scan_fold<32>(t, lane, 16);
+    scan_fold<16>(t, lane, 8);
+    scan_fold<8>(t, lane, 4);
+    scan_fold<4>(t, lane, 2);
+    scan_fold<2>(t, lane, 1);
+    rowp[lane] = t[0];
+  } else if constexpr (EPT == 16) {
+    scan_fold<16>(t, lane, 16);
+    scan_fold<8>(t, lane, 8);
+    scan_fold<4>(t, lane, 4);
+    scan_fold<2>(t, lane, 2);
+    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
+    if (!(lane & 1)) rowp[lane >> 1] = t[0];
+  } else {
+    static_assert(EPT == 8 && CW == 16, "pieces: 32 x 32, 16 x 32, 16 x 16");
+    scan_fold<8>(t, lane, 8);
+    scan_fold<4>(t, lane, 4);
+    scan_fold<2>(t, lane, 2);
+    t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
+    if (!(lane & 1)) rowp[lane / CW + 2 * ((lane & 15) >> 1)] = t[0];
+  }
+  // columns: this lane's rows (both half-warps' of a 16-wide piece)
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) t[i] = acc[i];
+#pragma unroll
+  for (int st = EPT / 2; st > 0; st >>= 1)
+#pragma unroll
+    for (int i = 0; i < st; ++i) t[i] += t[i + st];
+  if constexpr (CW == 16) t[0] += __shfl_xor_sync(0xffffffffu, t[0], 16);
+  if (lane < CW) colp[lane] = t[0];
 }
 
 struct ScanShared {
@@ -42,13 +85,15 @@ struct ScanShared {
 // through a ring of `depth` (a power of two) in shared memory, each thread
 // copying and reading its own elements (256 x 256 x 65536: 182 us against 211
 // with one segment ahead in registers).
-template <int UR, int CW>
-__global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__ F32TcParams p, int depth) {
-  if (*p.bad == p.epoch) return;
-  extern __shared__ float ring[];  // [depth][UR * CW / 32 + 2][threads]
+// WARP: one warp of a larger block runs the unit (nthr = 32), else the block.
+template <int UR, int CW, bool WARP>
+__device__ void scan_unit(const F32TcParams& p, int depth, ScanShared& X, float* ring, int tid, int nthr) {
   constexpr int EPT = UR * CW / 32, STEP = 32 / CW;
-  __shared__ ScanShared X;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
+  auto sync = [] {
+    if constexpr (WARP) __syncwarp();
+    else __syncthreads();
+  };
+  const int lane = tid & 31, warp = tid >> 5;
   const int wcols = p.un / CW, wr = warp / wcols, wc = warp - wr * wcols;
   const int I = blockIdx.x / p.nw, J = blockIdx.x - I * p.nw;
   const int row0 = I * p.um, col0 = J * p.un, ne = p.um + p.un;
@@ -64,7 +109,7 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
     X.fro[tid] = sqrtf(s);
   }
   if (tid == 0) X.reset = -1;
-  __syncthreads();
+  sync();
   // this thread's checksum entries: rows 0 .. um - 1, then columns
   const float* dsrc[2];
   long long dstride[2];
@@ -162,44 +207,8 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
       }
     }
     // ----- verification -----
-    {
-      float t[EPT];
-#pragma unroll
-      for (int i = 0; i < EPT; ++i) t[i] = acc[i];
-      // rows: over the CW lanes of a row
-      if constexpr (EPT == 32) {
-        scan_fold<32>(t, lane, 16);
-        scan_fold<16>(t, lane, 8);
-        scan_fold<8>(t, lane, 4);
-        scan_fold<4>(t, lane, 2);
-        scan_fold<2>(t, lane, 1);
-        X.rowp[wc][wr * UR + lane] = t[0];
-      } else if constexpr (EPT == 16) {
-        scan_fold<16>(t, lane, 16);
-        scan_fold<8>(t, lane, 8);
-        scan_fold<4>(t, lane, 4);
-        scan_fold<2>(t, lane, 2);
-        t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
-        if (!(lane & 1)) X.rowp[wc][wr * UR + (lane >> 1)] = t[0];
-      } else {
-        static_assert(EPT == 8 && CW == 16, "pieces: 32 x 32, 16 x 32, 16 x 16");
-        scan_fold<8>(t, lane, 8);
-        scan_fold<4>(t, lane, 4);
-        scan_fold<2>(t, lane, 2);
-        t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
-        if (!(lane & 1)) X.rowp[wc][wr * UR + rsub + 2 * ((lane & 15) >> 1)] = t[0];
-      }
-      // columns: this lane's rows (both half-warps' of a 16-wide piece)
-#pragma unroll
-      for (int i = 0; i < EPT; ++i) t[i] = acc[i];
-#pragma unroll
-      for (int st = EPT / 2; st > 0; st >>= 1)
-#pragma unroll
-        for (int i = 0; i < st; ++i) t[i] += t[i + st];
-      if constexpr (CW == 16) t[0] += __shfl_xor_sync(0xffffffffu, t[0], 16);
-      if (lane < CW) X.colp[wr][lc] = t[0];
-    }
-    __syncthreads();
+    scan_sums<UR, CW>(acc, lane, X.rowp[wc] + wr * UR, X.colp[wr] + wc * CW);
+    sync();
     const float grow = __fmul_rn(p.mu_u, sqrtf((float)min((ks + 1) * p.k_tb, p.K)));
     unsigned flags = 0u;
     float tau[2];
@@ -213,7 +222,13 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
       else for (int w = 0; w < p.um / UR; ++w) s += X.colp[w][e - p.um];
       if (fabsf(s - c[q]) > kScreen * tau[q]) flags |= 1u << q;
     }
-    if (!__syncthreads_or(flags != 0u)) continue;
+    bool any;
+    if constexpr (WARP) any = __any_sync(0xffffffffu, flags != 0u);
+    else any = __syncthreads_or(flags != 0u);
+    if (!any) {
+      if constexpr (WARP) __syncwarp();
+      continue;
+    }
     // ----- fp64 confirmation of the screened entries -----
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -226,13 +241,13 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
     if (tid == 0) {
       X.nr = 0; X.nc = 0; X.bestr = 0ull; X.bestc = 0ull; X.fix_row = -1; X.reset = -1;
     }
-    __syncthreads();
+    sync();
 #pragma unroll
     for (int i = 0; i < EPT; ++i) {
       if (X.flag[lrow(i)]) atomicAdd(&X.sum64[lrow(i)], (double)acc[i]);
       if (X.flag[p.um + lc]) atomicAdd(&X.sum64[p.um + lc], (double)acc[i]);
     }
-    __syncthreads();
+    sync();
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int e = tid + q * nthr;
@@ -248,7 +263,7 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
         atomicMax(&X.bestc, flag_key(sc, e - p.um));
       }
     }
-    __syncthreads();
+    sync();
     if (tid == 0 && (X.nr | X.nc)) {
       const int nr = X.nr, nc = X.nc;
       const int ir = nr ? key_index(X.bestr) : -1, jc = nc ? key_index(X.bestc) : -1, ec = p.um + jc;
@@ -278,7 +293,7 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
       }
       report_event(p.rep, p.recs, rec);
     }
-    __syncthreads();
+    sync();
     // ----- correct the located element, or reset the checksum -----
 #pragma unroll
     for (int i = 0; i < EPT; ++i)
@@ -286,7 +301,7 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
 #pragma unroll
     for (int q = 0; q < 2; ++q)
       if (tid + q * nthr == X.reset) c[q] = X.reset_value;
-    __syncthreads();  // the shared state is reused
+    sync();  // the shared state is reused
   }
   if (!col_ok) return;
   float* out = p.C + (long long)row0 * p.ldc + col0 + lc;
@@ -296,6 +311,144 @@ __global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__
     float* d = out + (long long)lrow(i) * p.ldc;
     const float v = p.alpha * acc[i];
     *d = p.beta != 0.f ? fmaf(p.beta, *d, v) : v;
+  }
+}
+
+template <int UR, int CW>
+__global__ void __launch_bounds__(512) f32tc_scan_kernel(const __grid_constant__ F32TcParams p, int depth) {
+  if (*p.bad == p.epoch) return;
+  extern __shared__ float ring[];  // [depth][UR * CW / 32 + 2][threads]
+  __shared__ ScanShared X;
+  scan_unit<UR, CW, false>(p, depth, X, ring, threadIdx.x, blockDim.x);
+}
+
+// Units of one warp and many periods: a block per unit, SCAN_GROUPS warps with
+// a share of the periods each.  A warp first adds up its segments, then starts
+// from the sums of the shares before its own and walks its periods again,
+// screening each as scan_unit does; the segments come from L2 the second time.
+// Where a fault is scheduled, or anything was flagged (nothing has been written
+// then), one warp runs the unit from the start, period by period.
+// Bound: the chain of one period, SCAN_GROUPS of them side by side.  One warp a
+// unit / this, us: 256 x 256 x 65536 with 16 x 16 units 182 / 50, with 32 x 32
+// 306 / 92; 384 x 384 x 16384 (32 x 32) 82 / 30; at 16 periods 512 x 512 x 4096
+// (16 x 16) 16 / 17, 640 x 384 x 4096 (32 x 32) 24 / 19.
+constexpr int SCAN_GROUPS = 8;
+template <int UR, int CW>
+__global__ void __launch_bounds__(32 * SCAN_GROUPS) f32tc_scan_groups_kernel(const __grid_constant__ F32TcParams p, int depth) {
+  if (*p.bad == p.epoch) return;
+  constexpr int EPT = UR * CW / 32, STEP = 32 / CW, G = SCAN_GROUPS, NV = EPT + 2;
+  extern __shared__ float ring[];  // [depth][NV][32]
+  __shared__ ScanShared X;
+  __shared__ float pre[G - 1][NV][32], rowp[G][UR], colp[G][CW];
+  const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
+  const int I = blockIdx.x / p.nw, J = blockIdx.x - I * p.nw, row0 = I * UR, col0 = J * CW;
+  const int lc = lane % CW;
+  auto lrow = [&](int i) { return lane / CW + STEP * i; };
+  const bool col_ok = col0 + lc < p.N;
+  if (tid < 2) {  // Frobenius norms of the unit's rows and columns
+    const float* sq = (tid ? p.sq16b : p.sq16a) + (tid ? col0 : row0) / 16;
+    const int cnt = min((tid ? CW : UR) / 16, ((tid ? p.N - col0 : p.M - row0) + 15) / 16);
+    float s = 0.f;
+    for (int i = 0; i < cnt; ++i) s += sq[i];
+    X.fro[tid] = sqrtf(s);
+  }
+  __syncthreads();
+  // this lane's checksum entries: rows 0 .. UR - 1, then columns
+  const float* dsrc[2];
+  long long dstride[2];
+  float tn[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int e = lane + 32 * q;
+    tn[q] = 0.f;
+    dsrc[q] = nullptr;
+    dstride[q] = 0;
+    if (e < UR) {
+      if (row0 + e < p.M) {
+        dsrc[q] = p.Dr + (long long)J * p.ldr_d + row0 + e;
+        dstride[q] = (long long)p.nw * p.ldr_d;
+        tn[q] = __fmul_rn(__fmul_rn(p.lam_u, p.nA[row0 + e]), X.fro[1]);
+      }
+    } else if (e < UR + CW && col0 + e - UR < p.N) {
+      dsrc[q] = p.Dc + (long long)I * p.ldc_d + col0 + e - UR;
+      dstride[q] = (long long)p.nv * p.ldc_d;
+      tn[q] = __fmul_rn(__fmul_rn(p.lam_u, X.fro[0]), p.nB[col0 + e - UR]);
+    }
+  }
+  const int tile = row0 / p.m_tb * p.tiles_n_sched + col0 / p.n_tb;
+  const int f0 = p.nfaults > 0 ? first_fault(p.faults, p.nfaults, tile) : 0;
+  if (f0 < p.nfaults && p.faults[f0].tile == tile) {
+    if (g == 0) scan_unit<UR, CW, true>(p, depth, X, ring, lane, 32);
+    return;
+  }
+  bool redo = false;
+
+  // this warp's periods and segments
+  const int segs = p.segs_per_split, spp = p.segs_per_period;
+  const int share = ((segs + spp - 1) / spp + G - 1) / G;
+  const int s0 = min((long long)segs, (long long)g * share * spp), s1 = min((long long)segs, (long long)(g + 1) * share * spp);
+  const float* src = p.P + (long long)row0 * p.ldp + col0 + lc;
+  const long long seg_step = (long long)p.M * p.ldp;
+  auto load = [&](int seg, float* v) {
+#pragma unroll
+    for (int i = 0; i < EPT; ++i)
+      v[i] = col_ok && row0 + lrow(i) < p.M ? __ldg(src + seg * seg_step + lrow(i) * p.ldp) : 0.f;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) v[EPT + q] = dsrc[q] ? __ldg(dsrc[q] + seg * dstride[q]) : 0.f;
+  };
+  float acc[NV], v[NV];  // the piece, then this lane's checksums
+#pragma unroll
+  for (int i = 0; i < NV; ++i) acc[i] = 0.f;
+  if (g < G - 1) {
+#pragma unroll 4
+    for (int seg = s0; seg < s1; ++seg) {
+      load(seg, v);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) acc[i] += v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      pre[g][i][lane] = acc[i];
+      acc[i] = 0.f;
+    }
+  }
+  if (s0 < s1) load(s0, v);
+  __syncthreads();
+  for (int h = 0; h < g; ++h)
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] += pre[h][i][lane];
+  for (int seg = s0, left = spp, period = g * share; seg < s1; ++seg) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) acc[i] += v[i];
+    if (seg + 1 < s1) load(seg + 1, v);
+    if (--left > 0 && seg + 1 < segs) continue;
+    left = spp;
+    const int ks = min((period + 1) * p.cadence, p.ksteps) - 1;
+    ++period;
+    scan_sums<UR, CW>(acc, lane, rowp[g], colp[g]);
+    __syncwarp();
+    const float grow = __fmul_rn(p.mu_u, sqrtf((float)min((ks + 1) * p.k_tb, p.K)));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int e = lane + 32 * q;
+      if (e >= UR + CW) continue;
+      const float c = acc[EPT + q], sum = e < UR ? rowp[g][e] : colp[g][e - UR];
+      redo |= fabsf(sum - c) > kScreen * __fmaf_rn(grow, fabsf(c), tn[q]);
+    }
+    __syncwarp();
+  }
+  if (__syncthreads_or(redo)) {
+    if (g == 0) scan_unit<UR, CW, true>(p, depth, X, ring, lane, 32);
+    return;
+  }
+  if (s0 >= s1 || s1 < segs || !col_ok) return;  // the last share's warp holds the result
+  float* out = p.C + (long long)row0 * p.ldc + col0 + lc;
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) {
+    if (row0 + lrow(i) >= p.M) continue;
+    float* d = out + (long long)lrow(i) * p.ldc;
+    const float o = p.alpha * acc[i];
+    *d = p.beta != 0.f ? fmaf(p.beta, *d, o) : o;
   }
 }
 
@@ -325,6 +478,14 @@ bool f32tc_scan_units(int um, int un) {
   return (um == 16 && un >= 16 && un <= 128) || (um >= 32 && un >= 32 && um <= 128 && un <= 128);
 }
 
+// Units of one warp, few enough that one warp each leaves the GPU idle, with
+// enough periods for shares.  One warp a unit / shares, us: 512 x 512 x 8192 with
+// 32 x 32 units 45 / 31, with 16 x 16 29 / 25; but 640 x 640 x 4096 (32 x 32) 26 /
+// 36, 1024 x 512 x 4096 (16 x 16) 19 / 32, 1024 x 1024 x 8192 (32 x 32) 57 / 112.
+bool f32tc_scan_groups(int M, int N, int um, int un, int periods) {
+  return um <= 32 && un <= 32 && (long long)M * N <= 1 << 18 && periods >= 2 * SCAN_GROUPS;
+}
+
 cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cudaStream_t st) {
   ++*launches;
   if (!abft) {
@@ -336,18 +497,23 @@ cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cu
   const int ur = p.um < 32 ? p.um : 32, cw = p.un < 32 ? p.un : 32, threads = p.um / ur * (p.un / cw) * 32;
   const int depth = p.um * p.un <= 4096 ? 4 : 2;
   const size_t smem = sizeof(float) * depth * (ur * cw / 32 + 2) * threads;  // at most 139,264 bytes (128 x 128)
-  auto go = [&](auto* k) {
+  auto go = [&](auto* k, int block) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // an ordinary launch: scheduled while the GEMM kernel drains, the small
     // blocks gather on the SMs that are free first (253 us against 182 for
-    // 256 x 256 x 65536)
-    k<<<units, threads, smem, st>>>(p, depth);
+    // 256 x 256 x 65536 with one warp a unit)
+    k<<<units, block, smem, st>>>(p, depth);
     return cudaGetLastError();
   };
-  if (ur == 32) return go(f32tc_scan_kernel<32, 32>);
-  if (cw == 32) return go(f32tc_scan_kernel<16, 32>);
-  return go(f32tc_scan_kernel<16, 16>);
+  if (f32tc_scan_groups(p.M, p.N, p.um, p.un, (p.segs_per_split + p.segs_per_period - 1) / p.segs_per_period)) {
+    if (ur == 32) return go(f32tc_scan_groups_kernel<32, 32>, 32 * SCAN_GROUPS);
+    if (cw == 32) return go(f32tc_scan_groups_kernel<16, 32>, 32 * SCAN_GROUPS);
+    return go(f32tc_scan_groups_kernel<16, 16>, 32 * SCAN_GROUPS);
+  }
+  if (ur == 32) return go(f32tc_scan_kernel<32, 32>, threads);
+  if (cw == 32) return go(f32tc_scan_kernel<16, 32>, threads);
+  return go(f32tc_scan_kernel<16, 16>, threads);
 }
 
 }  // namespace ftg
