@@ -342,7 +342,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     const int hq = (warp - 2) * 32 + lane;
     const int um_sh = 31 - __clz(p.um), un_sh = 31 - __clz(p.un);
     const int nRow = 128 * (BN >> un_sh), nE = nRow + BN * (128 >> um_sh);
-    constexpr int AHEAD = 4;  // entries a thread loads ahead (more would spill)
+    // entries a thread loads at a time (more would spill); one after the other
+    // the 2048 entries of 16 x 16 units took far longer than their period (1300 x
+    // 900 x 8192 584 us; now 315, still bound by these two warps)
+    constexpr int AHEAD = BN == 128 ? 8 : 4;
     uint32_t checks = 0;
     bool dead = false;
     auto both = [] { asm volatile("bar.sync 2, 64;" ::: "memory"); };
@@ -364,15 +367,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
         // segment g of this period at entry e: its address (null outside the
         // matrix) for g = 0 and the distance to the next
         const int s0 = x.z * p.segs_per_split + period * p.segs_per_period;
+        const int J0 = col0 >> un_sh, I0 = row0 >> um_sh;
+        const float* const dr = p.Dr + ((long long)s0 * p.nw + J0) * p.ldr_d + row0;
+        const float* const dc = p.Dc + ((long long)s0 * p.nv + I0) * p.ldc_d + col0;
         auto seg_of = [&](int e, long long* stride) -> const float* {
           if (e < nRow) {
-            const int J = (col0 >> un_sh) + (e >> 7), gr = row0 + (e & 127);
+            const int J = e >> 7, r = e & 127;
             *stride = (long long)p.nw * p.ldr_d;
-            return J < p.nw && gr < p.M ? p.Dr + ((long long)s0 * p.nw + J) * p.ldr_d + gr : nullptr;
+            return J0 + J < p.nw && row0 + r < p.M ? dr + J * p.ldr_d + r : nullptr;
           }
-          const int I = (row0 >> um_sh) + (e - nRow) / BN, gc = col0 + (e - nRow) % BN;
+          const int I = (e - nRow) / BN, c = (e - nRow) % BN;
           *stride = (long long)p.nv * p.ldc_d;
-          return I < p.nv && gc < p.N ? p.Dc + ((long long)s0 * p.nv + I) * p.ldc_d + gc : nullptr;
+          return I0 + I < p.nv && col0 + c < p.N ? dc + I * p.ldc_d + c : nullptr;
         };
         const int segs = min(p.segs_per_period, p.segs_per_split - period * p.segs_per_period);
         auto first = [&](int e) {
@@ -395,19 +401,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
                                : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), gc < p.N ? p.nB[gc] : 0.f);
           }
         };
-        float d[AHEAD];
-#pragma unroll
-        for (int i = 0; i < AHEAD; ++i) d[i] = first(hq + 64 * i);
-        if (checks > 0 && !dead && !mbar_wait(&T.chk_empty, (checks - 1) & 1u)) {
-          dead = true;
-          atomicExch(&T.abort, 1);
-        }
 #pragma unroll 1
-        for (int e = hq; e < nE; e += 64) {
-          enter(e, d[0]);
+        for (int e0 = hq; e0 < nE; e0 += 64 * AHEAD) {
+          float d[AHEAD];
 #pragma unroll
-          for (int i = 1; i < AHEAD; ++i) d[i - 1] = d[i];
-          d[AHEAD - 1] = first(e + 64 * AHEAD);
+          for (int i = 0; i < AHEAD; ++i) d[i] = first(e0 + 64 * i);
+          // (the loads of small units' further entries overlap the coming period)
+          if (e0 == hq && checks > 0 && !dead && !mbar_wait(&T.chk_empty, (checks - 1) & 1u)) {
+            dead = true;
+            atomicExch(&T.abort, 1);
+          }
+#pragma unroll
+          for (int i = 0; i < AHEAD; ++i)
+            if (e0 + 64 * i < nE) enter(e0 + 64 * i, d[i]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&T.chk_full);
@@ -684,9 +690,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
               const float* src = (is_row ? &T.rowpart[0][0] : &T.colpart[0][0]) + ((at >> sh) * per << sh) + (at & ((1 << sh) - 1));
               float w[128 / (GC < GR ? GC : GR)], s = 0.f;
 #pragma unroll
-              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) w[g] = src[(g < per ? g : 0) << sh];
+              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) w[g] = g < per ? src[g << sh] : 0.f;
 #pragma unroll
-              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) s += g < per ? w[g] : 0.f;
+              for (int g = 0; g < 128 / (GC < GR ? GC : GR); ++g) s += w[g];
               if (ok && fabsf(s - c) > kScreen * tau_of(e, c)) flags |= 1u << i;
             }
             if (bar_red_or(1, EPI_T, flags != 0u)) {
