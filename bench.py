@@ -11,7 +11,7 @@ magnitudes log-uniform in [1e-2, 1e3] x the expected tile maximum.  Inputs
 
 Prints one JSON line: TFLOP/s of the ABFT GEMM (2*M*N*K per step), overhead
 against the same kernel with ABFT off, detection / false-alarm counts, the
-roofline of the dominant kernel against the fp32 CUDA-core peak, the same
+roofline of the dominant kernel (six bf16 MMAs a product), the same
 metric end to end from host buffers, the CPU oracle as a bounded-sample
 baseline, clocks sampled during the timed region and the kernel launch count.
 
@@ -46,6 +46,7 @@ SCHED16 = dict(m_tb=128, n_tb=128, k_tb=16, m_w=64, n_w=64, m_t=16, n_t=8, caden
 SCHED_OFF_BEST = dict(m_tb=128, n_tb=128, k_tb=16, m_w=32, n_w=64, m_t=8, n_t=8, cadence=16, split_k=1)
 FAULTS_PER_MIN = 200.0
 KERNEL_SOURCES = ["simt_ftgemm.cuh", "simt_wide32.cu", "internal.cuh", "ptx.cuh", "mlp.cuh"]
+F32TC_KERNEL_SOURCES = ["f32tc_gemm.cu", "f32tc.cuh", "internal.cuh", "ptx.cuh"]
 TC_KERNEL_SOURCES = ["tc_gemm.cu", "internal.cuh", "ptx.cuh", "mlp.cuh"]
 
 
@@ -247,9 +248,11 @@ def committed_traffic(kernel_key, files=KERNEL_SOURCES):
     return ent.get("dram_bytes_per_launch")
 
 
-def fp32_peak_tflops(sms, mhz):
-    # CUDA-core fp32: SMs x 128 lanes x 2 flop (FMA) x clock
-    return sms * 128 * 2 * mhz * 1e6 / 1e12
+def fp32_tc_peak_tflops(key):
+    # fp32 on the tensor cores: six bf16 products per fp32 product, of the
+    # measured cuBLAS bf16 rate `key` (None where it was not measured)
+    pk = _peaks().get(key)
+    return pk / 6.0 if pk else None
 
 
 def make_faults(step_seed, t_kernel_s, n, ksteps):
@@ -1108,15 +1111,18 @@ def irregular_extras(ft, h, synth, dev, timed_loop):
         rep = h.gemm(A, B, C, level=ft.FT_AUTO, inject=[(a, b, ks, r, c, 64.0 * math.sqrt(K))])
         ok = [(x["row"], x["col"], x["kind"]) for x in rep.records] == [(a * s.m_tb + r, b * s.n_tb + c, 0)]
         # roofline of the shape: the slower of streaming A, B, C once through
-        # HBM (measured copy rate) and the fp32 ALU peak
+        # HBM (measured copy rate) and the six bf16 products of an fp32 one
         hbm = _peaks().get("hbm_gbs") or 0.0
         t_hbm = 4.0 * (M * K + K * N + M * N) / (hbm * 1e9) if hbm else 0.0
-        t_alu = fl / (fp32_peak_tflops(152, 2070.0) * 1e12)
-        attain = fl / max(t_hbm, t_alu) / 1e12
-        out[f"{M}x{N}x{K}"] = {"tflops": round(fl / (ms / 1e3) / 1e12, 3),
-                               "bound": "hbm" if t_hbm > t_alu else "alu",
-                               "attainable_tflops": round(attain, 3),
-                               "frac_of_attainable": round(fl / (ms / 1e3) / 1e12 / attain, 3),
+        pk = fp32_tc_peak_tflops("bf16_tflops")
+        t_mma = fl / (pk * 1e12) if pk else 0.0
+        t_low = max(t_hbm, t_mma)
+        attain = fl / t_low / 1e12 if t_low else None
+        tflops = fl / (ms / 1e3) / 1e12
+        out[f"{M}x{N}x{K}"] = {"tflops": round(tflops, 3),
+                               "bound": "hbm" if t_hbm > t_mma else "tensor",
+                               "attainable_tflops": round(attain, 3) if attain else None,
+                               "frac_of_attainable": round(tflops / attain, 3) if attain else None,
                                "ft_off_default_tflops": round(fl / (ms_off / 1e3) / 1e12, 3),
                                "torch_fp32_tflops": round(fl / (ms_t / 1e3) / 1e12, 3),
                                "level": [k for k, v in ft.LEVELS.items() if v == lv][0],
@@ -1241,21 +1247,19 @@ def main():
                             "uncorrectable": int(rep.uncorrectable), "checksum_only": int(rep.checksum_only)})
     kern_ms = st["kernel_ms"] / max(1, st["timed_launches"])
     achieved = flops / (kern_ms / 1e3) / 1e12
-    peak_spec = fp32_peak_tflops(sms, 2070.0)
-    peak_meas = fp32_peak_tflops(sms, clk["sm_mhz"]) if clk.get("sm_mhz") else None
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak_spec, "unit": "TFLOP/s",
-                "frac": achieved / peak_spec, "traffic": committed_traffic("simt_ftgemm_block_wide_16384"),
-                "kernel": "simt_ftgemm_kernel<128x128x32 (m_t=16, n_t=8, 3 stages), BLOCK>",
-                "peak_basis": f"fp32 CUDA cores: {sms} SMs x 128 x 2 flop x 2070 MHz (max SM clock)",
-                "peak_at_measured_clock": peak_meas,
-                "frac_at_measured_clock": achieved / peak_meas if peak_meas else None,
+    peak = fp32_tc_peak_tflops("bf16_tflops_sustained")
+    roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak if peak else None,
+                "traffic": committed_traffic("f32tc_block_16384", F32TC_KERNEL_SOURCES),
+                "kernel": "f32tc_kernel<256 columns, BLOCK> (three exact bf16 planes an operand, six MMAs a product)",
+                "peak_basis": "a sixth of the measured sustained cuBLAS bf16 rate (MEASURED_PEAKS.json)",
                 "kernel_ms": kern_ms}
 
     # ---- the encoding pass (Eq. 1-2): e^T A per 128-row block, B e per
     # 128-column block, row and column norms.  Algorithmic bytes: read A and
     # B, write the checksum vectors and norms.  Timed on its own through
     # ftgemm_encode, and inside the GEMM call as call time minus kernel time
-    # (there it also writes A^T for the k-major TMA stream).
+    # (there it also writes the three bf16 planes of A and B).
     tm_, tn_ = -(-n // 128), -(-n // 128)
     Venc = torch.empty(tm_, n, device=dev)
     Wenc = torch.empty(tn_, n, device=dev)
@@ -1265,7 +1269,8 @@ def main():
     hbm = _peaks().get("hbm_gbs")
     encode_pass = {"algorithmic_bytes": enc_bytes, "standalone_ms": ms_enc,
                    "standalone_gbs": enc_bytes / (ms_enc / 1e3) / 1e9,
-                   "in_gemm_ms": ms - kern_ms, "in_gemm_gbs": enc_bytes / ((ms - kern_ms) / 1e3) / 1e9,
+                   "in_gemm_ms": ms - kern_ms,
+                   "in_gemm_gbs": (enc_bytes + 12 * n * n) / ((ms - kern_ms) / 1e3) / 1e9,
                    "peak_gbs": hbm, "standalone_frac": (enc_bytes / (ms_enc / 1e3) / 1e9) / hbm if hbm else None,
                    "peak_basis": "measured copy bandwidth (MEASURED_PEAKS.json)"}
     del Venc, Wenc, nAe, nBe

@@ -11,10 +11,11 @@
 //   e4m3: x = sum_c q_c / s_c with s_c = s_0 * 16^c, q_c = e4m3(residual * s_c)
 //         and s_0 a power of two putting the block's largest |x| near 448.
 // Norms of the rows of A and of the columns of B scale the detection
-// threshold.  B is also transposed to the K-major layout the MMA reads,
-// except a bf16 B without checksums, which the MMA reads in place.
+// threshold.  B is also laid out as the MMA reads it: bf16 with checksums packed
+// by tiles beside its pieces, e4m3 transposed to K-major; a bf16 B without
+// checksums is read in place (transposed if it is not aligned).
 // Each operand is read once: one kernel reads A for its block sums and row
-// norms, one reads B for B^T, its block sums and column norms (partial
+// norms, one reads B for its layout, block sums and column norms (partial
 // norms per k-chunk, finished without atomics so results are reproducible).
 //
 // Quantizer: bf16 by round-to-nearest-even; e4m3 with a per-tensor scale
