@@ -338,7 +338,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
     // runs and added once it is verified; a tile's first period also forms the
     // thresholds' norm terms.  Done by the epilogue itself this kept the MMAs
     // waiting: the 256-column tiles of 8192^3 took 3.54 ms, now 3.35, those of
-    // 4096^3's three full waves 430 us, now 407.
+    // 4096^3's three full waves 430 us, now 407.  A tile's norms are loaded before
+    // its turn too: 16384 x 16384 x 32, one period a tile, 550 us a call without
+    // that, now 410.
     const int hq = (warp - 2) * 32 + lane;
     const int um_sh = 31 - __clz(p.um), un_sh = 31 - __clz(p.un);
     const int nRow = 128 * (BN >> un_sh), nE = nRow + BN * (128 >> um_sh);
@@ -355,8 +357,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       const int ks0 = x.z * p.ks_per_split, nks = min(p.ks_per_split, p.ksteps - ks0);
       // Frobenius norms of the units' rows and columns
       auto fro = [](const float* sq16, int first, int per, int count) {
-        float s = 0.f;
-        for (int g = 0; g < per && first + g < count; ++g) s += sq16[first + g];
+        float v[8], s = 0.f;  // (loads first: per <= 8)
+#pragma unroll
+        for (int g = 0; g < 8; ++g) v[g] = g < per && first + g < count ? sq16[first + g] : 0.f;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) s += v[g];
         return sqrtf(s);
       };
       both();  // the other warp is done with the tile before
@@ -386,7 +391,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           const float* src = e < nE ? seg_of(e, &stride) : nullptr;
           return src ? __ldg(src) : 0.f;
         };
-        auto enter = [&](int e, float d) {  // entry e, d its first segment
+        auto norm = [&](int e) {  // of the row or column of entry e
+          const int gr = row0 + (e & 127), gc = col0 + (e - nRow) % BN;
+          if (e < nRow) return gr < p.M ? p.nA[gr] : 0.f;
+          return e < nE && gc < p.N ? p.nB[gc] : 0.f;
+        };
+        auto enter = [&](int e, float d, float nrm) {  // entry e, d its first segment
           float c = (period > 0 ? T.c[e] : 0.f) + d;
           if (segs > 1) {  // periods longer than a segment
             long long stride;
@@ -396,9 +406,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           T.c[e] = c;
           if (period == 0) {
             // lambda * u times the norms, rounded as ft_tau does
-            const int gr = row0 + (e & 127), gc = col0 + (e - nRow) % BN;
-            T.tn[e] = e < nRow ? __fmul_rn(__fmul_rn(p.lam_u, gr < p.M ? p.nA[gr] : 0.f), T.sFB[e >> 7])
-                               : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), gc < p.N ? p.nB[gc] : 0.f);
+            T.tn[e] = e < nRow ? __fmul_rn(__fmul_rn(p.lam_u, nrm), T.sFB[e >> 7])
+                               : __fmul_rn(__fmul_rn(p.lam_u, T.sFA[(e - nRow) / BN]), nrm);
           }
         };
 #pragma unroll 1
@@ -406,6 +415,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           float d[AHEAD];
 #pragma unroll
           for (int i = 0; i < AHEAD; ++i) d[i] = first(e0 + 64 * i);
+          float nrm[AHEAD];
+#pragma unroll
+          for (int i = 0; i < AHEAD; ++i) nrm[i] = period == 0 ? norm(e0 + 64 * i) : 0.f;
           // (the loads of small units' further entries overlap the coming period)
           if (e0 == hq && checks > 0 && !dead && !mbar_wait(&T.chk_empty, (checks - 1) & 1u)) {
             dead = true;
@@ -413,7 +425,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           }
 #pragma unroll
           for (int i = 0; i < AHEAD; ++i)
-            if (e0 + 64 * i < nE) enter(e0 + 64 * i, d[i]);
+            if (e0 + 64 * i < nE) enter(e0 + 64 * i, d[i], nrm[i]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&T.chk_full);
