@@ -70,7 +70,8 @@ struct F32TcParams {
   const int* bad; int epoch;
 };
 
-// The encode pass: operand planes, and (um > 0) checksum vectors and norms.
+// The encode pass: operand planes, and (um > 0) checksum vectors and squared-norm
+// partials (the SUMS launch forms the norms from them).
 struct F32TcPrep {
   int M, N, K;
   int um, un, nv, nw;

@@ -6,18 +6,18 @@
 // CTA its own 128 rows, as the bf16 kernel does (tc_gemm.cu).  Warp 0 issues
 // TMA loads (the three planes of an operand tile in one 3-D box), warp 1 of
 // the even CTA the MMAs: per 32-element chunk of K the six plane products,
-// smallest first, into one of the tensor-memory accumulators.  Eight epilogue
-// warps read each finished chunk and add it to the accumulators they hold in
-// registers (thread = 4 rows x BN / 8 columns), while the MMAs of the next chunks
-// run.  At the end of a verification period they inject the scheduled faults
+// smallest first, into one of the tensor-memory accumulators.  Eight (sixteen)
+// epilogue warps read each finished chunk and add it to the accumulators they
+// hold in registers (64 a thread: 4 rows x 16 columns), while the MMAs of the next
+// chunks run.  At the end of a verification period they inject the scheduled faults
 // (Section 5.3), form the unit's row and column sums, compare them with the
 // checksums and locate and correct (Section 4.2.1), exactly as the CUDA-core
 // kernel does on its fragments (simt_ftgemm.cuh).
 //
 // The checksums (Eq. 4) come from the same kernel (SUMS = true) run first on
 // the encoded operands: (e^T A) B and A (B e), one result per segment of at
-// most 256 of K, all segments in parallel; the main kernel adds a period's
-// segments to the running checksums when it verifies the period.  They cost
+// most 256 of K, all segments in parallel; two warps of the main kernel add a
+// period's segments to the running checksums ahead of its verification.  They cost
 // the units' share of a tile (1/128 of the product each for 128 x 128 units)
 // instead of an extra operand row in every MMA, so the verification unit
 // stays the schedule's own tile.
@@ -36,11 +36,11 @@ cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cu
 // thread needs 64 cycles or more per MMA, which is what a 256 x 128 one runs
 // for, and some 300 between chunks; a 256 x 256 one runs 128 and its queue
 // covers the gap (8192^3 without checksums: 1080 cycles a chunk of 256 x 128,
-// 1560 of 256 x 256, against 768 and 1536 of MMA time; 4.4 and 3.5 ms).
+// 1560 of 256 x 256, against 768 and 1536 of MMA time; 4.4 and 3.3 ms).
 // What bounds it at BN = 256: the tensor cores without checksums (16384^3
-// 29.4-30.6 ms, 290 TFLOP/s = 1740 of bf16 MMAs, the power cap); with block
+// 28.7-30.6 ms, 295 TFLOP/s = 1770 of bf16 MMAs, the power cap); with block
 // checksums the verification, which stops the MMAs once both accumulators are
-// full (33.3-35 ms; the CUDA-core kernel 133.8).
+// full (32-34 ms; the CUDA-core kernel 133.8).
 template <int BN>
 struct F32TcCfg {
   static constexpr int BM = F32TC_BM, KC = F32TC_KC;

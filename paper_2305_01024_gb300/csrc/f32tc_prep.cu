@@ -1,7 +1,8 @@
 // f32tc_prep.cu -- encode pass of the fp32 GEMM on the tensor cores: the
 // three bf16 planes of A and B (f32tc.cuh), the checksum vectors e^T A per
 // row unit and B e per column unit (Eq. 1-2) in fp32 and as planes, and the
-// norms that scale the detection threshold.  Each operand is read once.
+// partials of the norms that scale the detection threshold.  Each operand is
+// read once.
 //
 // The planes are written in the order the GEMM kernel reads them: every
 // (128-row tile, 32-element chunk of K) of A, and every (64-column tile,
