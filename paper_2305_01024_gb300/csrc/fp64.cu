@@ -317,8 +317,11 @@ __global__ void __launch_bounds__(256, GM * GN == 1 ? 1 : 2) f64_gemm_kernel(con
         for (int j = 0; j < TN; ++j) acc[i][j] = f64_mac(acc[i][j], a[i], b[j]);
       if constexpr (ABFT) {
         // Eq. 4: c^c += (e^T A_I(:,k)) B_J(k,:),  c^r += A_I(:,k) (B_J(k,:) e)
-        if (own_c) csum = f64_mac(csum, vs[buf][kk], Bs[buf][kk][tid]);
-        else if (own_r) csum = f64_mac(csum, As[buf][kk][tid - BN], ws[buf][kk]);
+        // (one multiply-add whichever of the two the thread carries: the fp64
+        // pipe is the bound, and both under predicates cost 2 % of 4096 x 4096 x 2048)
+        const T cx = own_c ? vs[buf][kk] : As[buf][kk][own_r ? tid - BN : 0];
+        const T cy = own_c ? Bs[buf][kk][tid < BN ? tid : 0] : ws[buf][kk];
+        if (own_c || own_r) csum = f64_mac(csum, cx, cy);
       }
     }
     // faults scheduled after this k-step (Section 5.3): additive offsets
