@@ -49,7 +49,7 @@ cudaError_t launch_kmajor_operands_if(const int* gate, int epoch, const float* A
                                       long long ldt, const float* B, long long ldb, int N, float* Bp, long long ldbp,
                                       int* launches, cudaStream_t st);
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
-                               int* launches, cudaStream_t st);
+                               bool captured, int* launches, cudaStream_t st);
 bool f32tc_scan_units(int um, int un);
 bool f32tc_scan_groups(int M, int N, int um, int un, int periods);
 cudaError_t launch_f32tc(int bn, int tail, bool abft, const F32TcMaps& maps, const F32TcParams& p, int sms, int* launches, cudaStream_t st);
@@ -142,6 +142,7 @@ struct ftgemm_ctx {
   ftgemm_fault_record* recs = nullptr;
   int rep_cap = 1 << 16;
   HostReport* h_rep = nullptr;  // page-locked: where a fetch reads the report
+  int* bad = nullptr;           // device: the last fp32 tensor-core call that met a value its planes cannot hold
   int epoch = 0;                // number of the fp32 tensor-core call (never 0 in one)
   bool rep_clean = true;        // nothing that may report was enqueued since the counters were last zero
   bool rep_replayed = false;    // a captured call reports here whenever its graph is replayed: never clean
@@ -447,12 +448,14 @@ static int clear_report(ftgemm_ctx* h) {
   return FTGEMM_OK;
 }
 
-// A call whose events stay in the report until it is fetched.
-static int keep_report(ftgemm_ctx* h) {
+// A call whose events stay in the report until it is fetched (captured: set
+// when the stream is being captured).
+static int keep_report(ftgemm_ctx* h, bool* captured = nullptr) {
   h->rep_clean = false;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(h->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) h->rep_replayed = true;
+  if (captured) *captured = cs != cudaStreamCaptureStatusNone;
   return FTGEMM_OK;
 }
 extern "C" int ftgemm_report_fetch(ftgemm_handle_t h, ftgemm_report* out);
@@ -1139,6 +1142,8 @@ int ftgemm_create(ftgemm_handle_t* handle, int device, void* cuda_stream) {
   r.capacity = h->rep_cap;
   cudaError_t e = cudaMalloc(&h->rep, sizeof(DevReport));
   if (e == cudaSuccess) e = cudaMalloc(&h->recs, sizeof(ftgemm_fault_record) * h->rep_cap);
+  if (e == cudaSuccess) e = cudaMalloc(&h->bad, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(h->bad, 0, sizeof(int));  // (done before the copy begins)
   if (e == cudaSuccess) e = cudaMemcpy(h->rep, &r, sizeof(r), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaHostAlloc(&h->h_rep, sizeof(HostReport), cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->faults_free, cudaEventDisableTiming);
@@ -1158,6 +1163,7 @@ int ftgemm_destroy(ftgemm_handle_t h) {
   if (h->rep) cudaFree(h->rep);
   if (h->recs) cudaFree(h->recs);
   if (h->zimag) cudaFree(h->zimag);
+  if (h->bad) cudaFree(h->bad);
   if (h->h_rep) cudaFreeHost(h->h_rep);
   if (h->d_faults) cudaFree(h->d_faults);
   if (h->h_faults) cudaFreeHost(h->h_faults);
@@ -1656,8 +1662,9 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     if (rc) return rc;
   }
 
+  bool captured = false;
   {
-    int rc = report ? clear_report(h) : keep_report(h);
+    int rc = report ? clear_report(h) : keep_report(h, &captured);
     if (rc) return rc;
   }
 
@@ -1696,7 +1703,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   bool use_tc = !At_given && !detect && !learned && !sink &&
                 f32tc_plan(M, N, K, level, s, split, ks_per_split, cadence, m_u, n_u,
                            (h->num_sms > 0 ? h->num_sms : 148) / 2, &tc);
-  size_t oAt, oBp, oV, oW, oNa, oNb, oPart, oScr = 0, oCo = 0, oTc[10] = {};
+  size_t oAt, oBp, oV, oW, oNa, oNb, oPart, oScr = 0, oCo = 0, oTc[9] = {};
   if (use_tc) {
     auto planes = [&](int lines) { return (size_t)((lines + 127) / 128) * tc.nch * (3 * F32TC_APLANE / 2); };
     oAt = take(std::max(planes(M), nAt));
@@ -1712,8 +1719,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
       oTc[6] = take((size_t)tc.segs * nvb * tc.ldc_d);
       oTc[7] = take((size_t)tc.segs * nwb * tc.ldr_d);
     }
-    oTc[8] = take(1);
-    if (tc.by_segments) oTc[9] = take((size_t)tc.segs * M * tc.ldp);
+    if (tc.by_segments) oTc[8] = take((size_t)tc.segs * M * tc.ldp);
     if (ensure_ws(h, o) != FTGEMM_OK) {  // no room for the planes
       cudaGetLastError();
       use_tc = false;
@@ -1745,12 +1751,12 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
     e.Vp = (uint16_t*)(ws + oTc[0]); e.Wp = (uint16_t*)(ws + oTc[1]);
     e.pa = ws + oTc[2]; e.pb = ws + oTc[3];
     e.nA = ws + oNa; e.nB = ws + oNb; e.sq16a = ws + oTc[4]; e.sq16b = ws + oTc[5];
-    e.bad = (int*)(ws + oTc[8]);
+    e.bad = h->bad;
     h->epoch = h->epoch % 0x7fffffff + 1;
     e.epoch = h->epoch;
-    CK(launch_f32tc_split(Af, lda, Bf, ldb, e, &launches, h->stream));
+    CK(launch_f32tc_split(Af, lda, Bf, ldb, e, captured, &launches, h->stream));
     int rc = f32tc_run(h, tc, e, alpha, beta, C, ldc, al16(C), level, s, split, ks_per_split, cadence, ksteps, tiles_n,
-                       nf, ws + oTc[6], ws + oTc[7], ws + oTc[9], split > 1 ? ws + oPart : nullptr, &launches);
+                       nf, ws + oTc[6], ws + oTc[7], ws + oTc[8], split > 1 ? ws + oPart : nullptr, &launches);
     if (rc) return rc;
     gate = e.bad;
     if (report && split == 1) {

@@ -65,8 +65,9 @@ struct F32TcParams {
   float* partial;              // [split][M][N], or null
   const Fault* faults; int nfaults;
   DevReport* rep; ftgemm_fault_record* recs;
-  // the encode pass sets *bad to `epoch` (the call's own number) when an operand
-  // is outside the split's range: nothing to clear before a call
+  // the encode pass sets *bad (the handle's own word) to `epoch`, the call's own
+  // number, when an operand is outside the split's range: nothing to clear before
+  // a call, except in a graph, whose replays share one number (launch_f32tc_split)
   const int* bad; int epoch;
 };
 

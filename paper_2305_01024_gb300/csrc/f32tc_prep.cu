@@ -205,13 +205,25 @@ __global__ void __launch_bounds__(256) f32tc_split_kernel(const float* __restric
   store_planes8(P + row_unit(unit, k, nch), F32TC_APLANE, s);
 }
 
+__global__ void f32tc_clear_kernel(int* bad) { *bad = 0; }
+
+// captured: the launches go into a graph.  Its replays all carry the epoch of
+// the capture, so each clears the flag first: what one replay's operands held
+// does not send the next one to the CUDA cores.
 cudaError_t launch_f32tc_split(const float* A, long long lda, const float* B, long long ldb, const F32TcPrep& e,
-                               int* launches, cudaStream_t st) {
+                               bool captured, int* launches, cudaStream_t st) {
   const int veca = lda % 4 == 0 && ((uintptr_t)A & 15) == 0, vecb = ldb % 4 == 0 && ((uintptr_t)B & 15) == 0;
   const int kgroups = (e.K + 127) / 128;
   const long long ab = (long long)kgroups * ((e.M + 127) / 128), bb = (long long)kgroups * ((e.N + 127) / 128);
   if (ab + bb > 0x7fffffff) return cudaErrorInvalidValue;
-  cudaError_t er = launch_pdl(f32tc_split_kernel, (unsigned)(ab + bb), 256, 0, st, A, lda, B, ldb, e, veca, vecb, (int)ab);
+  cudaError_t er = cudaSuccess;
+  if (captured) {
+    f32tc_clear_kernel<<<1, 1, 0, st>>>(e.bad);
+    er = cudaGetLastError();
+    if (er != cudaSuccess) return er;
+    *launches += 1;
+  }
+  er = launch_pdl(f32tc_split_kernel, (unsigned)(ab + bb), 256, 0, st, A, lda, B, ldb, e, veca, vecb, (int)ab);
   *launches += 1;
   return er;
 }
