@@ -564,8 +564,9 @@ int ftgemm_encode(ftgemm_handle_t handle, int64_t m, int64_t n, int64_t k,
 
 /* Counters of the handle.  launches: kernels enqueued by this handle (all
  * kinds).  With timing enabled, CUDA events recorded on the handle's stream
- * bracket every main GEMM kernel launch; kernel_ms is the sum of their
- * durations and timed_launches their number. */
+ * bracket every call's main GEMM kernel; kernel_ms is the sum of their
+ * durations and timed_launches their number.  (An F32 call on the tensor cores
+ * whose CUDA-core stand-by is enqueued counts once, with the time of both.) */
 typedef struct {
   int64_t launches;
   int64_t timed_launches;

@@ -188,6 +188,7 @@ struct ftgemm_ctx {
   bool timing = false;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending, pool;
   int64_t timed = 0;
+  int64_t more = 0;  // of the pending spans, those of a call that has one already
   double kernel_ms = 0.0;
 };
 
@@ -437,6 +438,8 @@ static int drain_events(ftgemm_ctx* h) {
     h->timed += 1;
     h->pool.push_back(e);
   }
+  h->timed -= h->more;
+  h->more = 0;
   h->pending.clear();
   return FTGEMM_OK;
 }
@@ -1838,8 +1841,8 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   p.only_if = gate;
   p.epoch = h->epoch;
   std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-  const bool timed = h->timing && !gate;  // (the tensor-core kernels were timed themselves)
-  if (timed) {
+  // in place of the tensor-core kernels, it adds to the time of their call
+  if (h->timing) {
     int rc = take_events(h, &ev);
     if (rc) return rc;
     CK(cudaEventRecord(ev.first, h->stream));
@@ -1847,9 +1850,10 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
   if (detect) CK(simt_launch_wide32_detect(maps, p, split, h->stream));
   else CK(cfg->launch((int)level, maps, p, split, h->stream));
   ++launches;
-  if (timed) {
+  if (h->timing) {
     CK(cudaEventRecord(ev.second, h->stream));
     h->pending.push_back(ev);
+    if (use_tc) ++h->more;
   }
   if (split > 1) {
     CK(launch_splitk_reduce(ws + oPart, split, M, N, (float)alpha, (float)beta, C, ldc, h->stream));
