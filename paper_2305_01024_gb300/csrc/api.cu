@@ -1463,7 +1463,7 @@ struct F32TcPlan {
   int bn;                   // columns of a CTA pair's tile: 256 or 128
   int tail;                 // of the 256-column tiles, those run as two of 128 after the others
   long long ldc_d, ldr_d;   // row strides of the checksum segments
-  int seg, segs_per_period, segs_per_split;
+  F32TcSegs sg;
   long long segs;           // over all splits
   bool by_segments;         // few tiles, long K: the product by segments, then a scan
   long long ldp;            // row stride of the product's segments
@@ -1526,52 +1526,64 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
   }
   t.ldc_d = ((long long)N + 3) / 4 * 4;
   t.ldr_d = ((long long)M + 3) / 4 * 4;
-  t.seg = (period >= kps || period % F32TC_SEG == 0) ? F32TC_SEG : (int)period;
-  const long long span = std::min<long long>(kps, K);
-  t.segs_per_split = (int)((span + t.seg - 1) / t.seg);
-  t.segs_per_period = period >= kps ? t.segs_per_split : (int)(period / t.seg);
-  t.segs = (long long)split * t.segs_per_split;
+  const int span = (int)std::min<long long>(kps, K);
+  const double nv = abft ? (M + um - 1) / um : 0, nw = abft ? (N + un - 1) / un : 0;
+  auto fits = [&](const F32TcSegs& sg) {  // checksum segments: 2 GiB
+    return 4.0 * split * sg.per_split * (nv * t.ldc_d + nw * t.ldr_d) <= 2147483648.0;
+  };
   t.by_segments = false;
   t.ldp = ((long long)N + 3) / 4 * 4;
-  if (split == 1 && (!abft || f32tc_scan_units(um, un))) {
-    // Few tiles and a long K leave most CTA pairs idle in a pass over K; the
-    // segments of K run side by side and a scan adds them up.  Both routes in
-    // tens of SM cycles: a chunk 107 (127 with verification), the scan 135 a
-    // segment with verification (20 by shares), 300 for its launch, and 21 KB of segments
-    // written and read.  Measured, us per call, one pass / by segments: BLOCK
-    // 256x256x65536 1890 / 383, 512x512x8192 (32 x 32 units) 190 / 126, but
-    // 777x1531x2049 114 / 125, 2543x700x3717 189 / 197; OFF 640x640x4096 98 / 53.
-    const long long m2 = ((long long)M + 255) / 256, n1 = ((long long)N + 127) / 128, tiles = m2 * n1;
-    long long sums = 0;
-    int seg = t.seg, segs = t.segs_per_split;
-    if (abft) {
-      sums = ((M + um - 1) / um + 255) / 256 * n1 + ((N + un - 1) / un + 255) / 256 * (((long long)M + 127) / 128);
-    } else {
-      // no periods: as many segments as fill the device once, of 256 of K or more
-      segs = (int)std::min<long long>((K + 255) / 256, std::max<long long>(1, pairs / tiles));
-      seg = ((K + segs - 1) / segs + F32TC_KC - 1) / F32TC_KC * F32TC_KC;
-      segs = (K + seg - 1) / seg;
-    }
-    auto waves = [&](long long items) { return (items + pairs - 1) / pairs; };
-    const long long per = seg / F32TC_KC;
-    const long long direct = waves(tiles) * t.nch * (abft ? 127 : 107) + waves(sums * segs) * per * 107;
-    const bool groups = abft && f32tc_scan_groups(M, N, um, un, (segs + t.segs_per_period - 1) / t.segs_per_period);
+  // Few tiles and a long K leave most CTA pairs idle in a pass over K; the
+  // segments of K run side by side and a scan adds them up.  Both routes in
+  // tens of SM cycles: a chunk 107 (127 with verification), the scan 135 a
+  // segment with verification (20 by shares), 300 for its launch, and 21 KB of segments
+  // written and read.  Measured, us per call, one pass / by segments: BLOCK
+  // 256x256x65536 1890 / 383, 512x512x8192 (32 x 32 units) 190 / 126, but
+  // 777x1531x2049 114 / 125, 2543x700x3717 189 / 197; OFF 640x640x4096 98 / 53.
+  const long long m2 = ((long long)M + 255) / 256, n1 = ((long long)N + 127) / 128, tiles = m2 * n1;
+  auto waves = [&](long long items) { return (items + pairs - 1) / pairs; };
+  const long long sums = !abft ? 0 : ((M + um - 1) / um + 255) / 256 * n1 + ((N + un - 1) / un + 255) / 256 * (((long long)M + 127) / 128);
+  const bool may_scan = split == 1 && (!abft || f32tc_scan_units(um, un));
+  auto cost = [&](const F32TcSegs& sg, bool* by) {
+    const long long segs = (long long)split * sg.per_split, per = sg.seg / F32TC_KC;
+    const long long direct = waves(tiles * split) * ((span + F32TC_KC - 1) / F32TC_KC) * (abft ? 127 : 107) + waves(sums * segs) * per * 107;
+    *by = false;
+    if (!may_scan || segs <= 1 || 4.0 * segs * M * t.ldp > 536870912.0) return direct;
+    const bool groups = abft && f32tc_scan_groups(M, N, um, un, (sg.per_split + sg.per_period - 1) / sg.per_period);
     const long long scan = waves((tiles + sums) * segs) * per * 107 + (!abft ? 0 : groups ? 20 : 135) * segs + 300 +
                            8LL * segs * M * N / 21000;
-    if (segs > 1 && 4.0 * segs * M * t.ldp <= 536870912.0 && scan * 20 < direct * 19) {
-      t.by_segments = true;
-      t.bn = 128;
-      t.tail = 0;
-      t.seg = seg;
-      t.segs = t.segs_per_split = segs;
-      if (!abft) t.segs_per_period = segs;
+    *by = scan * 20 < direct * 19;
+    return *by ? scan : direct;
+  };
+  if (abft) {
+    t.sg = f32tc_segs(span, (int)period, F32TC_SEG);
+    const long long c = cost(t.sg, &t.by_segments);
+    if (period < kps && period > F32TC_SEG && period % F32TC_SEG) {
+      // A period cut unevenly, or as one segment: less parallel, but fewer results
+      // to write and add up.  Measured, us per call, cut / whole: BLOCK 2048x2048x8192
+      // at 3200 of K 358 / 506, 4096^3 at 3200 613 / 633, but 2048x2048x8192 at 384
+      // 383 / 379, 256x256x65536 (32 x 32 units) at 3200 312 / 236, 512x512x32768 at
+      // 3232 456 / 309; missed by the rule: 512x512x8192 (32 x 32) at 3200 109 / 119.
+      bool by;
+      const F32TcSegs one = f32tc_segs(span, (int)period, (int)period);
+      if (!fits(t.sg) || cost(one, &by) < c) {
+        t.sg = one;
+        cost(one, &t.by_segments);
+      }
     }
+    if (!fits(t.sg)) return false;
+  } else {
+    // no periods: as many segments as fill the device once, of 256 of K or more
+    const int segs = (int)std::min<long long>((K + 255) / 256, std::max<long long>(1, pairs / tiles));
+    t.sg = f32tc_segs(span, span, ((span + segs - 1) / segs + F32TC_KC - 1) / F32TC_KC * F32TC_KC);
+    cost(t.sg, &t.by_segments);
+  }
+  if (t.by_segments) {
+    t.bn = 128;
+    t.tail = 0;
   }
   if (!abft && !t.by_segments && (long long)split * ((M + 255) / 256) * ((N + 127) / 128) < 6) return false;
-  if (abft) {
-    const double nv = (M + um - 1) / um, nw = (N + un - 1) / un;
-    if (4.0 * t.segs * (nv * t.ldc_d + nw * t.ldr_d) > 2147483648.0) return false;  // checksum segments: 2 GiB
-  }
+  t.segs = (long long)split * t.sg.per_split;
   return true;
 }
 
@@ -1599,7 +1611,7 @@ static int f32tc_run(ftgemm_ctx* h, const F32TcPlan& t, const F32TcPrep& e, doub
   p.group_m = std::min(p.tiles_m2, 8);
   p.nsplit = split;
   p.k_per_split = (int)std::min<long long>((long long)ks_per_split * s.k_tb, e.K);
-  p.seg = t.seg; p.segs_per_period = t.segs_per_period; p.segs_per_split = t.segs_per_split;
+  p.sg = t.sg;
   p.um = abft ? e.um : 128; p.un = abft ? e.un : 128;
   p.nv = e.nv; p.nw = e.nw;
   p.m_tb = s.m_tb; p.n_tb = s.n_tb; p.k_tb = s.k_tb;

@@ -16,13 +16,14 @@
 // accumulators the ABFT scheme protects: faults are added there, and every
 // verification period the unit's row and column sums are formed from them.
 #pragma once
+#include "f32tc_seg.cuh"
 #include "internal.cuh"
 
 namespace ftg {
 
 constexpr int F32TC_KC = 32;    // elements of K per pipeline stage and per tensor-core accumulation
 constexpr int F32TC_BM = 128;   // rows of C per CTA (a CTA pair: 256)
-constexpr int F32TC_SEG = 256;  // most elements of K per checksum segment
+constexpr int F32TC_SEG = 256;  // elements of K per checksum segment (f32tc_plan: or one period, if that is no multiple of it)
 
 // Planes in memory: row operands (A, e^T A, (B e)^T) as blocks of 128 rows x
 // 32 elements of K, three planes of 128 64-byte rows each, the 16-byte units
@@ -34,8 +35,6 @@ constexpr int F32TC_SEG = 256;  // most elements of K per checksum segment
 // only reach results that are not stored).
 constexpr int F32TC_APLANE = 128 * F32TC_KC, F32TC_BPLANE = 64 * F32TC_KC;  // elements of a block's plane
 
-// Split into segments of `seg` elements of K (restarting at every split), a
-// verification period is `segs_per_period` whole segments.
 struct F32TcParams {
   int M, N, K;
   int tiles_m2, tiles_n;       // CTA-pair tile rows (2 * F32TC_BM each), tile columns
@@ -44,7 +43,7 @@ struct F32TcParams {
   // one on, in halves of 128 (what the 256-column launch before it leaves over)
   int tiles, half_first;
   int nsplit, k_per_split;     // splits of K and their length in elements
-  int seg, segs_per_period, segs_per_split;
+  F32TcSegs sg;
   // verification units and the schedule's tiling (what records and faults refer to)
   int um, un;                  // unit rows / columns (powers of two, 16 .. 128)
   int nv, nw;                  // units along M and N

@@ -16,7 +16,7 @@
 //
 // The checksums (Eq. 4) come from the same kernel (SUMS = true) run first on
 // the encoded operands: (e^T A) B and A (B e), one result per segment of at
-// most 256 of K, all segments in parallel; two warps of the main kernel add a
+// most 256 of K (of a whole period, where that costs less: f32tc_plan), all in parallel; two warps of the main kernel add a
 // period's segments to the running checksums ahead of its verification.  They cost
 // the units' share of a tile (1/128 of the product each for 128 x 128 units)
 // instead of an extra operand row in every MMA, so the verification unit
@@ -173,7 +173,7 @@ template <int BN, bool SUMS>
 __device__ __forceinline__ int f32tc_items(const F32TcParams& p) {
   if constexpr (!SUMS) return p.tiles;
   const F32TcSums t = f32tc_sums<BN>(p);
-  return p.nsplit * p.segs_per_split * (t.n[0] + t.n[1] + t.n[2]);
+  return p.nsplit * p.sg.per_split * (t.n[0] + t.n[1] + t.n[2]);
 }
 
 template <int BN, bool SUMS>
@@ -208,11 +208,10 @@ __device__ __forceinline__ F32TcItem f32tc_item(const F32TcParams& p, int id) {
     const int cols = t.type == 1 ? u.cols[1] : u.cols[0];
     t.row0 = j / cols * 256;
     t.col0 = j % cols * BN;
-    t.z = t.seg / p.segs_per_split;
-    const int s0 = (t.seg - t.z * p.segs_per_split) * p.seg;  // inside the split
-    t.k0 = t.z * p.k_per_split + s0;
-    t.klen = min(p.seg, min(p.k_per_split - s0, p.K - t.k0));
-    if (t.klen < 0) t.klen = 0;
+    t.z = t.seg / p.sg.per_split;
+    const int k0 = t.z * p.k_per_split;
+    f32tc_segment(p.sg, t.seg - t.z * p.sg.per_split, min(p.k_per_split, p.K - k0), &t.k0, &t.klen);
+    t.k0 += k0;
   }
   return t;
 }
@@ -371,7 +370,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
       for (int period = 0, done = 0; done < nks; ++period, done += p.cadence) {
         // segment g of this period at entry e: its address (null outside the
         // matrix) for g = 0 and the distance to the next
-        const int s0 = x.z * p.segs_per_split + period * p.segs_per_period;
+        const int s0 = x.z * p.sg.per_split + period * p.sg.per_period;
         const int J0 = col0 >> un_sh, I0 = row0 >> um_sh;
         const float* const dr = p.Dr + ((long long)s0 * p.nw + J0) * p.ldr_d + row0;
         const float* const dc = p.Dc + ((long long)s0 * p.nv + I0) * p.ldc_d + col0;
@@ -385,7 +384,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32TcCfg<BN>::THREAD
           *stride = (long long)p.nv * p.ldc_d;
           return I0 + I < p.nv && col0 + c < p.N ? dc + I * p.ldc_d + c : nullptr;
         };
-        const int segs = min(p.segs_per_period, p.segs_per_split - period * p.segs_per_period);
+        const int segs = min(p.sg.per_period, p.sg.per_split - period * p.sg.per_period);
         auto first = [&](int e) {
           long long stride;
           const float* src = e < nE ? seg_of(e, &stride) : nullptr;
@@ -926,7 +925,7 @@ static cudaError_t f32tc_run_bn(bool abft, const F32TcMaps& maps, F32TcParams p,
   if (abft && (p.um < F32TcCfg<BN>::GC || p.un < F32TcCfg<BN>::GC || p.um > 128 || p.un > 128)) return cudaErrorInvalidValue;
   if (abft || p.P) {
     const F32TcSums t = f32tc_sums<BN>(p);
-    const long long items = ((long long)t.n[0] + t.n[1] + t.n[2]) * p.nsplit * p.segs_per_split;
+    const long long items = ((long long)t.n[0] + t.n[1] + t.n[2]) * p.nsplit * p.sg.per_split;
     if (items > INT_MAX) return cudaErrorInvalidValue;
     cudaError_t e = f32tc_launch<BN, false, true>(maps, p, (int)items, sms, st);
     if (e != cudaSuccess) return e;

@@ -141,7 +141,7 @@ __device__ void scan_unit(const F32TcParams& p, int depth, ScanShared& X, float*
 #pragma unroll
   for (int i = 0; i < EPT; ++i) acc[i] = 0.f;
   const float* src = p.P + (long long)row0 * p.ldp + col0 + lc;
-  const int segs = p.segs_per_split;
+  const int segs = p.sg.per_split;
   unsigned ok_rows = 0u;  // bit i: row lrow(i) of this lane's column is inside the matrix
 #pragma unroll
   for (int i = 0; i < EPT; ++i) ok_rows |= (col_ok && row0 + lrow(i) < p.M ? 1u : 0u) << i;
@@ -172,7 +172,7 @@ __device__ void scan_unit(const F32TcParams& p, int depth, ScanShared& X, float*
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   for (int g = 0; g < depth - 1; ++g) fetch();
-  int left = p.segs_per_period;  // segments to the end of the period
+  int left = p.sg.per_period;  // segments to the end of the period
   for (int seg = 0, period = 0; seg < segs; ++seg) {
     // segment `seg` has landed: all but the depth - 2 newest groups
     if (depth == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
@@ -186,7 +186,7 @@ __device__ void scan_unit(const F32TcParams& p, int depth, ScanShared& X, float*
     }
     fetch();  // into the slot read one segment ago
     if (--left > 0 && seg + 1 < segs) continue;
-    left = p.segs_per_period;
+    left = p.sg.per_period;
     const int ks_first = period * p.cadence, ks = min((period + 1) * p.cadence, p.ksteps) - 1;
     ++period;
     if (has_fault) {
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(32 * SCAN_GROUPS) f32tc_scan_groups_kernel(con
   bool redo = false;
 
   // this warp's periods and segments
-  const int segs = p.segs_per_split, spp = p.segs_per_period;
+  const int segs = p.sg.per_split, spp = p.sg.per_period;
   const int share = ((segs + spp - 1) / spp + G - 1) / G;
   const int s0 = min((long long)segs, (long long)g * share * spp), s1 = min((long long)segs, (long long)(g + 1) * share * spp);
   const float* src = p.P + (long long)row0 * p.ldp + col0 + lc;
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(256) f32tc_sum_kernel(const __grid_constant__ 
   const float* s = p.P + (long long)r * p.ldp + c;
   float v = 0.f;
 #pragma unroll 8
-  for (int g = 0; g < p.segs_per_split; ++g) v += __ldg(s + (long long)g * p.M * p.ldp);
+  for (int g = 0; g < p.sg.per_split; ++g) v += __ldg(s + (long long)g * p.M * p.ldp);
   if (p.nfaults > 0) {
     const int tile = r / p.m_tb * p.tiles_n_sched + c / p.n_tb;
     for (int f = first_fault(p.faults, p.nfaults, tile); f < p.nfaults && p.faults[f].tile == tile; ++f)
@@ -506,7 +506,7 @@ cudaError_t launch_f32tc_scan(bool abft, const F32TcParams& p, int* launches, cu
     k<<<units, block, smem, st>>>(p, depth);
     return cudaGetLastError();
   };
-  if (f32tc_scan_groups(p.M, p.N, p.um, p.un, (p.segs_per_split + p.segs_per_period - 1) / p.segs_per_period)) {
+  if (f32tc_scan_groups(p.M, p.N, p.um, p.un, (p.sg.per_split + p.sg.per_period - 1) / p.sg.per_period)) {
     if (ur == 32) return go(f32tc_scan_groups_kernel<32, 32>, 32 * SCAN_GROUPS);
     if (cw == 32) return go(f32tc_scan_groups_kernel<16, 32>, 32 * SCAN_GROUPS);
     return go(f32tc_scan_groups_kernel<16, 16>, 32 * SCAN_GROUPS);
