@@ -221,6 +221,41 @@ static int ensure_ws(ftgemm_ctx* h, size_t floats) {
   return FTGEMM_OK;
 }
 
+// A workspace the call can do without: false if there is no room for it (or the
+// stream is being captured), and the one there is stays as it was.  It is given
+// up first only where the new one has no room beside it but some in its place.
+static bool try_ws(ftgemm_ctx* h, size_t floats) {
+  if (floats <= h->ws_floats) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  size_t room = 0, total = 0;
+  if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+      cudaMemGetInfo(&room, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const size_t page = 2 << 20, need = floats * sizeof(float) + page;
+  if (need > room + h->ws_floats * sizeof(float)) return false;
+  if (need > room) {
+    if (ensure_ws(h, floats) == FTGEMM_OK) return true;
+    cudaGetLastError();
+    return false;
+  }
+  float* ws = nullptr;
+  size_t want = std::max(floats, h->ws_floats * 3 / 2);
+  if (want * sizeof(float) + page > room) want = floats;
+  cudaError_t e = cudaMalloc(&ws, want * sizeof(float));
+  if (e == cudaSuccess && h->ws) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (ws) cudaFree(ws);
+    return false;
+  }
+  if (h->ws) cudaFree(h->ws);
+  h->ws = ws;
+  h->ws_floats = want;
+  return true;
+}
+
 static int ensure_faults(ftgemm_ctx* h, int n) {
   if (n <= h->faults_cap) return FTGEMM_OK;
   CK(cudaStreamSynchronize(h->stream));
@@ -1735,10 +1770,7 @@ static int simt_gemm(ftgemm_ctx* h, int64_t m, int64_t n, int64_t k, double alph
       oTc[7] = take((size_t)tc.segs * nwb * tc.ldr_d);
     }
     if (tc.by_segments) oTc[8] = take((size_t)tc.segs * M * tc.ldp);
-    if (ensure_ws(h, o) != FTGEMM_OK) {  // no room for the planes
-      cudaGetLastError();
-      use_tc = false;
-    }
+    use_tc = try_ws(h, o);  // (else there is no room for the planes)
   }
   if (!use_tc) {
     const size_t nScr = abft ? (size_t)std::max<long long>((long long)((K + 31) / 32) * M,
