@@ -1528,6 +1528,13 @@ static bool f32tc_plan(int M, int N, int K, ftgemm_ft_level level, const ftgemm_
   // call, CUDA cores / tensor cores: BLOCK 384^3 48 / 58, 512^3 61 / 56, 1024^3
   // 129 / 66, 2048x2048x64 44 / 47, 2048x2048x128 55 / 50, 256x256x8192 418 / 275;
   // OFF 512^3 28 / 35, 768^3 44 / 40, 256x256x8192 147 / 192, 512x512x2048 83 / 67.
+  // Products of less than a chunk of K stay on the CUDA cores: with nothing to
+  // average it, the truncation inside the chunk makes sums of like sign less
+  // exact than there.  Error against 64 bits over the sum of |a b|, rms in u,
+  // CUDA cores / tensor cores, 16384 x 16384 x K: U(0,1) K = 8 0.78 / 0.83, 32
+  // 1.40 / 0.99, 96 2.48 / 1.07; all near 1 K = 8 0.85 / 1.15, 16 1.05 / 1.15, 32
+  // 1.36 / 1.15; normal K = 8 0.46 / 0.40, 32 0.47 / 0.26.
+  if (K < F32TC_KC) return false;
   const double flop = 2.0 * M * N * K;
   if (abft ? flop < 2e8 || (K < 96 && flop < 4e9) : flop < 8e8 || (K < 192 && flop < 4e9)) return false;
   F32TcPlan& t = *out;
