@@ -766,7 +766,16 @@ __device__ __forceinline__ void for_each4(const float* __restrict__ x, long long
     for (int u = 0; u < 4; ++u) f(4 * (i + u * stride), v[u]);
   }
   for (; i < n4; i += stride) f(4 * i, __ldg(x4 + i));
-  for (i = 4 * n4 + t; i < n; i += stride) f1(i, x[i]);
+  // an x off the 16-byte boundary, and the last elements: eight loads in flight too
+  // (one a round, bf16 of 22 M values took 76 us instead of 27)
+  for (i = 4 * n4 + t; i + 7 * stride < n; i += 8 * stride) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldg(x + i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) f1(i + u * stride, v[u]);
+  }
+  for (; i < n; i += stride) f1(i, __ldg(x + i));
 }
 
 // Largest of a value over the block (256 threads), in every thread.
