@@ -767,7 +767,7 @@ __device__ __forceinline__ void for_each4(const float* __restrict__ x, long long
   }
   for (; i < n4; i += stride) f(4 * i, __ldg(x4 + i));
   // an x off the 16-byte boundary, and the last elements: eight loads in flight too
-  // (one a round, bf16 of 22 M values took 76 us instead of 27)
+  // (one a round: bf16 of 22 M values 76 us, e4m3 of 31 M 137; now 27 and 75)
   for (i = 4 * n4 + t; i + 7 * stride < n; i += 8 * stride) {
     float v[8];
 #pragma unroll
