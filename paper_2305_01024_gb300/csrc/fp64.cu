@@ -65,10 +65,6 @@ __device__ __forceinline__ double f64_shfl(double v, int o) { return __shfl_xor_
 __device__ __forceinline__ double2 f64_shfl(double2 v, int o) {
   return make_double2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
-__device__ __forceinline__ double f64_axpy(double w, double x, double y) { return fma(w, x, y); }
-__device__ __forceinline__ double2 f64_axpy(double w, double2 x, double2 y) {
-  return make_double2(fma(w, x.x, y.x), fma(w, x.y, y.y));
-}
 // real offset, or imaginary when `imag` (complex only)
 __device__ __forceinline__ double f64_offset(double, double d, bool) { return d; }
 __device__ __forceinline__ double2 f64_offset(double2, double d, bool imag) {
@@ -317,11 +313,20 @@ __global__ void __launch_bounds__(256, GM * GN == 1 ? 1 : 2) f64_gemm_kernel(con
         for (int j = 0; j < TN; ++j) acc[i][j] = f64_mac(acc[i][j], a[i], b[j]);
       if constexpr (ABFT) {
         // Eq. 4: c^c += (e^T A_I(:,k)) B_J(k,:),  c^r += A_I(:,k) (B_J(k,:) e)
-        // (one multiply-add whichever of the two the thread carries: the fp64
-        // pipe is the bound, and both under predicates cost 2 % of 4096 x 4096 x 2048)
-        const T cx = own_c ? vs[buf][kk] : As[buf][kk][own_r ? tid - BN : 0];
-        const T cy = own_c ? Bs[buf][kk][tid < BN ? tid : 0] : ws[buf][kk];
-        if (own_c || own_r) csum = f64_mac(csum, cx, cy);
+        // One multiply-add, whichever of the two the thread carries: the fp64 pipe is
+        // the bound, and both under predicates cost 2 % of 4096 x 4096 x 2048 (61.7 ms,
+        // now 60.5) and 1 % of 2048^3 in four pieces (16.25, now 16.09).  In eight
+        // pieces the choice costs more (163 x 1844 x 2901 3.45 ms, so 3.48).
+        if constexpr (GM * GN <= 4) {
+          if (own_c || own_r) {
+            const T cx = own_c ? vs[buf][kk] : As[buf][kk][tid - BN];
+            const T cy = own_c ? Bs[buf][kk][tid] : ws[buf][kk];
+            csum = f64_mac(csum, cx, cy);
+          }
+        } else {
+          if (own_c) csum = f64_mac(csum, vs[buf][kk], Bs[buf][kk][tid]);
+          else if (own_r) csum = f64_mac(csum, As[buf][kk][tid - BN], ws[buf][kk]);
+        }
       }
     }
     // faults scheduled after this k-step (Section 5.3): additive offsets
@@ -607,10 +612,10 @@ static cudaError_t f64_launch_g(const F64Params& p, int sms, cudaStream_t st) {
   if (tiles_m > 65535) return cudaErrorInvalidConfiguration;
   // The pieces whose waves end first.  With checksums a cluster costs a few
   // per cent: its barriers, and SMs that a GPC's clusters leave over.  Measured,
-  // ms, 1 / 4 / 8 pieces: BLOCK 2048^3 17.7 / 16.2 / 17.1, 4096x4096x2048 61.7 /
-  // 62.0 / 66.4, 1024^3 4.45 / 2.25 / 2.43, 300x260x520 2.28 / 0.62 / 0.36; OFF
-  // 2048^3 16.6 / 14.4 / 14.3, 512^3 2.08 / 0.54 / 0.29; complex BLOCK 1024^3 8.78 /
-  // 8.07, 200x150x96 0.45 / 0.15.
+  // ms, 1 / 4 / 8 pieces: BLOCK 2048^3 17.3 / 16.3 / 17.2, 4096x4096x2048 60.5 /
+  // 62.1 / 66.6, 1024^3 4.38 / 2.27 / 2.57, 300x260x520 2.25 / 0.63 / 0.37; OFF
+  // 2048^3 16.6 / 14.4 / 14.3, 512^3 2.09 / 0.54 / 0.29; complex BLOCK 1024^3 8.78 /
+  // 8.00, 200x150x96 0.46 / 0.16.
   const long long units = (long long)tiles_m * tiles_n;
   auto waves = [&](int pieces) { return (double)((units * pieces + sms - 1) / sms) / pieces; };
   int g = 1;
