@@ -134,15 +134,18 @@ struct ftgemm_ctx {
   int device = 0;
   int num_sms = 0;
   cudaStream_t stream = nullptr;
-  // workspace (floats), grown on demand
+  // workspace (floats), grown on demand; kWsHead floats before it are the
+  // handle's own: `bad`, the last fp32 tensor-core call that met a value its planes
+  // cannot hold (beside the planes: every kernel of a call reads it first, and in
+  // an allocation of its own it cost a call 1-3 us)
   float* ws = nullptr;
+  int* bad = nullptr;
   size_t ws_floats = 0;
   // report
   DevReport* rep = nullptr;
   ftgemm_fault_record* recs = nullptr;
   int rep_cap = 1 << 16;
   HostReport* h_rep = nullptr;  // page-locked: where a fetch reads the report
-  int* bad = nullptr;           // device: the last fp32 tensor-core call that met a value its planes cannot hold
   int epoch = 0;                // number of the fp32 tensor-core call (never 0 in one)
   bool rep_clean = true;        // nothing that may report was enqueued since the counters were last zero
   bool rep_replayed = false;    // a captured call reports here whenever its graph is replayed: never clean
@@ -207,17 +210,32 @@ struct ftgemm_ctx {
       FAIL(FTGEMM_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(_e));    \
   } while (0)
 
+constexpr size_t kWsHead = 64;
+
+static void free_ws(ftgemm_ctx* h) {
+  if (h->ws) cudaFree(h->ws - kWsHead);
+  h->ws = nullptr;
+  h->bad = nullptr;
+  h->ws_floats = 0;
+}
+
+// A new workspace in place of the handle's (given up by then), its own words zero.
+static cudaError_t set_ws(ftgemm_ctx* h, float* base, size_t floats) {
+  h->ws = base + kWsHead;
+  h->bad = reinterpret_cast<int*>(base);
+  h->ws_floats = floats;
+  return cudaMemsetAsync(base, 0, kWsHead * sizeof(float), h->stream);
+}
+
 static int ensure_ws(ftgemm_ctx* h, size_t floats) {
   if (floats <= h->ws_floats) return FTGEMM_OK;
   if (h->ws) {
     CK(cudaStreamSynchronize(h->stream));
-    CK(cudaFree(h->ws));
-    h->ws = nullptr;
-    h->ws_floats = 0;
+    free_ws(h);
   }
-  size_t want = std::max(floats, h->ws_floats * 3 / 2);
-  CK(cudaMalloc(&h->ws, want * sizeof(float)));
-  h->ws_floats = want;
+  float* base = nullptr;
+  CK(cudaMalloc(&base, (floats + kWsHead) * sizeof(float)));
+  CK(set_ws(h, base, floats));
   return FTGEMM_OK;
 }
 
@@ -229,31 +247,27 @@ static bool try_ws(ftgemm_ctx* h, size_t floats) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   size_t room = 0, total = 0;
   if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-      cudaMemGetInfo(&room, &total) != cudaSuccess) {
+      (h->ws && cudaMemGetInfo(&room, &total) != cudaSuccess)) {
     cudaGetLastError();
     return false;
   }
-  const size_t page = 2 << 20, need = floats * sizeof(float) + page;
-  if (need > room + h->ws_floats * sizeof(float)) return false;
-  if (need > room) {
+  const size_t bytes = (floats + kWsHead) * sizeof(float), page = 2 << 20;
+  if (h->ws && bytes + page > room) {
+    if (bytes + page > room + h->ws_floats * sizeof(float)) return false;
     if (ensure_ws(h, floats) == FTGEMM_OK) return true;
     cudaGetLastError();
     return false;
   }
-  float* ws = nullptr;
-  size_t want = std::max(floats, h->ws_floats * 3 / 2);
-  if (want * sizeof(float) + page > room) want = floats;
-  cudaError_t e = cudaMalloc(&ws, want * sizeof(float));
+  float* base = nullptr;
+  cudaError_t e = cudaMalloc(&base, bytes);
   if (e == cudaSuccess && h->ws) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    if (ws) cudaFree(ws);
+    if (base) cudaFree(base);
     return false;
   }
-  if (h->ws) cudaFree(h->ws);
-  h->ws = ws;
-  h->ws_floats = want;
-  return true;
+  free_ws(h);
+  return set_ws(h, base, floats) == cudaSuccess;
 }
 
 static int ensure_faults(ftgemm_ctx* h, int n) {
@@ -1180,8 +1194,6 @@ int ftgemm_create(ftgemm_handle_t* handle, int device, void* cuda_stream) {
   r.capacity = h->rep_cap;
   cudaError_t e = cudaMalloc(&h->rep, sizeof(DevReport));
   if (e == cudaSuccess) e = cudaMalloc(&h->recs, sizeof(ftgemm_fault_record) * h->rep_cap);
-  if (e == cudaSuccess) e = cudaMalloc(&h->bad, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(h->bad, 0, sizeof(int));  // (done before the copy begins)
   if (e == cudaSuccess) e = cudaMemcpy(h->rep, &r, sizeof(r), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaHostAlloc(&h->h_rep, sizeof(HostReport), cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->faults_free, cudaEventDisableTiming);
@@ -1197,11 +1209,10 @@ int ftgemm_destroy(ftgemm_handle_t h) {
   if (!h) return FTGEMM_OK;
   cudaSetDevice(h->device);
   cudaStreamSynchronize(h->stream);
-  if (h->ws) cudaFree(h->ws);
+  free_ws(h);
   if (h->rep) cudaFree(h->rep);
   if (h->recs) cudaFree(h->recs);
   if (h->zimag) cudaFree(h->zimag);
-  if (h->bad) cudaFree(h->bad);
   if (h->h_rep) cudaFreeHost(h->h_rep);
   if (h->d_faults) cudaFree(h->d_faults);
   if (h->h_faults) cudaFreeHost(h->h_faults);
