@@ -316,8 +316,9 @@ __global__ void __launch_bounds__(256, GM * GN == 1 ? 1 : 2) f64_gemm_kernel(con
         // One multiply-add, whichever of the two the thread carries: the fp64 pipe is
         // the bound, and both under predicates cost 2 % of 4096 x 4096 x 2048 (61.7 ms,
         // now 60.5) and 1 % of 2048^3 in four pieces (16.25, now 16.09).  In eight
-        // pieces the choice costs more (163 x 1844 x 2901 3.45 ms, so 3.48).
-        if constexpr (GM * GN <= 4) {
+        // pieces, and for complex, the choice costs more (163 x 1844 x 2901 3.45 ms, so
+        // 3.48; complex 2048^3 30.5, so 30.8).
+        if constexpr (!CPLX && GM * GN <= 4) {
           if (own_c || own_r) {
             const T cx = own_c ? vs[buf][kk] : As[buf][kk][tid - BN];
             const T cy = own_c ? Bs[buf][kk][tid] : ws[buf][kk];
