@@ -46,7 +46,7 @@ SCHED16 = dict(m_tb=128, n_tb=128, k_tb=16, m_w=64, n_w=64, m_t=16, n_t=8, caden
 SCHED_OFF_BEST = dict(m_tb=128, n_tb=128, k_tb=16, m_w=32, n_w=64, m_t=8, n_t=8, cadence=16, split_k=1)
 FAULTS_PER_MIN = 200.0
 KERNEL_SOURCES = ["simt_ftgemm.cuh", "simt_wide32.cu", "internal.cuh", "ptx.cuh", "mlp.cuh"]
-F32TC_KERNEL_SOURCES = ["f32tc_gemm.cu", "f32tc.cuh", "internal.cuh", "ptx.cuh"]
+F32TC_KERNEL_SOURCES = ["f32tc_gemm.cu", "f32tc.cuh", "f32tc_seg.cuh", "internal.cuh", "ptx.cuh"]
 TC_KERNEL_SOURCES = ["tc_gemm.cu", "internal.cuh", "ptx.cuh", "mlp.cuh"]
 
 
@@ -64,7 +64,8 @@ def parse():
                     help="run one small kernel case for a profiler and exit: tc-<bf16|e4m3>-<tile|off>-<n> "
                          "(tc1- single CTAs, tc2- CTA pairs, tc- the default), "
                          "tcgroup-bf16-<tile|off>-<problems>, f64-<d|z>-<block|off>-<n>, "
-                         "simt-<wide32|wide|huge16>-<off|thread|warp|block|detect>-<n>")
+                         "simt-<wide32|wide|huge16>-<off|thread|warp|block|detect>-<n> (the fp32 call on that "
+                         "tile tuple: the tensor cores at off, warp and block from about n = 512 on)")
     return ap.parse_args()
 
 
@@ -77,7 +78,7 @@ def run_case(case):
     kind, dtn, lvn, n = case.split("-")
     assert kind in ("tc", "tc1", "tc2", "tcgroup", "f64", "simt"), case
     n = int(n)
-    if kind == "simt":  # simt-<tuple>-<level>-<n>: the fp32 kernel on U(-1,1) operands
+    if kind == "simt":  # simt-<tuple>-<level>-<n>: the fp32 call on that tuple, U(-1,1) operands
         tuples = {"wide32": SCHED, "wide": SCHED16, "huge16": SCHED_OFF_BEST}
         h = ft.Handle(0)
         h.set_schedule(tuples[dtn])

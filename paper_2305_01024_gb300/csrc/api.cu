@@ -564,8 +564,10 @@ static int fetch_report(ftgemm_ctx* h, ftgemm_report* out, const int* flag, int*
 // CTA pairs for this operand type.  Automatic: bf16 on pairs (each SM moves a
 // third fewer operand bytes per k-block: 7-11% faster kernels measured at
 // 8192^3 and 16384^3, with or without checksums), e4m3 on single CTAs (its
-// operands are half the bytes per flop; pairs measured level without
-// checksums and 4% slower with them).
+// operands are half the bytes per flop).  The e4m3 line dates from the epilogue
+// before pairs stored runs of 128 bytes, when they measured level without
+// checksums and 4% slower with them; now pairs are ahead at 16384^3, 3613 against
+// 3383 TFLOP/s and 3171 against 3072, smaller sizes not measured.
 // A shape tuned by ftgemm_autotune_tc takes the schedule measured fastest.
 static bool tc_use_pair(const ftgemm_ctx* h, int dt, int64_t m = 0, int64_t n = 0, int64_t k = 0, int level = 0) {
   if (h->tc_pair >= 0) return h->tc_pair != 0;

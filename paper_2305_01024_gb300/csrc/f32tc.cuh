@@ -9,12 +9,14 @@
 // a3 b2, a3 b3: together below 2^-25 |a b|) are left out, half an ulp of one
 // fp32 product rounding.  The other six run as bf16 MMAs.
 //
-// The tensor-core accumulation truncates, so it only ever runs over F32TC_KC
-// elements of K: each chunk's products are summed in tensor memory in order
-// of size, smallest first, and the chunk's result is added to an fp32
-// accumulator in registers with round-to-nearest.  The registers are the
-// accumulators the ABFT scheme protects: faults are added there, and every
-// verification period the unit's row and column sums are formed from them.
+// The tensor-core accumulation truncates (a chunk's sum of one sign comes out
+// 0.7 to 1 u too small, u = 2^-24), so it only ever runs over F32TC_KC elements
+// of K, and a product of fewer stays on the CUDA cores.  Each chunk's products
+// are summed in tensor memory in order of size, smallest first, and the chunk's
+// result is added to an fp32 accumulator in registers with round-to-nearest.
+// The registers are the accumulators the ABFT scheme protects: faults are added
+// there, and every verification period the unit's row and column sums are formed
+// from them.
 #pragma once
 #include "f32tc_seg.cuh"
 #include "internal.cuh"

@@ -16,9 +16,10 @@
 //
 // The checksums (Eq. 4) come from the same kernel (SUMS = true) run first on
 // the encoded operands: (e^T A) B and A (B e), one result per segment of at
-// most 256 of K (of a whole period, where that costs less: f32tc_plan), all in parallel; two warps of the main kernel add a
-// period's segments to the running checksums ahead of its verification.  They cost
-// the units' share of a tile (1/128 of the product each for 128 x 128 units)
+// most 256 of K (or a whole period, where that costs less: f32tc_plan), all in
+// parallel; two warps of the main kernel add a period's segments to the running
+// checksums ahead of its verification.  They cost the units' share of a tile
+// (1/128 of the product each for 128 x 128 units)
 // instead of an extra operand row in every MMA, so the verification unit
 // stays the schedule's own tile.
 #include <climits>
